@@ -280,8 +280,10 @@ GS_API gs_status gs_similarity_coeffs(const gs_basis* h, const float* Y, long lo
  * with attribute probabilities as weights; Sec. 3.1 / 3.3: run on Gram-loc).
  * V = P R: P is N x M (fp32, ld = ldp), V is N x r of type v_dtype
  * (GS_F32 or GS_BF16, ld = ldv).  V is the Gram-loc of P C.
- * fp32 V: fp32 CUDA-core arithmetic.  bf16 V: bf16 tensor-core product with
- * fp32 accumulation when GS_PATH_AUTO/TENSOR and the shape allows it.
+ * Large calls with P 16-byte aligned and ldp % 4 == 0 (GS_PATH_AUTO / TENSOR): P and R
+ * split into bf16 hi / lo on the tensor cores (~2^-16 relative).  Otherwise at fp32
+ * accuracy (GS_PATH_AUTO: on the tensor cores with operands in three bf16 parts
+ * when the call is large; GS_PATH_SIMT: always fp32 CUDA cores).
  */
 GS_API gs_status gs_prob_vectorize(const gs_basis* h, const float* P, long long N, int ldp, void* V,
                             int v_dtype, int ldv, unsigned flags, void* stream);
@@ -298,7 +300,8 @@ GS_API gs_status gs_prob_vectorize(const gs_basis* h, const float* P, long long 
  * brings its largest magnitude to [2^14, 2^15), rounded once to fp16 into the
  * handle's scratch, multiplied by the dithered fp16 Q with fp32 accumulation,
  * and the row's scale is undone in fp32, so the result is accurate for rows of
- * any magnitude (down to a largest entry of 2^-112).  Otherwise fp32 CUDA cores.
+ * any magnitude (down to a largest entry of 2^-112).  Otherwise at fp32 accuracy, as
+ * gs_prob_vectorize.
  */
 GS_API gs_status gs_reconstruct(const gs_basis* h, const void* T, int t_dtype, long long N, int ldt,
                          float* Xhat, int ldxh, unsigned flags, void* stream);

@@ -365,7 +365,7 @@ gs_status gs_project_similarity(const gs_basis* h, const float* X, long long N, 
             a.ksplit = (int)std::min<long long>(gemm_ksplit(nc, r, D, h->device), room);
             a.kpart = a.ksplit > 1 ? scr : nullptr;
         }
-        cudaError_t e = gs::launch_gemm_simt(a, s);
+        cudaError_t e = gs::launch_gemm_fp32(a, flags == GS_PATH_SIMT, h->device, s);
         if (e != cudaSuccess) return from_cuda(e);
         if (!S && !argmax && !maxval) continue;
         float* Sbuf = S ? S + c0 * lds : scr;
@@ -376,7 +376,7 @@ gs_status gs_project_similarity(const gs_basis* h, const float* X, long long N, 
         b.C = Sbuf; b.c_type = gs::MAT_F32; b.ldc = ldsb;
         b.m = nc; b.n = M; b.k = r; b.batch = 1; b.alpha = scale;
         if (mode == GS_SCORE_COSINE) { b.rownorm = xn; b.colnorm = h->cnorm; }
-        e = gs::launch_gemm_simt(b, s);
+        e = gs::launch_gemm_fp32(b, flags == GS_PATH_SIMT, h->device, s);
         if (e != cudaSuccess) return from_cuda(e);
         if (argmax || maxval || mode == GS_SCORE_SOFTMAX) {
             e = gs::launch_row_finish(Sbuf, nc, M, (int)ldsb, mode == GS_SCORE_SOFTMAX,
@@ -513,7 +513,7 @@ gs_status gs_similarity_coeffs(const gs_basis* h, const float* Y, long long N, i
             b.C = Sbuf; b.c_type = gs::MAT_F32; b.ldc = ldsb;
             b.m = nc; b.n = M; b.k = r; b.batch = 1; b.alpha = scale;
             if (xn) { b.rownorm = xn; b.colnorm = h->cnorm; }
-            e = gs::launch_gemm_simt(b, s);
+            e = gs::launch_gemm_fp32(b, flags == GS_PATH_SIMT, h->device, s);
         }
         if (e != cudaSuccess) return from_cuda(e);
         if (argmax || maxval || mode == GS_SCORE_SOFTMAX) {
@@ -554,7 +554,7 @@ gs_status gs_prob_vectorize(const gs_basis* h, const float* P, long long N, int 
         a.C = (char*)V + (size_t)c0 * ldv * (v_dtype == GS_F32 ? 4 : 2);
         a.c_type = v_dtype == GS_F32 ? gs::MAT_F32 : gs::MAT_BF16; a.ldc = ldv;
         a.m = nc; a.n = h->r; a.k = h->M; a.batch = 1; a.alpha = 1.f;
-        cudaError_t e = gs::launch_gemm_simt(a, s);
+        cudaError_t e = gs::launch_gemm_fp32(a, flags == GS_PATH_SIMT, h->device, s);
         if (e != cudaSuccess) return from_cuda(e);
     }
     return GS_OK;
@@ -611,7 +611,7 @@ static gs_status reconstruct_rows(const gs_basis* h, const void* T, int t_dtype,
         a.B = Qb; a.b_type = gs::MAT_F32; a.ldb = ldqb; a.b_trans = false;
         a.C = Xhat + c0 * ldxh; a.c_type = gs::MAT_F32; a.ldc = ldxh;
         a.m = nc; a.n = h->D; a.k = h->r; a.batch = 1; a.alpha = 1.f;
-        cudaError_t e = gs::launch_gemm_simt(a, s);
+        cudaError_t e = gs::launch_gemm_fp32(a, flags == GS_PATH_SIMT, h->device, s);
         if (e != cudaSuccess) return from_cuda(e);
     }
     return GS_OK;
@@ -792,7 +792,7 @@ gs_status gs_attention_scores(const void* Yq, const void* Yk, int in_dtype, int 
     a.B = Yk; a.b_type = t; a.ldb = ldy; a.b_bstride = (long long)Lk * ldy; a.b_trans = true;
     a.C = A; a.c_type = gs::MAT_F32; a.ldc = Lk; a.c_bstride = (long long)Lq * Lk;
     a.m = Lq; a.n = Lk; a.k = r; a.batch = B; a.alpha = scale;
-    cudaError_t e = gs::launch_gemm_simt(a, s);
+    cudaError_t e = gs::launch_gemm_fp32(a, flags == GS_PATH_SIMT, dev, s);
     if (e != cudaSuccess) return from_cuda(e);
     if (apply_softmax) {
         e = gs::launch_row_softmax(A, (long long)B * Lq, Lk, Lk, s);
@@ -812,7 +812,7 @@ gs_status gs_stream_status(void* stream) {
     cudaError_t e = stream ? cudaStreamSynchronize((cudaStream_t)stream) : cudaDeviceSynchronize();
     if (e != cudaSuccess) return GS_ERR_CUDA;
     const unsigned w = gs::take_device_error_build() | gs::take_device_error_tc() | gs::take_device_error_gemm() |
-                       gs::take_device_error_attn() | gs::take_device_error_rbind();
+                       gs::take_device_error_attn() | gs::take_device_error_rbind() | gs::take_device_error_x3();
     if (w & GS_DEV_ERR_TIMEOUT) return GS_ERR_TIMEOUT;
     if (w & GS_DEV_ERR_RANGE) return GS_ERR_RANGE;
     if (w & GS_DEV_ERR_LAYOUT) return GS_ERR_UNSUPPORTED;

@@ -134,6 +134,9 @@ struct GemmArgs {
     float* kpart;
 };
 cudaError_t launch_gemm_simt(const GemmArgs& g, cudaStream_t s);
+// the same product at fp32 accuracy: on the tensor cores when it is large (gs_gemm_x3.cu: operands
+// split into three bf16 parts), else (and always with simt) launch_gemm_simt
+cudaError_t launch_gemm_fp32(const GemmArgs& g, bool simt, int device, cudaStream_t s);
 
 // per-row ||x||
 cudaError_t launch_rownorm(const float* X, long long N, int ldx, int D, float* out, cudaStream_t s);
@@ -227,6 +230,7 @@ unsigned take_device_error_tc();
 // one block whose wait on a never-completed mbarrier runs out (failure-detection self-test)
 cudaError_t launch_wait_selftest(cudaStream_t s);
 unsigned take_device_error_gemm();
+unsigned take_device_error_x3();
 unsigned take_device_error_attn();
 unsigned take_device_error_rbind();
 

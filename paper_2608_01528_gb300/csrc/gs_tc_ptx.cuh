@@ -93,6 +93,30 @@ static __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t pa
     const bool ok = mbar_wait(bar, parity, abort_flag, err_word);
     return __all_sync(0xffffffffu, ok);
 }
+// mbar_wait_warp without the call, for a warp that keeps many values in registers across the wait
+// (a call would have the caller spill all that the callee may use).
+static __device__ __forceinline__ bool mbar_wait_warp_inline(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
+                                                      unsigned* err_word) {
+    bool ok = true;
+    if (!mbar_try_wait(bar, parity)) {
+        const unsigned long long t0 = globaltimer();
+        for (uint32_t i = 1; !mbar_try_wait(bar, parity); ++i) {
+            if ((i & 255u) == 0) {
+                if (*abort_flag) {
+                    ok = false;
+                    break;
+                }
+                if (globaltimer() - t0 > kWaitLimitNs) {
+                    *abort_flag = 1;
+                    atomicOr(err_word, GS_DEV_ERR_TIMEOUT);
+                    ok = false;
+                    break;
+                }
+            }
+        }
+    }
+    return __all_sync(0xffffffffu, ok);
+}
 // Wait used while unwinding: bounded, ignores the abort flag.
 static __device__ __noinline__ void mbar_drain(uint64_t* bar, uint32_t parity, unsigned* err_word) {
     const unsigned long long t0 = globaltimer();

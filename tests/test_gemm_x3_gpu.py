@@ -1,0 +1,107 @@
+"""The fp32-accurate GEMM on the tensor cores (operands in three bf16 parts), through the calls that
+take it: large reconstructions and vectorizations whose rows are not 16-byte aligned, bf16 T, short
+rows, fp32 attention.  Element-wise against the 64-bit product:
+
+    |error| <= (20 + ceil(K / 256)) 2^-23 sum_k |a_k| |b_k|
+
+a bound from the kernel's arithmetic: at most 16 accumulation steps per 256 terms, each losing at
+most 2^-23 of the sum of magnitudes; the small products' steps, 2^-8 of that and 6 times as many; the
+products left out, below 2^-23; one fp32 addition per 256 terms.
+"""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+def bound(K, mag):
+    return (20 + -(-K // 256)) * 2.0 ** -23 * mag + 1e-30
+
+
+def bipolar(rng, M, D):
+    return torch.from_numpy((rng.integers(0, 2, size=(M, D)) * 2 - 1).astype(np.float32)).cuda()
+
+
+# (N, r, D): ragged row and column tiles, K a whole number of K-blocks, one past, one short, one and
+# several accumulation chunks, rows starting on 4-, 8- and 16-byte boundaries
+SHAPES = [(2049, 161, 8200), (1500, 255, 5001), (777, 130, 9001), (2048, 511, 1999), (1300, 513, 2050),
+          (1025, 922, 3000), (1100, 1031, 1500), (2000, 320, 900)]
+
+
+@pytest.mark.parametrize("N,r,D", SHAPES)
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_reconstruct_against_64_bits(gs, N, r, D, dtype):
+    rng = np.random.default_rng([N, r, D])
+    b = gs.build_basis(bipolar(rng, r, D))
+    T = torch.from_numpy(rng.standard_normal((N, b.r)).astype(np.float32)).cuda()
+    T[N // 2] *= 1e20  # rows of other magnitudes
+    T[N // 3] *= 1e-20
+    T = T.to(dtype)
+    X = gs.reconstruct(b, T)
+    gs.stream_status()
+    ref = T.double() @ b.Q.double()
+    if dtype == torch.float32 and b.r % 4 == 0 and D >= 1024:
+        tol = 1e-4 * T.double().norm(dim=1, keepdim=True)  # the fp16 path's documented bound
+    else:
+        tol = bound(b.r, T.double().abs() @ b.Q.double().abs())
+    assert bool(((X.double() - ref).abs() <= tol).all())
+
+
+@pytest.mark.parametrize("N,M", [(4001, 333), (9000, 517), (2500, 1030)])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_vectorize_unaligned(gs, N, M, dtype):
+    rng = np.random.default_rng([N, M])
+    b = gs.build_basis(bipolar(rng, M, 1536))
+    P = torch.softmax(torch.from_numpy(2 * rng.standard_normal((N, M)).astype(np.float32)).cuda(), 1)
+    base = torch.zeros(N * M + 1, device="cuda")
+    Pu = base[1:].view(N, M).copy_(P)  # rows off every vector boundary
+    V = gs.prob_vectorize(b, Pu, dtype=dtype)
+    gs.stream_status()
+    ref = P.double() @ b.R.double()
+    tol = bound(M, P.double() @ b.R.double().abs())
+    if dtype == torch.bfloat16:
+        tol = tol + 2.0 ** -8 * ref.abs()
+    assert bool(((V.double() - ref).abs() <= tol).all())
+
+
+def test_attention_fp32_batched(gs):
+    g = torch.Generator(device="cuda").manual_seed(3)
+    q = torch.randn((5, 391, 130), generator=g, device="cuda")
+    k = torch.randn((5, 1517, 130), generator=g, device="cuda")
+    A = gs.attention_scores(q, k, 0.5, apply_softmax=False)
+    gs.stream_status()
+    ref = 0.5 * (q.double() @ k.double().transpose(1, 2))
+    tol = 0.5 * bound(130, q.double().abs() @ k.double().abs().transpose(1, 2))
+    assert bool(((A.double() - ref).abs() <= tol).all())
+
+
+def test_scores_of_odd_dimension(gs):
+    """D % 4 != 0: the projection and the scores both take the general path."""
+    rng = np.random.default_rng(8)
+    C = bipolar(rng, 300, 2501)
+    b = gs.build_basis(C)
+    X = C[torch.arange(7000, device="cuda") % 300] + torch.randn((7000, 2501), device="cuda")
+    out = gs.project_similarity(b, X, mode="cosine", want_S=True)
+    gs.stream_status()
+    ref = (X.double() @ C.double().T) / (X.double().norm(dim=1)[:, None] * C.double().norm(dim=1)[None, :])
+    assert float((out["S"].double() - ref).abs().max()) <= 2e-5
+    assert torch.equal(out["argmax"].long(), ref.argmax(1))
+
+
+@pytest.mark.parametrize("bad", [float("inf"), -float("inf"), float("nan"), 3.4e38])
+def test_not_finite_as_on_the_cuda_cores(gs, bad):
+    """Rows with an infinity, a NaN or a value beyond bf16's range: the same infinities and NaN in the
+    same places as the CUDA-core path, every other output within the bound."""
+    rng = np.random.default_rng(5)
+    b = gs.build_basis(bipolar(rng, 131, 9003))
+    T = torch.from_numpy(rng.standard_normal((1100, b.r)).astype(np.float32)).cuda()
+    T[7, 3] = bad
+    T[1099, 130] = bad
+    X, S = gs.reconstruct(b, T), gs.reconstruct(b, T, path="simt")
+    gs.stream_status()
+    for f in (torch.isnan, torch.isposinf, torch.isneginf):
+        assert torch.equal(f(X), f(S))
+    rows = [i for i in range(1100) if i not in (7, 1099)]
+    ref = T.double() @ b.Q.double()
+    assert bool(((X.double() - ref).abs() <= bound(b.r, T.double().abs() @ b.Q.double().abs()))[rows].all())
