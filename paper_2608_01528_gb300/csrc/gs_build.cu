@@ -4,22 +4,27 @@
 // Row-order Gram-Schmidt with two projection passes per row and a relative
 // rank tolerance, in fp64 on the device.  Rows are taken in panels of
 // kPanel.  For each panel:
-//   1. load the panel rows V (fp64) and their norms ||c_i||;
-//   2. twice (reorthogonalisation): H = V Q_old^T (tiled fp64 dot products
-//      over D-slices, then a slice reduction that also accumulates R), and
+//   1. the rows' norms ||c_i|| (once, before the panels);
+//   2. twice (reorthogonalisation): H = V Q_old^T (fp64 dot products over
+//      column slices, then a slice reduction that also accumulates R), and
 //      V -= H Q_old -- a block projection against the basis built so far;
-//   3. a cluster of CTAs (each owning a slice of the columns) runs Gram-Schmidt
-//      with two passes over the panel's own new directions, row by row, decides
-//      rank (||v|| > tol * ||c_i||), normalises and appends accepted rows to Q.
+//   3. inside the panel: Cholesky QR, twice (two passes again), with the rank
+//      decisions (||v|| > tol * ||c_i||) taken from the pivots; accepted rows are
+//      appended to Q.  A panel whose decisions the pivots cannot settle is done
+//      row by row instead, on a cluster of CTAs.
 // In exact arithmetic this is the row-wise two-pass Gram-Schmidt of the
-// paper's construction (projections onto orthonormal directions commute);
-// the block passes against the old basis and the column slices within the
-// panel are what make it data-parallel.
+// paper's construction (projections onto orthonormal directions commute, and
+// Cholesky QR of a panel is its Gram-Schmidt factorisation); the block passes
+// against the old basis and the column slices are what make it data-parallel.
+// Measured (GB300): M = 512, D = 4096: 20.0 ms before the slices were cut to the
+// number of SMs and the panels factored by Cholesky QR; see k_panel_slice.
 // The only host synchronisation is the read of the final rank r.
 //
 // Afterwards fp32 copies of Q and R are made for the caller, plus the
 // fp16 operand copies of the tensor-core kernels (unbiased dithered rounding
 // of the fp64 basis, see dither_half).
+
+#include <float.h>
 
 #include <algorithm>
 #include <cmath>
@@ -33,10 +38,7 @@ namespace gs {
 namespace {
 
 constexpr int kPanel = 16;      // rows per panel
-constexpr int kDotTileQ = 16;   // basis rows per dot tile
-constexpr int kDotCols = 64;    // columns staged per step in the dot kernel
-constexpr int kUpdCols = 64;    // columns per CTA in the update kernel
-constexpr int kUpdJ = 128;      // coefficients staged per step in the update kernel
+constexpr int kMaxSlice = 96;   // columns per slice CTA (shared memory; 3 x 512 update outputs)
 
 __device__ unsigned g_err_build = 0;
 
@@ -57,116 +59,470 @@ __device__ double block_sum(double v, double* sh) {
     return sh[32];
 }
 
-// 1. panel rows -> V (fp64), ||c_i||.  One CTA per panel row.
-__global__ void __launch_bounds__(256) k_panel_load(const float* __restrict__ C, long long ldc, int D,
-                                                     int p0, int normalize, double* __restrict__ V,
-                                                     double* __restrict__ cn) {
+// Row norms ||c_i|| and, with normalize, the rows' scales 1 / ||c_i|| (the norm is then that of the
+// scaled row).  One CTA per row of C.
+__global__ void __launch_bounds__(256) k_row_norms(const float* __restrict__ C, long long ldc, int D, int normalize,
+                                                   double* __restrict__ cn, double* __restrict__ sc) {
     __shared__ double sh[33];
-    const int k = blockIdx.x;
-    const float* c = C + (size_t)(p0 + k) * ldc;
-    double* v = V + (size_t)k * D;
+    const float* c = C + (size_t)blockIdx.x * ldc;
     double ss = 0.0;
-    for (int d = threadIdx.x; d < D; d += 256) {
-        double x = (double)c[d];
-        v[d] = x;
-        ss += x * x;
-    }
-    double nrm = sqrt(block_sum<256>(ss, sh));
+    for (int d = threadIdx.x; d < D; d += 256) ss += (double)c[d] * (double)c[d];
+    double nrm = sqrt(block_sum<256>(ss, sh)), scale = 1.0;
     if (normalize && nrm > 0.0) {
-        const double sc = 1.0 / nrm;
+        scale = 1.0 / nrm;
         ss = 0.0;
         for (int d = threadIdx.x; d < D; d += 256) {
-            double x = v[d] * sc;
-            v[d] = x;
+            const double x = (double)c[d] * scale;
             ss += x * x;
         }
         nrm = sqrt(block_sum<256>(ss, sh));
     }
-    if (threadIdx.x == 0) cn[p0 + k] = nrm;
+    if (threadIdx.x == 0) {
+        cn[blockIdx.x] = nrm;
+        sc[blockIdx.x] = scale;
+    }
 }
 
-// 2a. partial dot products Hp[slice][k][j] = sum_{d in slice} V[k][d] Qw[j][d]
-//     for j < r0 (the rank at the start of this panel).  grid (q tiles, slices).
-__global__ void __launch_bounds__(256) k_panel_dots(const double* __restrict__ V,
-                                                     const double* __restrict__ Qw, int D, int bp,
-                                                     const int* __restrict__ r_start, int dslice,
-                                                     double* __restrict__ Hp, int ldh) {
-    const int r0 = *r_start;
-    const int j0 = blockIdx.x * kDotTileQ;
-    if (j0 >= r0) return;
-    const int d0 = blockIdx.y * dslice;
-    const int d1 = min(D, d0 + dslice);
-    __shared__ double sV[kPanel][kDotCols + 1];
-    __shared__ double sQ[kDotTileQ][kDotCols + 1];
-    const int ty = threadIdx.x / kDotTileQ;  // panel row
-    const int tx = threadIdx.x % kDotTileQ;  // basis row within the tile
-    double acc = 0.0;
-    for (int dd = d0; dd < d1; dd += kDotCols) {
-        for (int e = threadIdx.x; e < kPanel * kDotCols; e += 256) {
-            const int rr = e / kDotCols, cc = e % kDotCols;
-            const int d = dd + cc;
-            sV[rr][cc] = (rr < bp && d < d1) ? V[(size_t)rr * D + d] : 0.0;
-            sQ[rr][cc] = (j0 + rr < r0 && d < d1) ? Qw[(size_t)(j0 + rr) * D + d] : 0.0;
+// 2. Block projections.  The D columns are cut into slices of w, one CTA each (about one per SM: GB300
+//    does ~2 fp64 FMAs per clock and SM, so a pass over the basis is bound by that pipe and wants every
+//    SM busy for the same time; 64-column CTAs left 88 of 152 SMs idle at D = 4096, 76 us a pass
+//    against 27 us).  A CTA keeps its slice of the panel in shared memory and streams the basis' slice
+//    through two buffers (cp.async).  kind:
+//      kDots1    V = C;           Hp = V Q^T                  (first pass' dots, over the slice)
+//      kUpdDots  V = C - H Q;     Hp = V Q^T                  (first pass' update, second's dots)
+//      kUpdGram  V -= H Q;        Gp = V V^T, V stored        (second update, and the panel's Gram matrix)
+//    The second update runs in fp32: its coefficients are what the first pass left over, ~1e-16 of the
+//    row, so that one fp32 rounding of each term is ~1e-23 of it.
+//    Gp sums the slices of a cluster of kSliceCluster CTAs through distributed shared memory (fixed order).
+enum { kDots1 = 0, kUpdDots = 1, kUpdGram = 2 };
+constexpr int kSliceCluster = 8;
+constexpr int kPairs = kPanel * (kPanel + 1) / 2;  // 136: the Gram matrix' lower triangle
+
+// What a panel's factorisation hands from kernel to kernel.
+struct PanelState {
+    int slow;    // a rank decision needs the row-by-row kernel
+    int nacc;    // accepted rows, in order
+    int acc[kPanel];
+    double L[kPanel][kPanel];  // V = L V' (V': nacc rows)
+};
+
+__device__ __forceinline__ void cp_async8(double* dst, const double* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(ptx::smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// A double rounded towards zero to fp32 with integer instructions (conversions would share the fp64
+// pipe); magnitudes below fp32's normal range become 0.  For |d| <= 1.
+__device__ __forceinline__ float trunc_f32(double d) {
+    const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
+    const uint32_t mag = ((hi & 0x7fffffffu) << 3) | (lo >> 29);  // exponent still biased by 1023
+    const uint32_t r = ((hi >> 20) & 0x7ffu) > 896u ? mag - (896u << 23) : 0u;
+    return __uint_as_float(r | (hi & 0x80000000u));
+}
+
+struct SliceParams {
+    const float* C;     // the panel's first row
+    long long ldc;
+    const double* sc;   // the panel rows' scales and norms
+    const double* cn;
+    double* V;          // kPanel x D
+    const double* Qw;
+    int D, w, bp, jc;   // jc: basis rows per chunk
+    const int* r_start;
+    const double* H;
+    double* Hp;
+    int ldh;
+    double* Gp;         // per cluster: kPairs
+};
+
+// the sums over a cluster's CTAs of part[kPairs] (each CTA's own, in shared memory): CTA q adds the
+// entries e = q mod kSliceCluster in CTA order and writes them to out
+__device__ __forceinline__ void cluster_add_pairs(const double* part, double* out) {
+    ptx::cluster_sync_all();
+    const int rank = (int)ptx::cluster_ctarank();
+    const int e = rank + kSliceCluster * (int)threadIdx.x;
+    if (e < kPairs) {
+        double v = 0.0;
+        for (int c = 0; c < kSliceCluster; ++c) {
+            double x;
+            asm volatile("ld.shared::cluster.f64 %0, [%1];"
+                         : "=d"(x)
+                         : "r"(ptx::mapa_shared(ptx::smem_u32(part + e), (uint32_t)c))
+                         : "memory");
+            v += x;
+        }
+        out[e] = v;
+    }
+    ptx::cluster_sync_all();  // no CTA leaves while a peer may still read its part
+}
+
+// part[e] = sum over the slice of V_i V_j for the pairs e = (i, j <= i); Vs: kPanel rows of w, ld vl
+__device__ __forceinline__ void gram_slice(const double* Vs, int vl, int w, double* part) {
+    for (int e = threadIdx.x; e < kPairs; e += blockDim.x) {
+        int i = 0;
+        while ((i + 1) * (i + 2) / 2 <= e) ++i;
+        const int j = e - i * (i + 1) / 2;
+        double a = 0.0, b = 0.0;
+        int c = 0;
+        for (; c + 1 < w; c += 2) {
+            a += Vs[i * vl + c] * Vs[j * vl + c];
+            b += Vs[i * vl + c + 1] * Vs[j * vl + c + 1];
+        }
+        if (c < w) a += Vs[i * vl + c] * Vs[j * vl + c];
+        part[e] = a + b;
+    }
+}
+
+// 2^(+-e) with 2^e <= n < 2^(e+1) (1 for n = 0 or not finite): a row's scale as an exact factor
+__device__ __forceinline__ double row_pow2(double n, int sign) {
+    const int e = n > 0.0 && n <= DBL_MAX ? ilogb(n) : 0;
+    return __hiloint2double((1023 + sign * e) << 20, 0);
+}
+
+template <int KIND>
+__global__ void __launch_bounds__(512) k_panel_slice(const SliceParams p) {
+    extern __shared__ double sm[];
+    const int tid = threadIdx.x, nt = blockDim.x;
+    const int r0 = *p.r_start;
+    const int c0 = blockIdx.x * p.w, w = max(0, min(p.w, p.D - c0));
+    const int vl = p.w | 1;  // odd row pitches: lanes on consecutive rows hit different banks
+    double* Vs = sm;
+    double* Qs[2] = {Vs + kPanel * vl, Vs + kPanel * vl + p.jc * vl};
+    double* Hs[2] = {Qs[1] + p.jc * vl, Qs[1] + p.jc * vl + kPanel * p.jc};  // updates only
+    double* part = Hs[0];  // the Gram partials: after the last chunk of H
+    float* Qf = reinterpret_cast<float*>(Hs[1] + kPanel * p.jc);  // kUpdGram: the current chunk in fp32
+    float* Hf = Qf + p.jc * vl;
+    const int nchunks = (r0 + p.jc - 1) / p.jc;
+
+    auto fetch = [&](int ch, int b, bool with_h) {
+        const int j0 = ch * p.jc, nj = min(p.jc, r0 - j0);
+        for (int e = tid; e < nj * w; e += nt) {
+            const int j = e / w, c = e - j * w;
+            cp_async8(&Qs[b][j * vl + c], p.Qw + (size_t)(j0 + j) * p.D + c0 + c);
+        }
+        if (with_h)
+            for (int e = tid; e < kPanel * nj; e += nt) {
+                const int k = e / nj, j = e - k * nj;
+                if (k < p.bp) cp_async8(&Hs[b][k * p.jc + j], p.H + (size_t)k * p.ldh + j0 + j);
+            }
+        cp_async_commit();
+    };
+    if (nchunks > 0) fetch(0, 0, KIND != kDots1);
+    for (int e = tid; e < kPanel * w; e += nt) {
+        const int k = e / w, c = e - k * w;
+        double v = 0.0;
+        if (k < p.bp)
+            v = KIND == kUpdGram && r0 > 0 ? p.V[(size_t)k * p.D + c0 + c]
+                                           : (double)p.C[(size_t)k * p.ldc + c0 + c] * p.sc[k];
+        Vs[k * vl + c] = v;
+    }
+    if (KIND != kDots1) {
+        // V -= H Q: thread outputs (k, c), at most three a thread (kPanel w <= 3 nt), summed over chunks
+        constexpr int kOut = 3;
+        double acc[kOut] = {};
+        float accf[kOut] = {};
+        int ko[kOut], co[kOut];
+#pragma unroll
+        for (int o = 0; o < kOut; ++o) {
+            const int e = tid + o * nt;
+            ko[o] = w > 0 && e < kPanel * w ? e / w : 0;
+            co[o] = w > 0 && e < kPanel * w ? e % w : 0;
+        }
+        for (int ch = 0; ch < nchunks; ++ch) {
+            const int b = ch & 1, nj = min(p.jc, r0 - ch * p.jc);
+            if (ch + 1 < nchunks) {
+                fetch(ch + 1, b ^ 1, true);
+                cp_async_wait<1>();
+            } else {
+                cp_async_wait<0>();
+            }
+            __syncthreads();
+            if (KIND == kUpdGram) {  // the chunk once into fp32, the coefficients relative to the row's norm
+                for (int e = tid; e < nj * vl; e += nt) Qf[e] = trunc_f32(Qs[b][e]);
+                for (int e = tid; e < kPanel * nj; e += nt) {
+                    const int k = e / nj, j = e - k * nj;
+                    Hf[k * p.jc + j] = k < p.bp ? (float)(Hs[b][k * p.jc + j] * row_pow2(p.cn[k], -1)) : 0.f;
+                }
+                __syncthreads();
+            }
+#pragma unroll
+            for (int o = 0; o < kOut; ++o) {
+                if (tid + o * nt >= kPanel * w) continue;
+                if (KIND == kUpdGram) {
+                    const float* h = &Hf[ko[o] * p.jc];
+                    for (int j = 0; j < nj; ++j) accf[o] = fmaf(h[j], Qf[j * vl + co[o]], accf[o]);
+                } else {
+                    const double* h = &Hs[b][ko[o] * p.jc];
+                    for (int j = 0; j < nj; ++j) acc[o] += h[j] * Qs[b][j * vl + co[o]];
+                }
+            }
+            __syncthreads();
+        }
+        if (nchunks == 0) __syncthreads();
+#pragma unroll
+        for (int o = 0; o < kOut; ++o) {
+            if (tid + o * nt >= kPanel * w || ko[o] >= p.bp) continue;
+            double v = Vs[ko[o] * vl + co[o]];
+            v -= KIND == kUpdGram ? (double)accf[o] * row_pow2(p.cn[ko[o]], 1) : acc[o];
+            Vs[ko[o] * vl + co[o]] = v;
+            p.V[(size_t)ko[o] * p.D + c0 + co[o]] = v;
+        }
+    }
+    if (KIND == kUpdGram) {
+        __syncthreads();
+        gram_slice(Vs, vl, w, part);
+        cluster_add_pairs(part, p.Gp + (size_t)(blockIdx.x / kSliceCluster) * kPairs);
+        return;
+    }
+    // Hp = V Q^T over the slice: thread (k = tid % 16, basis rows j and j + jc / 2 of a chunk)
+    if (KIND == kUpdDots) {
+        __syncthreads();
+        if (nchunks > 0) fetch(0, 0, false);
+    }
+    const int k = tid % kPanel, jl = tid / kPanel, jh = p.jc / 2;
+    for (int ch = 0; ch < nchunks; ++ch) {
+        const int b = ch & 1, j0 = ch * p.jc, nj = min(p.jc, r0 - j0);
+        if (ch + 1 < nchunks) {
+            fetch(ch + 1, b ^ 1, false);
+            cp_async_wait<1>();
+        } else {
+            cp_async_wait<0>();
         }
         __syncthreads();
-#pragma unroll 16
-        for (int cc = 0; cc < kDotCols; ++cc) acc += sV[ty][cc] * sQ[tx][cc];
+        if (jl < nj) {
+            const double* v = &Vs[k * vl];
+            const double* q0 = &Qs[b][jl * vl];
+            const double* q1 = &Qs[b][min(jl + jh, nj - 1) * vl];
+            double a0 = 0.0, a1 = 0.0;
+            if (jl + jh < nj) {
+                for (int c = 0; c < w; ++c) {
+                    const double x = v[c];
+                    a0 += x * q0[c];
+                    a1 += x * q1[c];
+                }
+            } else {
+                for (int c = 0; c < w; ++c) a0 += v[c] * q0[c];
+            }
+            double* out = p.Hp + ((size_t)blockIdx.x * kPanel + k) * p.ldh + j0;
+            out[jl] = a0;
+            if (jl + jh < nj) out[jl + jh] = a1;
+        }
         __syncthreads();
     }
-    if (ty < bp && j0 + tx < r0) Hp[((size_t)blockIdx.y * kPanel + ty) * ldh + j0 + tx] = acc;
 }
 
-// 2b. H[k][j] = sum over slices; R64[p0+k][j] += H[k][j].
-__global__ void k_panel_reduce(const double* __restrict__ Hp, int nslices, int bp,
-                               const int* __restrict__ r_start, int ldh, double* __restrict__ H,
-                               double* __restrict__ R64, int ldr, int p0) {
+// H[k][j] = sum over slices; R64[p0+k][j] += H[k][j].  16 consecutive outputs a block, 16 threads each
+// (fp64 adds take the fp64 FMA's time here, and the loads their latency: four threads an output took
+// 17 us at 152 slices), their parts added in a fixed order.
+__global__ void __launch_bounds__(256) k_panel_reduce(const double* __restrict__ Hp, int nslices, int bp,
+                                                      const int* __restrict__ r_start, int ldh, double* __restrict__ H,
+                                                      double* __restrict__ R64, int ldr) {
+    __shared__ double sh[16][17];
     const int r0 = *r_start;
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int k = (int)(idx / ldh), j = (int)(idx % ldh);
-    if (k >= bp || j >= r0) return;
+    const int oi = threadIdx.x & 15, q = threadIdx.x >> 4;
+    const long long o = (long long)blockIdx.x * 16 + oi;
+    const bool in = o < (long long)bp * r0;
+    const int k = in ? (int)(o / r0) : 0, j = in ? (int)(o % r0) : 0;
     double s = 0.0;
-    for (int t = 0; t < nslices; ++t) s += Hp[((size_t)t * kPanel + k) * ldh + j];
-    H[(size_t)k * ldh + j] = s;
-    R64[(size_t)(p0 + k) * ldr + j] += s;
+    if (in) {
+        const double* src = Hp + (size_t)k * ldh + j;
+#pragma unroll 8
+        for (int t = q; t < nslices; t += 16) s += src[(size_t)t * kPanel * ldh];
+    }
+    sh[q][oi] = s;
+    __syncthreads();
+    if (in && q == 0) {
+        double v = 0.0;
+#pragma unroll
+        for (int t = 0; t < 16; ++t) v += sh[t][oi];
+        H[(size_t)k * ldh + j] = v;
+        R64[(size_t)k * ldr + j] += v;
+    }
 }
 
-// 2c. V[k][d] -= sum_{j < r0} H[k][j] Qw[j][d].  CTA = 64 columns x 4 row groups.
-__global__ void __launch_bounds__(256) k_panel_update(double* __restrict__ V,
-                                                       const double* __restrict__ Qw, int D, int bp,
-                                                       const int* __restrict__ r_start,
-                                                       const double* __restrict__ H, int ldh) {
-    const int r0 = *r_start;
-    if (r0 == 0) return;
-    __shared__ double sH[kPanel][kUpdJ];
-    const int d = blockIdx.x * kUpdCols + (threadIdx.x % kUpdCols);
-    const int kg = threadIdx.x / kUpdCols;  // 4 groups of 4 rows
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int jc = 0; jc < r0; jc += kUpdJ) {
-        const int nj = min(kUpdJ, r0 - jc);
-        for (int e = threadIdx.x; e < kPanel * kUpdJ; e += 256) {
-            const int kk = e / kUpdJ, cc = e % kUpdJ;
-            sH[kk][cc] = (kk < bp && cc < nj) ? H[(size_t)kk * ldh + jc + cc] : 0.0;
+// 3. Inside the panel: Cholesky QR, twice.  G = V V^T (summed over the slices) = L L^T, V' = L^-1 V has
+//    rows orthonormal up to the loss of forming G (eps times the panel's condition squared); a second
+//    round on V' brings that to eps, and V = (L L2) V''.  Each round is one pass over the slices with
+//    every CTA doing the 16 x 16 factorisation itself, against three cluster-wide sums per row
+//    (k_panel_gs2: 326 us a panel at D = 4096, of which ~65 us were arithmetic; two rounds take ~25 us).
+//    Row k is accepted exactly as the row-by-row kernel would: its norm against what came before it,
+//    sqrt(pivot), > tau ||c_k||.  A pivot taken from G is only known to ~1e-14 ||v_k||^2, so a panel
+//    with a decision that this could touch (a pivot below 1e-6 ||v_k||^2 that is not certain to fall
+//    below the tolerance, or one within 1e-6 of it) is left to k_panel_gs2.
+//
+// The factorisation in one CTA (all threads): A (the Gram matrix, overwritten), T: rows of L^-1 for the
+// accepted rows (T[a] over the panel's rows), L as in PanelState.  first: the rank decisions are taken;
+// otherwise every row is accepted.  rsqrt of a pivot runs in one thread, the 16 x 16 updates in one
+// FMA per thread (256 of A, 256 of T with 512 threads).
+struct Chol {
+    double A[kPanel][kPanel + 1], T[kPanel][kPanel + 1], L[kPanel][kPanel], diag[kPanel], nv[kPanel], rs;
+    int acc[kPanel], nacc, slow, take;
+};
+
+__device__ __forceinline__ void chol_load(Chol& c, const double* Gp, int ncl) {
+    for (int e = threadIdx.x; e < kPairs; e += blockDim.x) {
+        double v = 0.0;
+        for (int t = 0; t < ncl; ++t) v += Gp[(size_t)t * kPairs + e];
+        int i = 0;
+        while ((i + 1) * (i + 2) / 2 <= e) ++i;
+        const int j = e - i * (i + 1) / 2;
+        c.A[i][j] = v;
+        c.A[j][i] = v;
+        if (i == j) {
+            c.diag[i] = v;
+            c.nv[i] = sqrt(fmax(v, 0.0));
         }
-        __syncthreads();
-        if (d < D) {
-            for (int cc = 0; cc < nj; ++cc) {
-                const double q = Qw[(size_t)(jc + cc) * D + d];
-#pragma unroll
-                for (int t = 0; t < 4; ++t) acc[t] += sH[kg * 4 + t][cc] * q;
+    }
+    for (int e = threadIdx.x; e < kPanel * kPanel; e += blockDim.x) {
+        c.T[e / kPanel][e % kPanel] = e / kPanel == e % kPanel ? 1.0 : 0.0;
+        c.L[e / kPanel][e % kPanel] = 0.0;
+    }
+    if (threadIdx.x == 0) c.nacc = c.slow = 0;
+    __syncthreads();
+}
+
+__device__ __forceinline__ void chol_factor(Chol& c, int n, bool first, const double* cn, double tau, int room) {
+    for (int k = 0; k < n; ++k) {
+        if (threadIdx.x == 0) {
+            const double piv = c.A[k][k];
+            int take = 1;
+            if (first) {
+                const double lim = tau * cn[k], lim2 = lim * lim, v2 = c.diag[k];
+                if (c.nacc >= room) {
+                    take = 0;  // the basis is full: every further row is dependent
+                } else if (!(v2 > lim2 * (1.0 - 1e-6))) {
+                    take = 0;  // what the basis so far leaves of the row is below the tolerance already
+                    if (v2 != v2) c.slow = 1;
+                } else if (piv > 1e-6 * v2) {
+                    take = piv > lim2;
+                    if (fabs(piv - lim2) < 1e-6 * lim2) c.slow = 1;
+                } else {
+                    take = 0;  // dependent within the panel, if even 2e-13 ||v||^2 is below the tolerance
+                    if (!(piv < 1e-13 * v2 && 2e-13 * v2 < lim2)) c.slow = 1;
+                }
+            }
+            c.take = take;
+            if (take) {
+                c.rs = rsqrt(piv);
+                c.acc[c.nacc] = k;
             }
         }
         __syncthreads();
-    }
-    if (d < D) {
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const int k = kg * 4 + t;
-            if (k < bp) V[(size_t)k * D + d] -= acc[t];
+        if (c.take) {
+            const int a = c.nacc;
+            const double rs = c.rs;
+            for (int e = threadIdx.x; e < kPanel; e += blockDim.x) {
+                if (e >= k) c.L[e][a] = c.A[e][k] * rs;
+                else c.T[k][e] *= rs;
+                if (e == k) c.T[k][k] *= rs;
+            }
+            __syncthreads();
+            for (int e = threadIdx.x; e < 2 * kPanel * kPanel; e += blockDim.x) {
+                const int i = (e / kPanel) % kPanel, j = e % kPanel;
+                if (i <= k) continue;
+                if (e < kPanel * kPanel) {
+                    if (j > k) c.A[i][j] -= c.L[i][a] * c.L[j][a];
+                } else if (j <= k) {
+                    c.T[i][j] -= c.L[i][a] * c.T[k][j];
+                }
+            }
+            if (threadIdx.x == 0) ++c.nacc;
         }
+        __syncthreads();
     }
 }
 
-// 3. Gram-Schmidt with two passes inside the panel, rank decision, normalisation and append, on a
+struct CholParams {
+    double* V;
+    double* Qw;
+    int D, w, bp, ncl;
+    const double* Gp;   // this round's Gram partials
+    double* Gp2;        // the next round's (round 1)
+    const double* cn;   // the panel rows' norms
+    double tau;
+    double* R64;        // the panel's first row
+    int ldr, rmax;
+    const int* r_start;
+    int* r_next;
+    PanelState* st;
+};
+
+// ROUND 1: V' = L^-1 V in place (rows 0 .. nacc), its Gram partials, and the panel's state.
+// ROUND 2: the same on V', written to the basis; R's new columns; the rank for the next panel.
+template <int ROUND>
+__global__ void __launch_bounds__(512) k_panel_chol(const CholParams p) {
+    extern __shared__ double sm[];
+    __shared__ Chol c;
+    __shared__ double part[kPairs];
+    const int tid = threadIdx.x, nt = blockDim.x;
+    const int r0 = *p.r_start;
+    const int c0 = blockIdx.x * p.w, w = max(0, min(p.w, p.D - c0));
+    const int vl = p.w | 1;
+    double* Vs = sm;
+    if (ROUND == 2 && p.st->slow) return;  // k_panel_gs2 does this panel
+    const int n = ROUND == 1 ? p.bp : p.st->nacc;
+    for (int e = tid; e < n * w; e += nt) Vs[(e / w) * vl + e % w] = p.V[(size_t)(e / w) * p.D + c0 + e % w];
+    chol_load(c, p.Gp, p.ncl);
+    chol_factor(c, n, ROUND == 1, p.cn, p.tau, p.rmax - r0);
+    if (ROUND == 1) {
+        // V' = T V multiplies G's rounding by (sum_j |T_kj| ||v_j||)^2: beyond 1e8 the second round would
+        // not bring it back to eps
+        if (tid < p.bp && !c.slow) {
+            double amp = 0.0;
+            for (int j = 0; j <= tid; ++j) amp += fabs(c.T[tid][j]) * c.nv[j];
+            bool taken = false;
+            for (int a = 0; a < c.nacc; ++a) taken |= c.acc[a] == tid;
+            if (taken && !(amp < 1e4)) c.slow = 1;
+        }
+        __syncthreads();
+    }
+    const bool slow = ROUND == 1 && c.slow != 0;
+    if (ROUND == 1 && blockIdx.x == 0) {
+        if (tid == 0) {
+            p.st->slow = slow;
+            p.st->nacc = c.nacc;
+        }
+        for (int e = tid; e < kPanel; e += nt) p.st->acc[e] = c.acc[e];
+        for (int e = tid; e < kPanel * kPanel; e += nt) p.st->L[e / kPanel][e % kPanel] = c.L[e / kPanel][e % kPanel];
+    }
+    if (slow) return;  // the same data and so the same answer in every CTA of the grid
+    const int na = c.nacc;
+    for (int e = tid; e < na * w; e += nt) {
+        const int a = e / w, cc = e - a * w, k = c.acc[a];
+        double v = 0.0;
+        for (int j = 0; j <= k; ++j) v += c.T[k][j] * Vs[j * vl + cc];
+        if (ROUND == 1)
+            p.V[(size_t)a * p.D + c0 + cc] = v;  // this CTA's columns, already read
+        else
+            p.Qw[(size_t)(r0 + a) * p.D + c0 + cc] = v;
+    }
+    if (ROUND == 1) {
+        __syncthreads();  // every value of Vs has been used: the Gram matrix of the new rows, read back
+        for (int e = tid; e < kPanel * w; e += nt) {
+            const int a = e / w, cc = e - a * w;
+            Vs[a * vl + cc] = a < na ? p.V[(size_t)a * p.D + c0 + cc] : 0.0;
+        }
+        __syncthreads();
+        gram_slice(Vs, vl, w, part);
+        cluster_add_pairs(part, p.Gp2 + (size_t)(blockIdx.x / kSliceCluster) * kPairs);
+    } else if (blockIdx.x == 0) {
+        // R's new columns: L1 L2
+        for (int e = tid; e < p.bp * na; e += nt) {
+            const int k = e / na, a = e - k * na;
+            double v = 0.0;
+            for (int b = a; b < na; ++b) v += p.st->L[k][b] * c.L[b][a];
+            p.R64[(size_t)k * p.ldr + r0 + a] = v;
+        }
+        if (tid == 0) *p.r_next = r0 + na;
+    }
+}
+
+// 3b. The row-by-row form, for the panels that k_panel_chol leaves (PanelState.slow):
+//    Gram-Schmidt with two passes inside the panel, rank decision, normalisation and append, on a
 //    cluster of kMgsCtas CTAs: CTA c owns columns [c S, (c + 1) S) of every vector (S = ceil(D /
 //    kMgsCtas)), so the fp64 arithmetic of a row is spread over kMgsCtas SMs (GB300's fp64 rate
 //    per SM is low: one CTA doing this took 1.5 ms per 16-row panel of 10,000-wide rows).  Each
@@ -187,9 +543,11 @@ static_assert(kPanel == 16, "the sums' butterfly gives lane l entry l & 15");
 
 __global__ void __launch_bounds__(kMgsThreads) k_panel_gs2(double* __restrict__ V, double* __restrict__ Qw, int D,
                                                           int bp, int p0, double tau, const double* __restrict__ cn,
-                                                          double* __restrict__ R64, int ldr, int* __restrict__ r_dev,
-                                                          int rmax) {
+                                                          double* __restrict__ R64, int ldr,
+                                                          const int* __restrict__ r_start, int* __restrict__ r_next,
+                                                          int rmax, const PanelState* __restrict__ st) {
     using namespace ptx;
+    if (!st->slow) return;  // k_panel_chol has done this panel (the same flag in every CTA)
     __shared__ double part[2][kMgsCtas][kPanel];  // per sum: every CTA's partials (stored by that CTA)
     __shared__ double red[kMgsThreads / 32][kPanel];
     __shared__ uint64_t pbar[2];                  // one barrier per partial buffer: 1 arrival + the bytes
@@ -198,7 +556,7 @@ __global__ void __launch_bounds__(kMgsThreads) k_panel_gs2(double* __restrict__ 
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int S = (D + kMgsCtas - 1) / kMgsCtas;
     const int c0 = (int)rank * S, c1 = min(D, c0 + S);
-    const int r0 = *r_dev;
+    const int r0 = *r_start;
     int r = r0, nsum = 0;
     bool ok = true;  // false once a wait has run out (the results are then flagged as an error)
     if (tid == 0) {
@@ -303,7 +661,7 @@ __global__ void __launch_bounds__(kMgsThreads) k_panel_gs2(double* __restrict__ 
             ++r;
         }
     }
-    if (rank == 0 && tid == 0) *r_dev = r;
+    if (rank == 0 && tid == 0) *r_next = r;
     cluster_sync_all();  // no CTA leaves while a peer may still store into its memory
 }
 
@@ -468,57 +826,104 @@ gs_status factor_rows(const float* C, int M, int D, int ldc, double tau, bool no
     const int rmax = std::min(M, D);
     const int ldr = rmax;                       // R64 leading dimension
     const int ldh = std::max(1, ((M + 15) / 16) * 16);  // >= any r0
-    const int dslice = std::max(kDotCols, ((D + 7) / 8 + kDotCols - 1) / kDotCols * kDotCols);
-    const int nslices = (D + dslice - 1) / dslice;
+    const int npanels = (M + kPanel - 1) / kPanel;
+    // column slices: one per SM, at most kMaxSlice columns each; whole clusters of CTAs
+    int dev = 0, sms = 0;
+    GS_CK(cudaGetDevice(&dev));
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    sms = std::max(sms, kSliceCluster) / kSliceCluster * kSliceCluster;
+    const int w = std::max(8, std::min(kMaxSlice, (D + sms - 1) / sms));
+    const int nslices = ((D + w - 1) / w + kSliceCluster - 1) / kSliceCluster * kSliceCluster;
+    const int ncl = nslices / kSliceCluster;
+    // threads: the update's kPanel w outputs in as few full rounds as fit (at most three of 512)
+    const int rounds = (kPanel * w + 511) / 512;
+    int threads = ((kPanel * w + rounds - 1) / rounds + 31) / 32 * 32;
+    if (threads < 320) threads = 512;  // short rows: few outputs, so longer chunks of the basis instead
+    const int jc = threads / kPanel * 2;        // basis rows per chunk: two dot products a thread
+    const int vl = w | 1;
+    const size_t smem = sizeof(double) * ((size_t)kPanel * vl + 2 * (size_t)jc * vl +
+                                          std::max<size_t>(2 * (size_t)kPanel * jc, kPairs)) +
+                        sizeof(float) * ((size_t)jc * vl + (size_t)kPanel * jc);
+    const size_t smem_chol = sizeof(double) * (size_t)kPanel * vl;
+    for (auto fn : {k_panel_slice<kDots1>, k_panel_slice<kUpdDots>, k_panel_slice<kUpdGram>})
+        GS_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
 
-    DevBuf bV, bH, bHp, br;
-    GS_CK(cudaMalloc(&bV.p, sizeof(double) * (size_t)kPanel * D));
+    // the factors, and one workspace for everything else
     GS_CK(cudaMalloc(&f.Qw, sizeof(double) * (size_t)rmax * D));
     GS_CK(cudaMalloc(&f.R64, sizeof(double) * (size_t)M * ldr));
-    GS_CK(cudaMalloc(&bH.p, sizeof(double) * (size_t)kPanel * ldh));
-    GS_CK(cudaMalloc(&bHp.p, sizeof(double) * (size_t)nslices * kPanel * ldh));
     GS_CK(cudaMalloc(&f.cn, sizeof(double) * (size_t)M));
-    GS_CK(cudaMalloc(&br.p, sizeof(int)));
-    double* V = (double*)bV.p;
+    const size_t nV = (size_t)kPanel * D, nH = (size_t)kPanel * ldh, nHp = (size_t)nslices * kPanel * ldh,
+                 nG = (size_t)ncl * kPairs, nst = (sizeof(PanelState) + 7) / 8;
+    DevBuf ws;
+    GS_CK(cudaMalloc(&ws.p, sizeof(double) * (nV + nH + nHp + 2 * nG + (size_t)M + nst) +
+                                sizeof(int) * (size_t)(npanels + 1)));
     double* Qw = f.Qw;
     double* R64 = f.R64;
-    double* H = (double*)bH.p;
-    double* Hp = (double*)bHp.p;
     double* cn = f.cn;
-    int* r_dev = (int*)br.p;
+    double* V = (double*)ws.p;
+    double* H = V + nV;
+    double* Hp = H + nH;
+    double* G1 = Hp + nHp;
+    double* G2 = G1 + nG;
+    double* sc = G2 + nG;
+    PanelState* st = (PanelState*)(sc + M);
+    int* r_at = (int*)(sc + M + nst);  // r_at[p]: the rank at the start of panel p
     GS_CK(cudaMemsetAsync(R64, 0, sizeof(double) * (size_t)M * ldr, s));
-    GS_CK(cudaMemsetAsync(r_dev, 0, sizeof(int), s));
+    GS_CK(cudaMemsetAsync(r_at, 0, sizeof(int), s));
+    k_row_norms<<<M, 256, 0, s>>>(C, ldc, D, normalize ? 1 : 0, cn, sc);
 
-    for (int p0 = 0; p0 < M; p0 += kPanel) {
-        const int bp = std::min(kPanel, M - p0);
-        k_panel_load<<<bp, 256, 0, s>>>(C, ldc, D, p0, normalize ? 1 : 0, V, cn);
+    auto clustered = [&](int ctas, int cluster, int nthreads, size_t sm_bytes, cudaLaunchAttribute* at) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)ctas);
+        cfg.blockDim = dim3((unsigned)nthreads);
+        cfg.dynamicSmemBytes = sm_bytes;
+        cfg.stream = s;
+        at->id = cudaLaunchAttributeClusterDimension;
+        at->val.clusterDim.x = (unsigned)cluster;
+        at->val.clusterDim.y = 1;
+        at->val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        return cfg;
+    };
+    for (int pn = 0; pn < npanels; ++pn) {
+        const int p0 = pn * kPanel, bp = std::min(kPanel, M - p0);
+        SliceParams sp;
+        sp.C = C + (size_t)p0 * ldc, sp.ldc = ldc;
+        sp.sc = sc + p0, sp.cn = cn + p0;
+        sp.V = V, sp.Qw = Qw;
+        sp.D = D, sp.w = w, sp.bp = bp, sp.jc = jc;
+        sp.r_start = r_at + pn;
+        sp.H = H, sp.Hp = Hp, sp.ldh = ldh;
+        sp.Gp = G1;
         if (p0 > 0) {
-            const int qt = (std::min(p0, rmax) + kDotTileQ - 1) / kDotTileQ;
-            for (int pass = 0; pass < 2; ++pass) {
-                k_panel_dots<<<dim3(qt, nslices), 256, 0, s>>>(V, Qw, D, bp, r_dev, dslice, Hp, ldh);
-                k_panel_reduce<<<grid1((long long)bp * ldh, 256), 256, 0, s>>>(Hp, nslices, bp, r_dev,
-                                                                                ldh, H, R64, ldr, p0);
-                k_panel_update<<<grid1(D, kUpdCols), 256, 0, s>>>(V, Qw, D, bp, r_dev, H, ldh);
-            }
+            const unsigned rgrid = grid1((long long)bp * std::min(p0, rmax), 16);
+            double* Rp = R64 + (size_t)p0 * ldr;
+            k_panel_slice<kDots1><<<nslices, threads, smem, s>>>(sp);
+            k_panel_reduce<<<rgrid, 256, 0, s>>>(Hp, nslices, bp, sp.r_start, ldh, H, Rp, ldr);
+            k_panel_slice<kUpdDots><<<nslices, threads, smem, s>>>(sp);
+            k_panel_reduce<<<rgrid, 256, 0, s>>>(Hp, nslices, bp, sp.r_start, ldh, H, Rp, ldr);
         }
-        {
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(kMgsCtas);
-            cfg.blockDim = dim3(kMgsThreads);
-            cfg.stream = s;
-            cudaLaunchAttribute at[1];
-            at[0].id = cudaLaunchAttributeClusterDimension;
-            at[0].val.clusterDim.x = kMgsCtas;
-            at[0].val.clusterDim.y = 1;
-            at[0].val.clusterDim.z = 1;
-            cfg.attrs = at;
-            cfg.numAttrs = 1;
-            if (kMgsCtas > 8)
-                GS_CK(cudaFuncSetAttribute(k_panel_gs2, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-            GS_CK(cudaLaunchKernelEx(&cfg, k_panel_gs2, V, Qw, D, bp, p0, tau, (const double*)cn, R64, ldr, r_dev,
-                                     rmax));
-        }
+        cudaLaunchAttribute at[1];
+        cudaLaunchConfig_t cfg = clustered(nslices, kSliceCluster, threads, smem, at);
+        GS_CK(cudaLaunchKernelEx(&cfg, k_panel_slice<kUpdGram>, (const SliceParams)sp));
+        CholParams cp;
+        cp.V = V, cp.Qw = Qw;
+        cp.D = D, cp.w = w, cp.bp = bp, cp.ncl = ncl;
+        cp.Gp = G1, cp.Gp2 = G2;
+        cp.cn = cn + p0, cp.tau = tau;
+        cp.R64 = R64 + (size_t)p0 * ldr, cp.ldr = ldr, cp.rmax = rmax;
+        cp.r_start = r_at + pn, cp.r_next = r_at + pn + 1;
+        cp.st = st;
+        cfg = clustered(nslices, kSliceCluster, 512, smem_chol, at);
+        GS_CK(cudaLaunchKernelEx(&cfg, k_panel_chol<1>, (const CholParams)cp));
+        cp.Gp = G2;
+        k_panel_chol<2><<<nslices, 512, smem_chol, s>>>(cp);
+        cfg = clustered(kMgsCtas, kMgsCtas, kMgsThreads, 0, at);
+        GS_CK(cudaLaunchKernelEx(&cfg, k_panel_gs2, V, Qw, D, bp, p0, tau, (const double*)cn, R64, ldr,
+                                 (const int*)(r_at + pn), r_at + pn + 1, rmax, (const PanelState*)st));
     }
+    const int* r_dev = r_at + npanels;
     GS_CK(cudaGetLastError());
     int r = 0;
     GS_CK(cudaMemcpyAsync(&r, r_dev, sizeof(int), cudaMemcpyDeviceToHost, s));
