@@ -40,6 +40,7 @@ struct gs_basis {
     // R is lower echelon, so half h needs only its first tc_nkr_half[h] K-blocks of 64
     int tc_nh = 0, tc_half_rows = 0, tc_nkr_half[2] = {0, 0};
     int tc_npad = 0, tc_mpad = 0;
+    int ps_clusters[3] = {0, 0, 0};  // fused kernel: clusters of 2, 4, 8 CTAs that the GPU holds at once
     // R^T split the same way (tc_npad x tc_mpad), the B operand of V = P R
     void* tc_Rth = nullptr;
     void* tc_Rtl = nullptr;

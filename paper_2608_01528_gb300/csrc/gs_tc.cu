@@ -87,6 +87,7 @@ constexpr int kMaxSX = 6, kMaxSA = 2, kMaxSB = 4;
 constexpr int kTmemCols = 512;
 constexpr int kMaxKR = 4;            // K-blocks of 64 in r <= 256
 constexpr int kSCol = 256;           // first TMEM column of the score accumulator
+constexpr int kMaxKS = 8;            // CTAs that may share a tile's K range
 
 // ----------------------------------------------------------------- work split
 struct TileRange {
@@ -120,6 +121,9 @@ struct PsParams {
     long long N;
     int D, r, npad, M, mpad, nkb;
     int nh, half_rows, nkr_h[2];  // GEMM2: halves of codewords, K-blocks of R each half needs
+    int ks;                 // SPLIT: CTAs of a cluster that share a tile's K range
+    int xch_ld;             // SPLIT: floats between exchanged Y rows (npad + 4)
+    int bs_off;             // bytes from the X staging to the B ring
     int sx, sa, sb;         // ring depths: fp32 X staging, fp16 A, B operand tiles
     int box_rows;           // rows of each X TMA box (>= every tile's rows)
     int xstage;             // bytes between X staging tiles (box_rows x 256, 1 KB aligned)
@@ -131,6 +135,7 @@ struct PsParams {
     int ldy;
     float* S;
     int lds;
+    int s_vec;              // S rows are 16-byte aligned
     int* argmax;
     float* maxval;
 };
@@ -143,10 +148,11 @@ struct Ctl {
     uint64_t ysplit[kMaxKR];  // Y columns [64 k, 64 k + 64) split in TMEM (GEMM2 K-block k may start)
     uint64_t xn_full[2], xn_empty[2];
     uint64_t dec_full[2];     // redo decision of regular tile t published in slot t % 2
+    uint64_t peer_ready, xch_full;  // SPLIT: every CTA's GEMM1 is done; the peers' parts of my rows are here
     uint64_t mma_done;
     float xn[2][kBM];  // ||x||^2 per row, both converter groups add into it
     int8_t rsc[2][kBM];      // per-row exponent s of the redo's scale 2^s, for the tile in that slot
-    int redo[2][kEpiWarps];  // per epilogue warp: some row of its lane quadrant needs the redo
+    int redo[2][kMaxKS];     // per epilogue warp (SPLIT: per deciding warp of the cluster): some row needs the redo
     uint32_t tmem_base;
     int abort_flag;
 };
@@ -179,16 +185,24 @@ __device__ __forceinline__ bool walk_tiles(const CtaRows& cr, Ctl& c, Wait wait,
             const volatile int* rd = c.redo[slot];
             bool again = false;
 #pragma unroll
-            for (int w = 0; w < kEpiWarps; ++w) again |= rd[w] != 0;
+            for (int w = 0; w < kMaxKS; ++w) again |= rd[w] != 0;
             if (again && !body(d, true, q++)) return false;
         }
     }
     return true;
 }
 
+// SPLIT: for batches with fewer 128-row tiles than half the SMs, a cluster of ks CTAs takes one tile:
+// each runs GEMM1 over its part of D, then sends its partial Y (and ||x||^2) of the rows that peer q
+// owns (rows [q 128 / ks, (q + 1) 128 / ks)) into q's shared memory; q adds the parts in a fixed order
+// and goes on alone with its rows (GEMM2 over all 128 TMEM lanes, of which its own are read).  Without
+// it a 4,096-query batch ran on 32 of 152 SMs, each streaming its X tile and all of Q: 150 us at D =
+// 8192, r = M = 256 (softmax, scores out) against 58 us on 38 clusters of 4.  Splitting the rows
+// instead would have every SM stream all of Q (4 MB each, 620 MB of L2 reads).  The exchange reuses the
+// X staging and A stages, after every CTA of the cluster has finished GEMM1 (peer_ready).
 // FULL = false: raw scores with only argmax / maxval out (the large-batch lookup); true: every
 // mode and output.  A template parameter, so the lookup kernel carries none of the other paths.
-template <bool FULL>
+template <bool FULL, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 1)
     k_ps_tc(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_q,
             const __grid_constant__ CUtensorMap tmap_rh, const __grid_constant__ CUtensorMap tmap_rl,
@@ -199,12 +213,17 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint8_t* base = smem_raw + (((raw + 1023u) & ~1023u) - raw);
     uint8_t* Xs = base;
     uint8_t* As = Xs + (size_t)p.sx * p.xstage;
-    uint8_t* Bs = As + (size_t)p.sa * kAStageBytes;
+    uint8_t* Bs = Xs + p.bs_off;
     Ctl& c = *reinterpret_cast<Ctl*>(Bs + (size_t)p.sb * kBStageBytes);
     volatile int* abort_flag = &c.abort_flag;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const CtaRows cr(p.N, gridDim.x, blockIdx.x);
+    const int ks = SPLIT ? p.ks : 1;
+    const int rank = SPLIT ? (int)cluster_ctarank() : 0;
+    const CtaRows cr(p.N, gridDim.x / ks, blockIdx.x / ks);
+    const int kb0 = SPLIT ? p.nkb * rank / ks : 0, kb1 = SPLIT ? p.nkb * (rank + 1) / ks : p.nkb;
+    const int own_rows = kBM / ks;                                    // rows this CTA carries on with
+    const int own_warps = SPLIT ? std::max(1, kEpiWarps / ks) : kEpiWarps;  // epilogue warps that hold them
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < p.sx; ++s) {
@@ -220,14 +239,19 @@ __global__ void __launch_bounds__(kThreads, 1)
             mbar_init(&c.b_empty[s], 1);
         }
         mbar_init(&c.y_full, 1);
-        for (int k = 0; k < kMaxKR; ++k) mbar_init(&c.ysplit[k], kEpiWarps);
+        for (int k = 0; k < kMaxKR; ++k) mbar_init(&c.ysplit[k], own_warps);
         mbar_init(&c.s_full, 1);
-        mbar_init(&c.s_empty, kEpiWarps);
+        mbar_init(&c.s_empty, own_warps);
         mbar_init(&c.gemm2_done, 1);
         for (int b = 0; b < 2; ++b) {
             mbar_init(&c.xn_full[b], kCvtWarps);
             mbar_init(&c.xn_empty[b], kEpiWarps);
-            mbar_init(&c.dec_full[b], kEpiWarps);
+            mbar_init(&c.dec_full[b], SPLIT ? ks * own_warps : kEpiWarps);
+            for (int w = 0; w < kMaxKS; ++w) c.redo[b][w] = 0;
+        }
+        if (SPLIT) {
+            mbar_init(&c.peer_ready, ks);
+            mbar_init(&c.xch_full, (ks - 1) * own_warps);
         }
         mbar_init(&c.mma_done, 1);
         c.abort_flag = 0;
@@ -240,10 +264,19 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     tc_fence_before();
     __syncthreads();
+    if (SPLIT) cluster_sync_all();  // every CTA's barriers exist before a peer signals them
     tc_fence_after();
     const uint32_t tmem = c.tmem_base;
     auto wait_1t = [&](uint64_t* bar, uint32_t par) { return mbar_wait_1t(bar, par, abort_flag, &g_err_tc); };
     auto wait_warp = [&](uint64_t* bar, uint32_t par) { return mbar_wait_warp(bar, par, abort_flag, &g_err_tc); };
+    // a tile's redo decision: from this CTA's epilogue, or (SPLIT) from every CTA of the cluster
+    auto dec_1t = [&](uint64_t* bar, uint32_t par) {
+        return SPLIT ? mbar_wait_cluster(bar, par, abort_flag, &g_err_tc) : wait_1t(bar, par);
+    };
+    auto dec_warp = [&](uint64_t* bar, uint32_t par) {
+        return SPLIT ? __all_sync(0xffffffffu, mbar_wait_cluster(bar, par, abort_flag, &g_err_tc)) != 0
+                     : wait_warp(bar, par);
+    };
 
     if (warp == kXWarp) {
         // ------------------------------------------------------------- X tiles via TMA
@@ -252,9 +285,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             const uint32_t bytes = (uint32_t)p.box_rows * kBK * 4;
             int it = 0;
             RingPos xs;
-            walk_tiles(cr, c, wait_1t, [&](int t, bool, int) {
+            walk_tiles(cr, c, dec_1t, [&](int t, bool redo, int) {
                 const TileRange tr = cr.tile(t);
-                for (int kb = 0; kb < p.nkb; ++kb, ++it, xs.next(p.sx)) {
+                if (SPLIT && redo) fence_proxy_async();  // the exchanged rows lay where X lands again
+                for (int kb = kb0; kb < kb1; ++kb, ++it, xs.next(p.sx)) {
                     if (!wait_1t(&c.x_empty[xs.idx], xs.phase ^ 1u)) return false;
                     mbar_arrive_expect_tx(&c.x_full[xs.idx], bytes);
                     tma_load_2d(Xs + (size_t)xs.idx * p.xstage, &tmap_x, &c.x_full[xs.idx], kb * kBK, (int)tr.row0,
@@ -273,19 +307,19 @@ __global__ void __launch_bounds__(kThreads, 1)
             const uint64_t pol = l2_policy_evict_last();
             const uint32_t qbytes = (uint32_t)p.npad * kBK * 2, rbytes = 2u * (uint32_t)p.half_rows * kBK * 2;
             const uint32_t rl_off = (uint32_t)p.half_rows * kBK * 2;  // Rl after Rh in the slot
-            const int per_tile = p.nkb + p.nkr_h[0] + p.nkr_h[1];
+            const int nkb = kb1 - kb0, per_tile = nkb + p.nkr_h[0] + p.nkr_h[1];
             int it = 0;
             RingPos bs;
-            walk_tiles(cr, c, wait_1t, [&](int, bool, int) {
+            walk_tiles(cr, c, dec_1t, [&](int, bool, int) {
                 for (int k = 0; k < per_tile; ++k, ++it, bs.next(p.sb)) {
                     const int s = bs.idx;
                     if (!wait_1t(&c.b_empty[s], bs.phase ^ 1u)) return false;
                     uint8_t* dst = Bs + (size_t)s * kBStageBytes;
-                    if (k < p.nkb) {
+                    if (k < nkb) {
                         mbar_arrive_expect_tx(&c.b_full[s], qbytes);
-                        tma_load_2d(dst, &tmap_q, &c.b_full[s], k * kBK, 0, pol);
+                        tma_load_2d(dst, &tmap_q, &c.b_full[s], (kb0 + k) * kBK, 0, pol);
                     } else {
-                        const int j = k - p.nkb;
+                        const int j = k - nkb;
                         const int h = j < p.nkr_h[0] ? 0 : 1;
                         const int kr = h ? j - p.nkr_h[0] : j;
                         mbar_arrive_expect_tx(&c.b_full[s], rbytes);
@@ -304,10 +338,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             const uint32_t idesc2 = idesc_bf16_f32(p.half_rows);
             const uint32_t y_tmem = tmem, s_tmem = tmem + kSCol;
             RingPos ra, rb;
-            walk_tiles(cr, c, wait_1t, [&](int, bool, int q) {
+            walk_tiles(cr, c, dec_1t, [&](int, bool, int q) {
                 const uint32_t pt = (uint32_t)q & 1u;
                 // GEMM1: Y = X Q^T into columns [0, npad)
-                for (int kb = 0; kb < p.nkb; ++kb, ra.next(p.sa), rb.next(p.sb)) {
+                for (int kb = kb0; kb < kb1; ++kb, ra.next(p.sa), rb.next(p.sb)) {
                     const int sa = ra.idx, sb = rb.idx;
                     if (!wait_1t(&c.a_full[sa], ra.phase) || !wait_1t(&c.b_full[sb], rb.phase)) return false;
                     tc_fence_after();
@@ -316,7 +350,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
                     for (int k = 0; k < kBK / 16; ++k)
                         mma_f16_ss(y_tmem, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc1,
-                                   (kb | k) != 0 ? 1u : 0u);
+                                   (kb != kb0 || k != 0) ? 1u : 0u);
                     mma_commit(&c.a_empty[sa]);
                     mma_commit(&c.b_empty[sb]);
                 }
@@ -374,11 +408,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         float amax = 0.f;
         int it = 0;
         RingPos rx, ra;  // every K-block advances both rings; this group takes those with it % 2 == g
-        walk_tiles(cr, c, wait_warp, [&](int t, bool redo, int q) {
+        walk_tiles(cr, c, dec_warp, [&](int t, bool redo, int q) {
             const TileRange tr = cr.tile(t);
             const int b = q & 1;
             const int8_t* rs = c.rsc[t & 1];  // the rows' scale exponents (redo only)
-            for (int kb = 0; kb < p.nkb; ++kb, ++it, rx.next(p.sx), ra.next(p.sa)) {
+            for (int kb = kb0; kb < kb1; ++kb, ++it, rx.next(p.sx), ra.next(p.sa)) {
                 if ((it & 1) != g) continue;
                 const int sx = rx.idx, sa = ra.idx;
                 if (!wait_warp(&c.x_full[sx], rx.phase) || !wait_warp(&c.a_empty[sa], ra.phase ^ 1u)) return false;
@@ -441,14 +475,51 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int i = threadIdx.x;  // row within the tile = TMEM lane
         const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
         const uint32_t ty = tmem + lane_base, ts = tmem + lane_base + kSCol;
-        walk_tiles(cr, c, wait_warp, [&](int t, bool redo, int q) {
+        walk_tiles(cr, c, dec_warp, [&](int t, bool redo, int q) {
             const uint32_t pt = (uint32_t)q & 1u;
             const int b = q & 1;
             if (!wait_warp(&c.y_full, pt)) return false;
             tc_fence_after();
             const TileRange tr = cr.tile(t);
-            const bool valid = i < tr.nrows;
             const long long row = tr.row0 + i;
+            const int owner = SPLIT ? i / own_rows : 0;  // the CTA that carries on with this row
+            const bool mine = owner == rank;
+            const bool valid = i < tr.nrows && mine;
+            float xn2 = 0.f;
+            const float* parts = nullptr;  // SPLIT: this row's parts from the peers, in CTA order
+            if (SPLIT) {
+                if (!wait_warp(&c.xn_full[b], (uint32_t)(q >> 1) & 1u)) return false;
+                xn2 = c.xn[b][i];
+                c.xn[b][i] = 0.f;
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&c.xn_empty[b]);
+                // the peers may write over this CTA's X and A stages, and it over theirs
+                if (warp == 0 && lane < ks) mbar_arrive_cluster(mapa_shared(smem_u32(&c.peer_ready), (uint32_t)lane));
+                if (!__all_sync(0xffffffffu, mbar_wait_cluster(&c.peer_ready, pt, abort_flag, &g_err_tc))) return false;
+                const int src = rank < owner ? rank : rank - 1;
+                const uint32_t dst = mapa_shared(smem_u32(Xs) + 4u * (uint32_t)((src * own_rows + i % own_rows) * p.xch_ld),
+                                                 (uint32_t)owner);
+                for (int jc = 0; jc < p.npad; jc += 16) {
+                    float y[16];
+                    tmem_ld16(ty + (uint32_t)jc, y);
+                    if (!mine) {
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            st_cluster_f32x4(dst + 4u * (uint32_t)(jc + 4 * u), y[4 * u], y[4 * u + 1], y[4 * u + 2],
+                                             y[4 * u + 3]);
+                    }
+                }
+                if (!mine) st_cluster_f32x4(dst + 4u * (uint32_t)p.npad, xn2, 0.f, 0.f, 0.f);
+                __syncwarp();
+                // one arrival per group of rows of one owner (a release: the lanes' stores come before it)
+                if (!mine && lane % std::min(32, own_rows) == 0)
+                    mbar_arrive_cluster(mapa_shared(smem_u32(&c.xch_full), (uint32_t)owner));
+                if (__ballot_sync(0xffffffffu, mine) == 0u) return true;  // none of this warp's rows stay here
+                if (!__all_sync(0xffffffffu, mbar_wait_cluster(&c.xch_full, pt, abort_flag, &g_err_tc))) return false;
+                parts = reinterpret_cast<const float*>(Xs) + (size_t)(i % own_rows) * p.xch_ld;
+                if (mine)
+                    for (int u = 0; u < ks - 1; ++u) xn2 += parts[(size_t)u * own_rows * p.xch_ld + p.npad];
+            }
             // a redone tile ran on x 2^s: Y and ||x|| come back multiplied by 2^s
             const float unscale = redo ? pow2f(-c.rsc[t & 1][i]) : 1.f;
             // split Y in place: chunk of 16 fp32 columns -> 8 columns bf16(Y) + 8 columns
@@ -462,6 +533,20 @@ __global__ void __launch_bounds__(kThreads, 1)
                     tmem_ld32(ty + (uint32_t)jc, y);
                 else
                     tmem_ld16(ty + (uint32_t)jc, y);
+                if (SPLIT && mine) {
+                    for (int u = 0; u < ks - 1; ++u) {
+                        const float4* src = reinterpret_cast<const float4*>(parts + (size_t)u * own_rows * p.xch_ld + jc);
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            if (4 * j >= w) break;
+                            const float4 f = src[j];
+                            y[4 * j] += f.x;
+                            y[4 * j + 1] += f.y;
+                            y[4 * j + 2] += f.z;
+                            y[4 * j + 3] += f.w;
+                        }
+                    }
+                }
                 if (redo) {
 #pragma unroll
                     for (int j = 0; j < 32; ++j) y[j] *= unscale;
@@ -493,11 +578,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                     if (lane == 0) mbar_arrive(&c.ysplit[jc >> 6]);
                 }
             }
-            if (!wait_warp(&c.xn_full[b], (uint32_t)(q >> 1) & 1u)) return false;
-            const float xn2 = c.xn[b][i];
-            c.xn[b][i] = 0.f;  // ready for the tile after next (both groups add into it)
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&c.xn_empty[b]);
+            if (!SPLIT) {
+                if (!wait_warp(&c.xn_full[b], (uint32_t)(q >> 1) & 1u)) return false;
+                xn2 = c.xn[b][i];
+                c.xn[b][i] = 0.f;  // ready for the tile after next (both groups add into it)
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&c.xn_empty[b]);
+            }
             const float xnorm = sqrtf(xn2) * unscale;
             if (!redo) {
                 // one fp16 rounding of x is accurate when every element is inside fp16's range
@@ -505,20 +592,29 @@ __global__ void __launch_bounds__(kThreads, 1)
                 // sqrt(D): the subnormals' absolute errors, at most 2^-25 each, then add at most
                 // 2^-19 ||x|| to the error of <x, q_j>); any other nonzero row has its tile redone
                 // with an exact power-of-two scale (a norm that is not a number keeps scale 1)
-                const bool bad = xn2 > 0.f && !(xn2 >= p.xn2_lo && xn2 <= p.xn2_hi);
+                const bool bad = mine && xn2 > 0.f && !(xn2 >= p.xn2_lo && xn2 <= p.xn2_hi);
                 const int slot = t & 1;
-                c.rsc[slot][i] = (int8_t)row_scale_exp(xn2);
+                const int8_t e = (int8_t)row_scale_exp(xn2);
                 const unsigned any = __ballot_sync(0xffffffffu, bad);
-                if (lane == 0) c.redo[slot][warp] = any != 0u;
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&c.dec_full[slot]);
+                if (SPLIT) {  // to every CTA of the cluster (this one among them)
+                    const uint32_t a_rsc = smem_u32(&c.rsc[slot][i]);
+                    const uint32_t a_redo = smem_u32(&c.redo[slot][own_warps > 1 ? warp : rank]);
+                    for (int d = 0; d < ks; ++d)
+                        if (mine) st_cluster_u8(mapa_shared(a_rsc, (uint32_t)d), (uint32_t)(uint8_t)e);
+                    if (lane < ks) st_cluster_u32(mapa_shared(a_redo, (uint32_t)lane), any != 0u);
+                    __syncwarp();
+                    if (lane < ks) mbar_arrive_cluster(mapa_shared(smem_u32(&c.dec_full[slot]), (uint32_t)lane));
+                } else {
+                    c.rsc[slot][i] = e;
+                    if (lane == 0) c.redo[slot][warp] = any != 0u;
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&c.dec_full[slot]);
+                }
             }
             if (!wait_warp(&c.s_full, pt)) return false;
             tc_fence_after();
-            float best = -FLT_MAX, run_max = -FLT_MAX, run_sum = 0.f;
-            int besti = 0;
-            for (int ic = 0; ic < p.mpad; ic += 16) {
-                float sv[16];
+            // scores ci .. ci + 15 of this thread's row
+            auto scores = [&](int ic, float (&sv)[16]) {
                 tmem_ld16(ts + (uint32_t)ic, sv);
                 if (p.nkr_h[ic >= p.half_rows ? 1 : 0] == 0) {  // a half with no nonzero R: S = 0
 #pragma unroll
@@ -526,38 +622,71 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
 #pragma unroll
                 for (int j = 0; j < 16; ++j) {
+                    sv[j] *= p.scale;
+                    if (FULL && p.mode == GS_SCORE_COSINE) {
+                        const float den = ic + j < p.M ? xnorm * p.cnorm[ic + j] : 0.f;
+                        sv[j] = den > 0.f ? sv[j] / den : 0.f;
+                    }
+                }
+            };
+            auto store = [&](int ic, const float (&sv)[16]) {
+                float* dst = p.S + (size_t)row * p.lds + ic;
+                if (p.s_vec && ic + 16 <= p.M) {
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        reinterpret_cast<float4*>(dst)[u] = make_float4(sv[4 * u], sv[4 * u + 1], sv[4 * u + 2], sv[4 * u + 3]);
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 16; ++j)
+                        if (ic + j < p.M) dst[j] = sv[j];
+                }
+            };
+            float best = -FLT_MAX, run_max = -FLT_MAX, run_sum = 0.f;
+            int besti = 0;
+            for (int ic = 0; ic < p.mpad; ic += 16) {
+                float sv[16];
+                scores(ic, sv);
+                if (FULL && p.mode == GS_SCORE_SOFTMAX) {
+                    // online, sixteen at a time: one rescaling exponential per chunk, one per score
+                    float nm = run_max, add = 0.f;
+#pragma unroll
+                    for (int j = 0; j < 16; ++j)
+                        if (ic + j < p.M) nm = fmaxf(nm, sv[j]);
+#pragma unroll
+                    for (int j = 0; j < 16; ++j)
+                        if (ic + j < p.M) add += __expf(sv[j] - nm);
+                    run_sum = run_sum * __expf(run_max - nm) + add;
+                    run_max = nm;
+                }
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
                     const int ci = ic + j;
                     if (ci >= p.M) break;
-                    float g = p.scale * sv[j];
-                    if (FULL && p.mode == GS_SCORE_COSINE) {
-                        const float den = xnorm * p.cnorm[ci];
-                        g = den > 0.f ? g / den : 0.f;
-                    }
-                    if (g > best) {
-                        best = g;
+                    if (sv[j] > best) {
+                        best = sv[j];
                         besti = ci;
                     }
-                    if (FULL && p.mode == GS_SCORE_SOFTMAX) {
-                        const float nm = fmaxf(run_max, g);
-                        run_sum = run_sum * __expf(run_max - nm) + __expf(g - nm);
-                        run_max = nm;
-                    }
-                    if (FULL && p.S && valid) p.S[(size_t)row * p.lds + ci] = g;
+                }
+                if (FULL && p.S && valid && p.mode != GS_SCORE_SOFTMAX) store(ic, sv);
+            }
+            float outmax = best;
+            if (FULL && p.mode == GS_SCORE_SOFTMAX) {
+                const float inv = 1.f / run_sum;
+                outmax = __expf(best - run_max) * inv;
+                // the scores once more from TMEM (they were written unnormalised and read back before:
+                // three passes of one 4-byte access per lane and row)
+                for (int ic = 0; p.S && ic < p.mpad; ic += 16) {
+                    float sv[16];
+                    scores(ic, sv);
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) sv[j] = __expf(sv[j] - run_max) * inv;
+                    if (valid) store(ic, sv);
                 }
             }
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&c.s_empty);
             if (!valid) return true;
-            float outmax = best;
-            if (FULL && p.mode == GS_SCORE_SOFTMAX) {
-                const float inv = 1.f / run_sum;
-                outmax = __expf(best - run_max) * inv;
-                if (p.S) {
-                    float* sr = p.S + (size_t)row * p.lds;
-                    for (int ci = 0; ci < p.M; ++ci) sr[ci] = __expf(sr[ci] - run_max) * inv;
-                }
-            }
             if (p.argmax) p.argmax[row] = besti;
             if (p.maxval) p.maxval[row] = outmax;
             return true;
@@ -566,6 +695,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     tc_fence_before();
     __syncthreads();
+    if (SPLIT) cluster_sync_all();  // no CTA leaves while a peer may still write to it or signal it
     if (warp == kMmaWarp) {
         tc_fence_after();
         tmem_dealloc(tmem, kTmemCols);
@@ -617,8 +747,12 @@ constexpr size_t kSmemCap = 227 * 1024;
 // bytes between fp32 X staging tiles of `box_rows` rows (SW128 operand areas follow: 1 KB aligned)
 int ps_xstage(int box_rows) { return (box_rows * kBK * 4 + 1023) / 1024 * 1024; }
 
-size_t ps_smem_bytes(Rings g, int xstage) {
-    return 1024 + (size_t)g.sx * xstage + (size_t)g.sa * kAStageBytes + (size_t)g.sb * kBStageBytes + sizeof(Ctl);
+// xch: bytes of the exchanged rows (0: no K split), which share the X staging's and A stages' place
+size_t ps_bs_off(Rings g, int xstage, size_t xch) {
+    return std::max((size_t)g.sx * xstage + (size_t)g.sa * kAStageBytes, (xch + 1023) / 1024 * 1024);
+}
+size_t ps_smem_bytes(Rings g, int xstage, size_t xch) {
+    return 1024 + ps_bs_off(g, xstage, xch) + (size_t)g.sb * kBStageBytes + sizeof(Ctl);
 }
 
 // Ring depths for X boxes of `box_rows` rows: the deepest X ring that fits, then the
@@ -628,14 +762,30 @@ size_t ps_smem_bytes(Rings g, int xstage) {
 // can reach the stage two phases on while the other group's load into it is still in
 // flight (TMA loads may land out of order), and the parity test would then pass on the
 // stage's older, completed phase and hand over stale data.
-Rings ps_rings(int box_rows) {
+Rings ps_rings(int box_rows, size_t xch) {
     const int xs = ps_xstage(box_rows);
     for (int sx = kMaxSX; sx >= 2; sx -= 2)
         for (int sb = kMaxSB; sb >= 2; --sb) {
             Rings g{sx, kMaxSA, sb};
-            if (ps_smem_bytes(g, xs) <= kSmemCap) return g;
+            if (ps_smem_bytes(g, xs, xch) <= kSmemCap) return g;
         }
     return Rings{2, kMaxSA, 2};
+}
+
+// launch configuration of a K-split launch: `ctas` CTAs in clusters of ks
+cudaLaunchConfig_t ps_cluster_config(int ctas, int ks, size_t smem, cudaStream_t s, cudaLaunchAttribute* at) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)ctas);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    at->id = cudaLaunchAttributeClusterDimension;
+    at->val.clusterDim.x = (unsigned)ks;
+    at->val.clusterDim.y = 1;
+    at->val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cfg;
 }
 
 }  // namespace
@@ -731,18 +881,25 @@ gs_status tc_prepare(gs_basis* h) {
         !make_tmap_2d(&h->tmap_rl, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, h->tc_Rl, mpad, npad, npad, kBK,
                       h->tc_half_rows, CU_TENSOR_MAP_SWIZZLE_128B))
         return GS_ERR_CUDA;
-    if (cudaFuncSetAttribute(k_ps_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemCap) !=
-            cudaSuccess ||
-        cudaFuncSetAttribute(k_ps_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemCap) !=
-            cudaSuccess)
-        return GS_ERR_CUDA;
     // the fused kernel needs all of its threads resident in one CTA; otherwise the
     // basis simply has no fused tensor-core similarity path
-    cudaFuncAttributes fa, fb;
-    if (cudaFuncGetAttributes(&fa, k_ps_tc<false>) != cudaSuccess ||
-        cudaFuncGetAttributes(&fb, k_ps_tc<true>) != cudaSuccess)
-        return GS_ERR_CUDA;
-    h->has_tmap_q16 = fa.maxThreadsPerBlock >= kThreads && fb.maxThreadsPerBlock >= kThreads;
+    bool fits = true;
+    for (auto fn : {k_ps_tc<false, false>, k_ps_tc<true, false>, k_ps_tc<false, true>, k_ps_tc<true, true>}) {
+        cudaFuncAttributes fa;
+        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemCap) != cudaSuccess ||
+            cudaFuncGetAttributes(&fa, fn) != cudaSuccess)
+            return GS_ERR_CUDA;
+        fits = fits && fa.maxThreadsPerBlock >= kThreads;
+    }
+    h->has_tmap_q16 = fits;
+    // clusters of 2, 4 and 8 CTAs that the GPU holds at once (GPCs need not hold whole numbers of them)
+    for (int i = 0; i < 3; ++i) {
+        cudaLaunchAttribute at[1];
+        cudaLaunchConfig_t cfg = ps_cluster_config(2 << i, 2 << i, kSmemCap, 0, at);
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, k_ps_tc<true, true>, &cfg) != cudaSuccess) return GS_ERR_CUDA;
+        h->ps_clusters[i] = n;
+    }
     return GS_OK;
 }
 
@@ -750,7 +907,17 @@ cudaError_t launch_ps_tc(const gs_basis* h, const float* X, long long N, int ldx
                          int ldy, float* S, int lds, int* argmax, float* maxval, cudaStream_t s) {
     if (!h->has_tmap_q16) return cudaErrorNotSupported;
     const long long tiles = (N + kBM - 1) / kBM;
-    const int grid = (int)std::min<long long>(num_sms(h->device), tiles);
+    // Fewer tiles than half the SMs: clusters of ks CTAs share each tile's K range, as many clusters as
+    // the GPU holds (their rows even out).  A K-block takes a CTA ~0.65 us, the exchange and what only the
+    // row's owner does after it up to ~20 us at r = M = 256 (10 us at 32), so the K-blocks saved have
+    // to be worth 20 us.  Measured at r = M = 256, 4,096 queries: D = 4096: 39 us (50 without), 8192: 50
+    // (92), 16,384: 70; D = 2048 is left alone.
+    const int nkb = (h->D + kBK - 1) / kBK;
+    int ks = 1, clusters = 0;
+    for (int i = 0; i < 3; ++i)
+        if (tiles <= h->ps_clusters[i] && 0.65 * (nkb - nkb / (2 << i)) > 20.0)
+            ks = 2 << i, clusters = h->ps_clusters[i];
+    const int grid = (int)(ks > 1 ? std::min<long long>(clusters, N) : std::min<long long>(num_sms(h->device), tiles));
     // the X box must cover the largest tile of any CTA (CTAs differ by one row)
     int box_rows = 1;
     for (int cta : {0, grid - 1}) box_rows = std::max(box_rows, CtaRows(N, grid, cta).tsize);
@@ -758,7 +925,9 @@ cudaError_t launch_ps_tc(const gs_basis* h, const float* X, long long N, int ldx
     if (!make_tmap_2d(&tmx, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, X, N, h->D, ldx, kBK, box_rows,
                       CU_TENSOR_MAP_SWIZZLE_NONE))
         return cudaErrorInvalidValue;
-    const Rings g = ps_rings(box_rows);
+    const int xch_ld = h->tc_npad + 4;  // 16 bytes of shift per row: the row-per-thread accesses spread over the banks
+    const size_t xch = ks > 1 ? sizeof(float) * (size_t)(ks - 1) * (kBM / ks) * xch_ld : 0;
+    const Rings g = ps_rings(box_rows, xch);
     if (g.sx % kCvtGroups != 0 || g.sa % kCvtGroups != 0) return cudaErrorInvalidConfiguration;
     PsParams p;
     p.N = N;
@@ -767,7 +936,7 @@ cudaError_t launch_ps_tc(const gs_basis* h, const float* X, long long N, int ldx
     p.npad = h->tc_npad;
     p.M = h->M;
     p.mpad = h->tc_mpad;
-    p.nkb = (h->D + kBK - 1) / kBK;
+    p.nkb = nkb;
     p.nh = h->tc_nh;
     p.half_rows = h->tc_half_rows;
     p.nkr_h[0] = h->tc_nkr_half[0];
@@ -777,6 +946,10 @@ cudaError_t launch_ps_tc(const gs_basis* h, const float* X, long long N, int ldx
     p.sb = g.sb;
     p.box_rows = box_rows;
     p.xstage = ps_xstage(box_rows);
+    p.ks = ks;
+    p.xch_ld = xch_ld;
+    p.bs_off = (int)ps_bs_off(g, p.xstage, xch);
+    p.s_vec = (uintptr_t)S % 16 == 0 && lds % 4 == 0;
     // one fp16 rounding of a row is accurate for 2^-8 sqrt(D) <= ||x|| <= 2^15; other rows are redone
     p.xn2_lo = (float)h->D * 0x1p-16f;
     p.xn2_hi = 0x1p30f;
@@ -789,11 +962,20 @@ cudaError_t launch_ps_tc(const gs_basis* h, const float* X, long long N, int ldx
     p.lds = lds;
     p.argmax = argmax;
     p.maxval = maxval;
-    if (mode == GS_SCORE_RAW && !Y && !S)
-        k_ps_tc<false><<<grid, kThreads, ps_smem_bytes(g, p.xstage), s>>>(tmx, h->tmap_q16, h->tmap_rh, h->tmap_rl, p);
-    else
-        k_ps_tc<true><<<grid, kThreads, ps_smem_bytes(g, p.xstage), s>>>(tmx, h->tmap_q16, h->tmap_rh, h->tmap_rl, p);
-    return cudaGetLastError();
+    const bool full = mode != GS_SCORE_RAW || Y || S;
+    const size_t smem = ps_smem_bytes(g, p.xstage, xch);
+    if (smem > kSmemCap) return cudaErrorInvalidConfiguration;
+    if (ks == 1) {
+        if (full)
+            k_ps_tc<true, false><<<grid, kThreads, smem, s>>>(tmx, h->tmap_q16, h->tmap_rh, h->tmap_rl, p);
+        else
+            k_ps_tc<false, false><<<grid, kThreads, smem, s>>>(tmx, h->tmap_q16, h->tmap_rh, h->tmap_rl, p);
+        return cudaGetLastError();
+    }
+    cudaLaunchAttribute at[1];
+    cudaLaunchConfig_t cfg = ps_cluster_config(grid * ks, ks, smem, s, at);
+    return cudaLaunchKernelEx(&cfg, full ? k_ps_tc<true, true> : k_ps_tc<false, true>, tmx, h->tmap_q16, h->tmap_rh,
+                              h->tmap_rl, p);
 }
 
 }  // namespace gs

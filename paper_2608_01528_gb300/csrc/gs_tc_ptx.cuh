@@ -318,6 +318,17 @@ static __device__ __forceinline__ void tma_load_2d_pair(void* dst, const CUtenso
 static __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cbar) {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cbar) : "memory");
 }
+// Plain stores into the shared memory of a CTA of the cluster (shared::cluster address).
+static __device__ __forceinline__ void st_cluster_f32x4(uint32_t caddr, float a, float b, float c, float d) {
+    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(caddr), "f"(a), "f"(b), "f"(c), "f"(d)
+                 : "memory");
+}
+static __device__ __forceinline__ void st_cluster_u32(uint32_t caddr, uint32_t v) {
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(caddr), "r"(v) : "memory");
+}
+static __device__ __forceinline__ void st_cluster_u8(uint32_t caddr, uint32_t v) {
+    asm volatile("st.shared::cluster.u8 [%0], %1;" ::"r"(caddr), "r"(v) : "memory");
+}
 // Instruction descriptor of a pair MMA, kind::f16: D f32, A = B = f16, both K-major, N, M = 256.
 __host__ __device__ constexpr uint32_t idesc2_f16_f32(int n) {
     return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
