@@ -56,6 +56,8 @@ struct AttnParams {
     float scale;
     float* A;                // B x Lq x Lk
     int a_vec;               // rows aligned for two-element stores (Lk even, A 8-byte aligned)
+    int cl_ctas;             // k_attn_cl: CTAs of a cluster
+    int a_tma;               // k_attn_cl: A's rows are 16-byte aligned (tensor stores)
 };
 
 struct Ctl {
@@ -345,11 +347,15 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 // ================================================================= one pass, key units spread over a cluster
-// With the row softmax and Lk <= 4 x 256, the G = ceil(Lk / 256) CTAs of a thread-block
-// cluster share each work item: CTA g computes the logits of keys [256 g, 256 g + 256)
-// for the item's 128 queries, once.  The epilogue warps form two teams that take the
-// items in turn (team t: items t, t + 2, ...; TMEM accumulator t), so one team's exchange
-// and writes overlap the other team's statistics.  A team thread owns one query row and
+// With the row softmax and Lk <= 16 x 256, the CTAs of a thread-block cluster share each work
+// item: every key unit of 256 is computed once, for the item's 128 queries.  Up to four units
+// (U = 1): one per CTA, CTA g taking keys [256 g, 256 g + 256); the epilogue warps form two teams
+// that take the items in turn (team t: items t, t + 2, ...; TMEM accumulator t), so one team's
+// exchange and writes overlap the other team's statistics.  Five to sixteen units (U = 2): two per CTA,
+// clusters of G = 3 to 8 (larger clusters than 8 leave GPCs partly empty); team t takes unit 2 g + t
+// of every item, and the next item's MMAs of a unit start when its team has read its accumulator.
+// (The two-pass kernel above computes every logit twice: 8 sequences of 2,900 x 2,900, r = 384: 241 us
+// there, 114 us here.)  A team thread owns one query row and
 // 128 of the unit's keys, read from TMEM in two 64-key passes: the statistics pass takes,
 // in base-2 units, the max m of c s_j (c = scale log2 e) and l = sum 2^(c s_j - m); the two
 // key halves of each row meet in shared memory, the team posts each row's CTA result to
@@ -357,7 +363,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 // row's max M and sum L are known; the writing pass reads the logits again and writes
 // 2^(c s_j - M) / L.  The logits never leave the chip.  Outputs go through a 64-byte-
 // swizzled 32 x 16 fp32 tile per warp and TMA tensor stores over a 3-D map (B x Lq x Lk),
-// which clips rows past Lq and keys past Lk.  (Multicasting the query tile across the cluster
+// which clips rows past Lq and keys past Lk; rows that are not 16-byte aligned (Lk % 4 != 0) are
+// stored from the tile by the warp's lanes, half a row of 16 floats each.  (Multicasting the query tile across the cluster
 // halved its L2 reads but tied every CTA's stage release to the slowest CTA: 2 % slower.)
 //
 // Warp roles (576 threads): 0-7 team 0 and 8-15 team 1 (warp w: TMEM lanes 32 (w % 4) =
@@ -365,7 +372,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 // merge and post their rows), 16 TMA producer (query and key K-blocks into one stage), 17
 // TMEM allocator + MMA issuer.
 
-constexpr int kClMaxG = 4;
+constexpr int kClMaxG = 8;                 // CTAs of a cluster
+constexpr int kClOneG = 4;                 // up to this many units: one per CTA
+constexpr int kClMaxUnits = 2 * kClMaxG;
 constexpr int kClStageBytes = kQBlockBytes + kKStageBytes;  // 48 KB: query block, then key block
 constexpr int kClStages = 3;
 constexpr int kClEpiWarps = 16;
@@ -382,7 +391,8 @@ struct ClCtl {
     uint64_t x_full[2][2];           // team t, slot s: every CTA's row results of an item
     uint64_t mma_done;
     float2 part[2][2][kBM];             // [team][key half][query row] = (max, sum)
-    float2 xch[2][2][kClMaxG][kBM];     // [team][slot][rank][query row] = (max, sum)
+    // [team][slot][rank][query row] (U = 1) or [slot][unit][query row] (U = 2) = (max, sum)
+    float2 xch[2 * kClMaxUnits * kBM];
     uint32_t tmem_base;
     int abort_flag;
 };
@@ -409,18 +419,20 @@ __device__ __forceinline__ float row_extreme(const float* v, int n) {
 }
 
 // merge of partial (max, sum) pairs taken in base 2 (empty parts are (-inf, 0))
+template <int MAXN>
 __device__ __forceinline__ float2 merge_stats(const float2* e, int n) {
     float M = -INFINITY;
 #pragma unroll
-    for (int j = 0; j < kClMaxG; ++j)
+    for (int j = 0; j < MAXN; ++j)
         if (j < n) M = fmaxf(M, e[j].x);
     float L = 0.f;
 #pragma unroll
-    for (int j = 0; j < kClMaxG; ++j)
+    for (int j = 0; j < MAXN; ++j)
         if (j < n && e[j].y > 0.f) L += e[j].y * ex2_approx(e[j].x - M);
     return make_float2(M, L);
 }
 
+template <int U>
 __global__ void __launch_bounds__(kClThreads, 1)
     k_attn_cl(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
               const __grid_constant__ CUtensorMap tmap_a, const AttnParams p) {
@@ -435,7 +447,7 @@ __global__ void __launch_bounds__(kClThreads, 1)
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
-    const int G = p.ntiles;  // CTAs per cluster = key units per row
+    const int G = p.cl_ctas;
     const long long cid = cluster_id_x(), ncl = cluster_count_x();
     const long long items = (long long)p.B * p.qtiles;
     const int nitems = items > cid ? (int)((items - 1 - cid) / ncl + 1) : 0;
@@ -480,9 +492,9 @@ __global__ void __launch_bounds__(kClThreads, 1)
             RingPos st;
             int it = 0;
             bool ok = true;
-            for (int li = 0; li < nitems && ok; ++li) {
+            for (int li = 0; li < nitems * U && ok; ++li) {  // (item, unit of this CTA)
                 int b, qt;
-                item_bq(li, b, qt);
+                item_bq(li / U, b, qt);
                 for (int kb = 0; kb < nkb; ++kb, ++it, st.next(kClStages)) {
                     if (!mbar_wait_1t(&c.empty[st.idx], st.phase ^ 1u, abort_flag, err)) {
                         ok = false;
@@ -492,7 +504,7 @@ __global__ void __launch_bounds__(kClThreads, 1)
                     mbar_arrive_expect_tx(&c.full[st.idx], kClStageBytes);
                     tma_load_2d(dst, &tmap_q, &c.full[st.idx], kb * kBK, b * p.Lq + qt * kBM, pol);
                     tma_load_2d(dst + kQBlockBytes, &tmap_k, &c.full[st.idx], kb * kBK,
-                                b * p.Lk + (int)rank * kBN, pol);
+                                b * p.Lk + ((int)rank * U + li % U) * kBN, pol);
                 }
             }
             for (int j = std::max(0, it - kClStages); j < it; ++j)
@@ -504,7 +516,7 @@ __global__ void __launch_bounds__(kClThreads, 1)
             const uint32_t idesc = idesc_bf16_f32(kBN);
             RingPos st;
             bool ok = true;
-            for (int li = 0; li < nitems && ok; ++li) {
+            for (int li = 0; li < nitems * U && ok; ++li) {
                 const int buf = li & 1;
                 if (!mbar_wait_1t(&c.d_empty[buf], ((uint32_t)(li >> 1) & 1u) ^ 1u, abort_flag, err)) break;
                 tc_fence_after();
@@ -533,15 +545,19 @@ __global__ void __launch_bounds__(kClThreads, 1)
         // ------------------------------------------------------------- epilogue (two teams)
         const int team = warp >> 3, quad = warp & 3, kh = (warp >> 2) & 1;
         const int i = quad * 32 + lane;                          // query row within the item
-        const int keyh = (int)rank * kBN + kh * (kBN / 2);       // first of this warp's 128 keys
+        const int unit = U == 1 ? (int)rank : 2 * (int)rank + team;
+        const int keyh = unit * kBN + kh * (kBN / 2);            // first of this warp's 128 keys
         const float c2 = p.scale * 1.4426950408889634f;
         uint8_t* sb = Stg + (size_t)warp * kClStgBytes;
         const uint32_t lane_base = (uint32_t)(quad * 32) << 16;
         const uint32_t tcol = (uint32_t)(team * kBN + kh * (kBN / 2));
-        for (int li = team; li < nitems; li += 2) {
+        const int nunits = G * U;
+        const int xbar = U == 1 ? team : 0;          // barrier pair of the exchange
+        for (int li = team; li < nitems * U; li += 2) {
             int b, qt;
-            item_bq(li, b, qt);
+            item_bq(li / U, b, qt);
             const int k = li >> 1;                   // this team's k-th item
+            float2* xch = c.xch + (U == 1 ? (team * 2 + (k & 1)) * kClOneG : (k & 1) * kClMaxUnits) * kBM;
             const uint32_t ph = (uint32_t)k & 1u;    // phase of d_full[team] / p_full[team]
             const int xs = k & 1;                    // exchange slot (two per team)
             const uint32_t xph = (uint32_t)(k >> 1) & 1u;
@@ -587,27 +603,29 @@ __global__ void __launch_bounds__(kClThreads, 1)
             if (lane == 0) mbar_arrive(&c.p_full[team]);
             if (kh == 0) {
                 if (!mbar_wait_warp(&c.p_full[team], ph, abort_flag, err)) break;
-                float2 e[kClMaxG];
+                float2 e[2];
                 e[0] = c.part[team][0][i];
                 e[1] = c.part[team][1][i];
-                const float2 rc = merge_stats(e, 2);
-                const uint32_t slot = smem_u32(&c.xch[team][xs][rank][i]);
-                const uint32_t bar = smem_u32(&c.x_full[team][xs]);
+                const float2 rc = merge_stats<2>(e, 2);
+                const uint32_t slot = smem_u32(xch + unit * kBM + i);
+                const uint32_t bar = smem_u32(&c.x_full[xbar][xs]);
                 // the barrier's one arrival per phase carries the byte count of every CTA's
                 // posts; the posts are asynchronous stores that complete those bytes (a
                 // release-arrive after plain remote stores cost microseconds per item)
-                if (quad == 0 && lane == 0) mbar_arrive_expect_tx(&c.x_full[team][xs], (uint32_t)(G * kBM * 8));
+                if (quad == 0 && lane == 0 && team == (U == 1 ? team : 0))
+                    mbar_arrive_expect_tx(&c.x_full[xbar][xs], (uint32_t)(nunits * kBM * 8));
                 for (int g = 0; g < G; ++g)
                     st_async_f32x2(mapa_shared(slot, (uint32_t)g), rc.x, rc.y, mapa_shared(bar, (uint32_t)g));
             }
-            const bool got = mbar_wait_cluster(&c.x_full[team][xs], xph, abort_flag, err);
+            const bool got = mbar_wait_cluster(&c.x_full[xbar][xs], xph, abort_flag, err);
             if (!__all_sync(0xffffffffu, got)) break;
             float M, invL;
             {
-                float2 e[kClMaxG];
+                constexpr int kMax = U == 1 ? kClOneG : kClMaxUnits;
+                float2 e[kMax];
 #pragma unroll
-                for (int q = 0; q < kClMaxG; ++q) e[q] = q < G ? c.xch[team][xs][q][i] : make_float2(-INFINITY, 0.f);
-                const float2 rw = merge_stats(e, G);
+                for (int q = 0; q < kMax; ++q) e[q] = q < nunits ? xch[q * kBM + i] : make_float2(-INFINITY, 0.f);
+                const float2 rw = merge_stats<kMax>(e, nunits);
                 M = rw.x;
                 invL = rw.y > 0.f ? __fdividef(1.f, rw.y) : 0.f;
             }
@@ -645,11 +663,23 @@ __global__ void __launch_bounds__(kClThreads, 1)
                                                      ex2_approx(fmaf(vv[3], c2, -M)) * invL);
                         *reinterpret_cast<float4*>(sb + lane * 64 + ((u ^ ((lane >> 1) & 3)) << 4)) = o;
                     }
-                    fence_proxy_async();
-                    __syncwarp();
-                    if (lane == 0) {
-                        if (x < p.Lk && y < p.Lq) tma_store_3d(&tmap_a, sb, x, y, b);
-                        bulk_commit();
+                    if (p.a_tma) {
+                        fence_proxy_async();
+                        __syncwarp();
+                        if (lane == 0) {
+                            if (x < p.Lk && y < p.Lq) tma_store_3d(&tmap_a, sb, x, y, b);
+                            bulk_commit();
+                        }
+                    } else {
+                        __syncwarp();
+                        const int key = x + (lane & 15);
+                        float* dst = p.A + ((size_t)b * p.Lq + y + (lane >> 4)) * p.Lk + key;
+#pragma unroll 4
+                        for (int rr = lane >> 4; rr < 32; rr += 2, dst += 2 * (size_t)p.Lk) {
+                            const float o = *reinterpret_cast<const float*>(
+                                sb + rr * 64 + ((((lane & 15) >> 2) ^ ((rr >> 1) & 3)) << 4) + (lane & 3) * 4);
+                            if (key < p.Lk && y + rr < p.Lq) __stcs(dst, o);
+                        }
                     }
                 }
             }
@@ -675,7 +705,7 @@ static_assert(kSmemBytes <= 227 * 1024, "attention kernel shared memory exceeds 
 
 bool g_attr_set[64];
 bool g_cl_attr_set[64];
-int g_cl_max[64][kClMaxG + 1];  // active clusters of k_attn_cl per device and cluster size
+int g_cl_max[64][2][kClMaxG + 1];  // active clusters of k_attn_cl per device, U - 1 and cluster size
 
 }  // namespace
 
@@ -712,11 +742,15 @@ cudaError_t launch_attn_tc(const void* Yq, const void* Yk, int B, int Lq, int Lk
         return cudaErrorInvalidValue;
     const long long items = (long long)B * p.qtiles;
     CUtensorMap ta;
-    if (softmax && p.ntiles <= kClMaxG && Lk % 4 == 0 && (uintptr_t)A % 16 == 0 &&
-        make_tmap_3d(&ta, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, A, Lk, Lq, B, Lk, (long long)Lq * Lk, kClStgCols, 32,
-                     CU_TENSOR_MAP_SWIZZLE_64B)) {
-        // one pass: the key units of a row spread over a cluster of ntiles CTAs
-        const int G = p.ntiles;
+    p.a_tma = Lk % 4 == 0 && (uintptr_t)A % 16 == 0;
+    if (softmax && p.ntiles <= kClMaxUnits &&
+        make_tmap_3d(&ta, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, p.a_tma ? (const void*)A : Yq, p.a_tma ? Lk : 16,
+                     p.a_tma ? Lq : 1, p.a_tma ? B : 1, p.a_tma ? Lk : 16, p.a_tma ? (long long)Lq * Lk : 16, kClStgCols,
+                     32, CU_TENSOR_MAP_SWIZZLE_64B)) {  // (without tensor stores: any valid map, never used)
+        // one pass: the key units of a row spread over a cluster, one unit per CTA or two
+        const int U = p.ntiles <= kClOneG ? 1 : 2, G = (p.ntiles + U - 1) / U;
+        auto kern = U == 1 ? k_attn_cl<1> : k_attn_cl<2>;
+        p.cl_ctas = G;
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -730,23 +764,24 @@ cudaError_t launch_attn_tc(const void* Yq, const void* Yk, int B, int Lq, int Lk
         cfg.numAttrs = 1;
         if (device < 0 || device >= 64) return cudaErrorInvalidDevice;
         if (!g_cl_attr_set[device]) {
-            cudaError_t e =
-                cudaFuncSetAttribute(k_attn_cl, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClSmemBytes);
-            if (e != cudaSuccess) return e;
+            for (auto fn : {k_attn_cl<1>, k_attn_cl<2>}) {
+                cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClSmemBytes);
+                if (e != cudaSuccess) return e;
+            }
             g_cl_attr_set[device] = true;
         }
-        int& ncl_max = g_cl_max[device][G];
+        int& ncl_max = g_cl_max[device][U - 1][G];
         if (ncl_max <= 0) {
             int sms = 0;
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
             cfg.gridDim = dim3((unsigned)(std::max(sms, G) / G * G));
-            cudaError_t e = cudaOccupancyMaxActiveClusters(&ncl_max, k_attn_cl, &cfg);
+            cudaError_t e = cudaOccupancyMaxActiveClusters(&ncl_max, kern, &cfg);
             if (e != cudaSuccess) return e;
             if (ncl_max <= 0) return cudaErrorInvalidConfiguration;
         }
         const long long ncl = std::min<long long>(ncl_max, items);
         cfg.gridDim = dim3((unsigned)(ncl * G));
-        cudaError_t e = cudaLaunchKernelEx(&cfg, k_attn_cl, tq, tk, ta, p);
+        cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tq, tk, ta, p);
         if (e != cudaSuccess) return e;
         return cudaGetLastError();
     }

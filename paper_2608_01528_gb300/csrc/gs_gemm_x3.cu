@@ -57,7 +57,7 @@ constexpr int kThreads = (kCvt0 + kCvtWarps) * 32;  // 544: at most five warps a
 constexpr int kPlane = 128 * 64 * 2;                // 16 KB: one bf16 plane of 128 rows, two K-blocks wide
 constexpr int kPairBytes = 6 * kPlane;              // A h, m, l then B h, m, l of two K-blocks
 constexpr int kStages = 4;                          // K-blocks: stage s is half s & 1 of pair s >> 1
-constexpr int kChunk = 8;                           // K-blocks of hh summed on the tensor core at a time
+constexpr int kChunk = 4;                           // K-blocks of hh summed on the tensor core at a time
 constexpr int kSlots = 4;                           // tasks of one warp, per operand: 16 tasks over four warps
 constexpr int kTmemCols = 512;                      // hh: 2 x 128, small products: 2 x 128
 

@@ -1,0 +1,41 @@
+"""Row-softmax attention scores over more than 1,024 keys (two key units per CTA of a cluster) and over
+rows that are not 16-byte aligned, against 64-bit scores of the same bf16 inputs: relative 2e-2 is the
+documented bound; the inputs are exact in bf16, so 1e-4 of the row's maximum must hold (fp32 sums of at
+most 512 products, exponentials good to 2^-22)."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B,Lq,Lk,r", [
+    (2, 130, 1025, 64), (1, 256, 1280, 512), (3, 100, 1537, 72), (2, 300, 2048, 128), (1, 129, 2049, 200),
+    (2, 513, 2900, 384), (1, 128, 3333, 8), (2, 200, 4095, 96), (40, 131, 4096, 64), (1, 200, 4097, 64),
+    (9, 200, 1, 512), (5, 129, 255, 256), (4, 300, 257, 192), (3, 500, 1022, 128), (64, 300, 1023, 64)])
+@pytest.mark.parametrize("scale", [0.06, -0.2])
+def test_softmax_rows(gs, B, Lq, Lk, r, scale):
+    g = torch.Generator(device="cuda").manual_seed(B * 1000 + Lk)
+    q = torch.randn((B, Lq, r), generator=g, device="cuda").bfloat16()
+    k = torch.randn((B, Lk, r), generator=g, device="cuda").bfloat16()
+    ref = torch.softmax(scale * (q.double() @ k.double().transpose(1, 2)), dim=2)
+    first = None
+    for _ in range(3):
+        out = torch.full((B * Lq * Lk + 8,), -7.0, device="cuda")
+        A = gs.attention_scores(q, k, scale, path="tensor", out=out[:B * Lq * Lk].view(B, Lq, Lk))
+        gs.stream_status()
+        assert bool((out[B * Lq * Lk:] == -7.0).all())  # nothing past the end
+        err = (A.double() - ref).abs()
+        assert bool((err <= 1e-4 * ref.amax(2, keepdim=True)).all())
+        first = A if first is None else first
+        assert torch.equal(A, first)
+
+
+def test_unaligned_output(gs):
+    g = torch.Generator(device="cuda").manual_seed(1)
+    q = torch.randn((2, 200, 64), generator=g, device="cuda").bfloat16()
+    k = torch.randn((2, 1600, 64), generator=g, device="cuda").bfloat16()
+    out = torch.empty(2 * 200 * 1600 + 1, device="cuda")[1:].view(2, 200, 1600)
+    A = gs.attention_scores(q, k, 0.1, path="tensor", out=out)
+    gs.stream_status()
+    ref = torch.softmax(0.1 * (q.double() @ k.double().transpose(1, 2)), dim=2)
+    assert float((A.double() - ref).abs().max()) <= 1e-5
