@@ -92,6 +92,7 @@ struct GemmParams {
     int c_bf16, c_vec;      // c_vec: rows aligned for two-element stores
     float alpha;
     const float* rownorm;
+    const float* rownorm2;  // the squared norms in two parts (i and m + i), in place of rownorm
     const float* colnorm;
     // K-blocks [kb_lo[tn], kb_hi[tn]) of column tile tn (krange = 1); outside them B's rows of the
     // tile are zero (R's echelon structure), so skipping them changes no sum
@@ -522,7 +523,13 @@ __global__ void __maxnreg__(96)  // 608 threads: at most 96 registers each (see 
                 float rn[2], rm[2];
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    rn[h] = (p.rownorm && row[h] < p.m) ? p.rownorm[row[h]] : 1.f;
+                    rn[h] = 1.f;
+                    if (row[h] < p.m) {
+                        if (p.rownorm2)
+                            rn[h] = sqrtf(p.rownorm2[row[h]] + p.rownorm2[p.m + row[h]]);
+                        else if (p.rownorm)
+                            rn[h] = p.rownorm[row[h]];
+                    }
                     rm[h] = (p.rowmul && row[h] < p.m) ? p.rowmul[row[h]] * p.alpha : p.alpha;
                 }
                 for (int jc = 32 * chunk; jc < tw; jc += 32 * nchunks) {
@@ -946,7 +953,7 @@ cudaError_t launch_gemm_tc(const GemmTcArgs& a, int device, cudaStream_t s) {
     // fp16 A (T rounded once, the reconstruction): the CTA-pair kernel, whose SMs stage half of B each,
     // for products of at least one full pair tile (256 rows, 256 columns: the pair MMA is run at
     // N = 256 only, the only width its tests cover; the reconstruction needs D >= 1024 anyway)
-    if (a.a_half && !a.split && !a.c_bf16 && !a.rownorm && !a.colnorm && !a.b_klo && a.m >= 256 && a.n >= 256 &&
+    if (a.a_half && !a.split && !a.c_bf16 && !a.rownorm && !a.rownorm2 && !a.colnorm && !a.b_klo && a.m >= 256 && a.n >= 256 &&
         (uintptr_t)a.C % 16 == 0 && a.ldc % 4 == 0)  // the output's tensor map: 16-byte rows
         return launch_gemm_tc2(a, device, s);
     GemmParams p;
@@ -1007,6 +1014,7 @@ cudaError_t launch_gemm_tc(const GemmTcArgs& a, int device, cudaStream_t s) {
     p.c_vec = ((uintptr_t)a.C % (a.c_bf16 ? 4 : 8) == 0) && (a.ldc % 2 == 0);
     p.alpha = a.alpha;
     p.rownorm = a.rownorm;
+    p.rownorm2 = a.rownorm2;
     p.colnorm = a.colnorm;
     p.xn2 = p.amode == kAF16 ? a.xn2_out : nullptr;
     p.rowmul = a.rowmul;

@@ -12,10 +12,10 @@
 // left out are below 2^-24 of each term.  The tensor core's fp32 accumulation loses a bounded
 // amount at every step, which grows with the number of steps rather than with its square root, so
 // (1) hh has an accumulator of its own, the five small products share another (their sum is ~2^-8 of
-// hh's, and so are its losses), and (2) hh's accumulator is emptied every kChunk K-blocks (256 terms)
+// hh's, and so are its losses), and (2) hh's accumulator is emptied every kChunk K-blocks (128 terms)
 // into fp32 registers (round to nearest).  Relative error against 64 bits, 16,384 x 922 -> 10,000:
-// 1.3e-7, the CUDA-core GEMM's 5.4e-7; at 300 terms 1.5e-7 and 3.1e-7.  (Chunks of 512 terms: 2.4e-7,
-// and 5.1e-7 against 4.5e-7 where all terms of a sum have one sign.)
+// 9e-8, the CUDA-core GEMM's 5.4e-7; at 300 terms 9e-8 and 3.1e-7.  (Chunks of 256 terms: 1.3e-7 at the
+// same speed, but 4.9e-7 against 4.1e-7 where all terms of a sum have one sign; of 512: 2.4e-7.)
 // Outputs of a thread that holds one that is not finite (an operand that is not, or beyond bf16's
 // range) are computed again as plain fp32 dot products, so infinities and NaN come out as the
 // CUDA-core GEMM has them.
@@ -517,7 +517,7 @@ unsigned take_device_error_x3() {
     return v;
 }
 
-static cudaError_t launch_gemm_x3(const GemmArgs& g, int sms, cudaStream_t s) {
+static cudaError_t launch_gemm_x3(const GemmArgs& g, int sms, int device, cudaStream_t s) {
     X3Params p;
     p.A = g.A;
     p.B = (const float*)g.B;
@@ -548,8 +548,13 @@ static cudaError_t launch_gemm_x3(const GemmArgs& g, int sms, cudaStream_t s) {
     const int grid = (int)std::min<long long>(sms, p.tiles);
 #define GS_X3_CASE(TA, BT, VEC)                                                                     \
     if (g.a_type == TA && g.b_trans == BT && vec == VEC) {                                          \
-        cudaError_t e = cudaFuncSetAttribute(k_gemm_x3<TA, BT, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
-        if (e != cudaSuccess) return e;                                                             \
+        static bool set[64];                                                                        \
+        if (device < 0 || device >= 64) return cudaErrorInvalidDevice;                              \
+        if (!set[device]) {                                                                         \
+            cudaError_t e = cudaFuncSetAttribute(k_gemm_x3<TA, BT, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
+            if (e != cudaSuccess) return e;                                                         \
+            set[device] = true;                                                                     \
+        }                                                                                           \
         k_gemm_x3<TA, BT, VEC><<<grid, kThreads, smem, s>>>(p);                                     \
         return cudaGetLastError();                                                                  \
     }
@@ -580,7 +585,7 @@ cudaError_t launch_gemm_fp32(const GemmArgs& g, bool simt, int device, cudaStrea
         sms = std::max(sms, 1);
         const double tiles = (double)((g.m + kBM - 1) / kBM) * ((g.n + kBN - 1) / kBN) * g.batch;
         const double x3_us = 8.0 + std::ceil(tiles / sms) * (0.9 * ((g.k + kBK - 1) / kBK) + 6.0);
-        if (x3_us < simt_us) return launch_gemm_x3(g, sms, s);
+        if (x3_us < simt_us) return launch_gemm_x3(g, sms, device, s);
     }
     return launch_gemm_simt(g, s);
 }

@@ -190,6 +190,9 @@ struct GemmTcArgs {
     const void* B0; const void* B1; long long ldb; int n;
     void* C; long long ldc; bool c_bf16; float alpha;
     const float* rownorm; const float* colnorm;
+    // instead of rownorm: its square in two parts, rownorm2[i] + rownorm2[m + i] (an earlier product's
+    // xn2_out for the same rows)
+    const float* rownorm2;
     // optional HOST arrays (n each): B row j is zero outside K columns [b_klo[j], b_khi[j]);
     // K-blocks outside a column tile's union are skipped (exact: only zero products dropped)
     const int* b_klo; const int* b_khi;

@@ -296,26 +296,32 @@ __global__ void __launch_bounds__(256) k_gemm(GemmArgs g) {
     gemm_tile<TA, TB, TC, BT>(g, (long long)blockIdx.y * kTM, blockIdx.x * kTN, blockIdx.z, As, Bs);
 }
 
-// The gated product (gate_xn2): persistent blocks walk the 64 x 64 tiles, n fastest, and compute
-// only those whose 64 rows hold a selected row; with no such row the launch is one pass over
-// the norms.
+// The gated product (gate_xn2): each block takes a run of consecutive 64 x 64 tiles, n fastest, and
+// computes only those whose 64 rows hold a selected row.  It looks at all its rows first (a run spans few
+// row blocks), so with no such row the launch is one round of loads and a barrier (12 us before, with a
+// barrier per tile: 16,384 x 922).
 template <int TA, int TB, int TC, bool BT>
-__global__ void __launch_bounds__(256) k_gemm_gated(GemmArgs g) {
+__global__ void __launch_bounds__(256) k_gemm_gated(GemmArgs g, long long per) {
     __shared__ float As[kTK][kTM + 4];
     __shared__ __align__(16) float Bs[kTK][kTN + 4];
     const int tiles_n = (g.n + kTN - 1) / kTN;
     const long long tiles = (g.m + kTM - 1) / kTM * tiles_n;
+    const long long t0 = (long long)blockIdx.x * per, t1 = t0 + per < tiles ? t0 + per : tiles;
+    if (t0 >= t1) return;
+    auto selected = [&](long long i) {
+        const float xn2 = g.gate_xn2[i] + g.gate_xn2[g.gate_ld + i];
+        return xn2 > 0.f && !(xn2 >= g.gate_lo && xn2 <= g.gate_hi);
+    };
+    const long long r0 = t0 / tiles_n * kTM, r1 = (t1 - 1) / tiles_n * kTM + kTM;
+    bool mine = false;
+    for (long long i = r0 + threadIdx.x; i < r1 && i < g.m; i += 256) mine |= selected(i);
+    if (!__syncthreads_or(mine)) return;
     long long last_m0 = -1;
     bool any = false;
-    for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
+    for (long long t = t0; t < t1; ++t) {
         const long long m0 = t / tiles_n * kTM;
         if (m0 != last_m0) {
-            bool mine = false;
-            if (threadIdx.x < kTM && m0 + threadIdx.x < g.m) {
-                const long long i = m0 + threadIdx.x;
-                const float xn2 = g.gate_xn2[i] + g.gate_xn2[g.gate_ld + i];
-                mine = xn2 > 0.f && !(xn2 >= g.gate_lo && xn2 <= g.gate_hi);
-            }
+            mine = threadIdx.x < kTM && m0 + threadIdx.x < g.m && selected(m0 + threadIdx.x);
             any = __syncthreads_or(mine) != 0;
             last_m0 = m0;
         }
@@ -656,8 +662,8 @@ cudaError_t launch_gemm_simt(const GemmArgs& g, cudaStream_t s) {
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         const long long tiles = (g.m + kTM - 1) / kTM * ((g.n + kTN - 1) / kTN);
-        const int grid = (int)std::min<long long>(tiles, 4LL * std::max(sms, 1));
-        k_gemm_gated<MAT_F32, MAT_F32, MAT_F32, true><<<grid, 256, 0, s>>>(g);
+        const long long grid = std::min<long long>(tiles, 4LL * std::max(sms, 1)), per = (tiles + grid - 1) / grid;
+        k_gemm_gated<MAT_F32, MAT_F32, MAT_F32, true><<<(unsigned)((tiles + per - 1) / per), 256, 0, s>>>(g, per);
         return cudaGetLastError();
     }
     dim3 grid((unsigned)((g.n + kTN - 1) / kTN), (unsigned)((g.m + kTM - 1) / kTM),

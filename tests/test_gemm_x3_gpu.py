@@ -2,11 +2,11 @@
 take it: large reconstructions and vectorizations whose rows are not 16-byte aligned, bf16 T, short
 rows, fp32 attention.  Element-wise against the 64-bit product:
 
-    |error| <= (20 + ceil(K / 256)) 2^-23 sum_k |a_k| |b_k|
+    |error| <= (12 + ceil(K / 128)) 2^-23 sum_k |a_k| |b_k|
 
-a bound from the kernel's arithmetic: at most 16 accumulation steps per 256 terms, each losing at
+a bound from the kernel's arithmetic: at most 8 accumulation steps per 128 terms, each losing at
 most 2^-23 of the sum of magnitudes; the small products' steps, 2^-8 of that and 6 times as many; the
-products left out, below 2^-23; one fp32 addition per 256 terms.
+products left out, below 2^-23; one fp32 addition per 128 terms.
 """
 import numpy as np
 import pytest
@@ -16,7 +16,7 @@ pytestmark = pytest.mark.gpu
 
 
 def bound(K, mag):
-    return (20 + -(-K // 256)) * 2.0 ** -23 * mag + 1e-30
+    return (12 + -(-K // 128)) * 2.0 ** -23 * mag + 1e-30
 
 
 def bipolar(rng, M, D):
