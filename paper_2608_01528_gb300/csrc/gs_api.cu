@@ -339,14 +339,43 @@ gs_status gs_project_similarity(const gs_basis* h, const float* X, long long N, 
         return !aligned ? GS_ERR_ALIGNMENT : GS_ERR_UNSUPPORTED;
     }
     if (r <= 32) {
-        return from_cuda(gs::launch_ps_warp(X, N, ldx, D, h->Q, r, h->R, h->ldr, M, h->cnorm, mode, scale,
-                                            Y, ldy, S, lds, argmax, maxval, s));
+        return from_cuda(gs::launch_ps_small(X, N, ldx, D, h->Q, r, h->R, h->ldr, M, h->cnorm, mode, scale,
+                                             Y, ldy, S, lds, argmax, maxval, s));
     }
+    const bool simt = flags == GS_PATH_SIMT;
     // generic chunked fp32 path: Y = X Q^T, S = Y R^T (+ cosine / scale), row finish
     const long long chunk = std::min(h->chunk_rows, kMaxGemmRows);
     for (long long c0 = 0; c0 < N; c0 += chunk) {
         const long long nc = std::min(chunk, N - c0);
         float* scr = h->scratch;
+        gs::GemmArgs a{};
+        a.A = X + c0 * ldx; a.a_type = gs::MAT_F32; a.lda = ldx;
+        a.B = h->Q; a.b_type = gs::MAT_F32; a.ldb = D; a.b_trans = true;
+        a.c_type = gs::MAT_F32;
+        a.m = nc; a.n = r; a.k = D; a.batch = 1; a.alpha = 1.f;
+        const bool wanted = S || argmax || maxval;
+        // narrow bases: the projection's K chunks (with the rows' squared norms for the cosine) go
+        // straight to the scoring kernel, which sums them, scores and picks in the same launch (1,024
+        // queries, D = 8192, r = M = 40, cosine: 83 us as norms, product, sum, product and row pass)
+        if (r <= gs::kMaxScoresR && !gs::gemm_fp32_on_tensor(a, simt, h->device)) {
+            const long long room = h->scratch_floats / (nc * (r + 1));
+            a.ksplit = (int)std::min<long long>(gemm_ksplit(nc, r, D, h->device), room);
+            a.kpart = scr;
+            a.xx_part = mode == GS_SCORE_COSINE ? scr + (long long)a.ksplit * nc * r : nullptr;
+            cudaError_t e = gs::launch_gemm_simt_parts(a, s, false);
+            if (e != cudaSuccess) return from_cuda(e);
+            gs::ScoreArgs q{};
+            q.part = a.kpart; q.xx = a.xx_part; q.ks = a.ksplit;
+            q.Yout = Y ? Y + c0 * ldy : nullptr; q.ldyo = ldy;
+            q.N = nc; q.r = r; q.R = h->R; q.ldr = h->ldr; q.M = M; q.cnorm = h->cnorm;
+            q.mode = mode; q.scale = scale;
+            q.S = S ? S + c0 * lds : nullptr; q.lds = lds;
+            q.argmax = argmax ? argmax + c0 : nullptr;
+            q.maxval = maxval ? maxval + c0 : nullptr;
+            e = gs::launch_scores(q, s);
+            if (e != cudaSuccess) return from_cuda(e);
+            continue;
+        }
         float* Ybuf = Y ? Y + c0 * ldy : scr;
         const long long ldyb = Y ? ldy : r;
         scr += Y ? 0 : nc * r;
@@ -357,11 +386,7 @@ gs_status gs_project_similarity(const gs_basis* h, const float* X, long long N, 
             cudaError_t e = gs::launch_rownorm(X + c0 * ldx, nc, ldx, D, xn, s);
             if (e != cudaSuccess) return from_cuda(e);
         }
-        gs::GemmArgs a{};
-        a.A = X + c0 * ldx; a.a_type = gs::MAT_F32; a.lda = ldx;
-        a.B = h->Q; a.b_type = gs::MAT_F32; a.ldb = D; a.b_trans = true;
-        a.C = Ybuf; a.c_type = gs::MAT_F32; a.ldc = ldyb;
-        a.m = nc; a.n = r; a.k = D; a.batch = 1; a.alpha = 1.f;
+        a.C = Ybuf; a.ldc = ldyb;
         // few output tiles (a small batch against a narrow basis): cut D into chunks so that
         // every SM gets work; the partial products go to the scratch after Y and the norms
         // (the score rows are written there only later) and are summed in a fixed order
@@ -371,9 +396,21 @@ gs_status gs_project_similarity(const gs_basis* h, const float* X, long long N, 
             a.ksplit = (int)std::min<long long>(gemm_ksplit(nc, r, D, h->device), room);
             a.kpart = a.ksplit > 1 ? scr : nullptr;
         }
-        cudaError_t e = gs::launch_gemm_fp32(a, flags == GS_PATH_SIMT, h->device, s);
+        cudaError_t e = gs::launch_gemm_fp32(a, simt, h->device, s);
         if (e != cudaSuccess) return from_cuda(e);
-        if (!S && !argmax && !maxval) continue;
+        if (!wanted) continue;
+        if (r <= gs::kMaxScoresR) {
+            gs::ScoreArgs q{};
+            q.Y = Ybuf; q.ldy = (int)ldyb; q.xnorm = xn;
+            q.N = nc; q.r = r; q.R = h->R; q.ldr = h->ldr; q.M = M; q.cnorm = h->cnorm;
+            q.mode = mode; q.scale = scale;
+            q.S = S ? S + c0 * lds : nullptr; q.lds = lds;
+            q.argmax = argmax ? argmax + c0 : nullptr;
+            q.maxval = maxval ? maxval + c0 : nullptr;
+            e = gs::launch_scores(q, s);
+            if (e != cudaSuccess) return from_cuda(e);
+            continue;
+        }
         float* Sbuf = S ? S + c0 * lds : scr;
         const long long ldsb = S ? lds : M;
         gs::GemmArgs b{};
@@ -382,7 +419,7 @@ gs_status gs_project_similarity(const gs_basis* h, const float* X, long long N, 
         b.C = Sbuf; b.c_type = gs::MAT_F32; b.ldc = ldsb;
         b.m = nc; b.n = M; b.k = r; b.batch = 1; b.alpha = scale;
         if (mode == GS_SCORE_COSINE) { b.rownorm = xn; b.colnorm = h->cnorm; }
-        e = gs::launch_gemm_fp32(b, flags == GS_PATH_SIMT, h->device, s);
+        e = gs::launch_gemm_fp32(b, simt, h->device, s);
         if (e != cudaSuccess) return from_cuda(e);
         if (argmax || maxval || mode == GS_SCORE_SOFTMAX) {
             e = gs::launch_row_finish(Sbuf, nc, M, (int)ldsb, mode == GS_SCORE_SOFTMAX,
@@ -482,9 +519,14 @@ gs_status gs_similarity_coeffs(const gs_basis* h, const float* Y, long long N, i
     const bool tc_ok = h->has_split && r >= 1 && (uintptr_t)Y % 16 == 0 && ldy % 4 == 0;
     const bool tensor = flags == GS_PATH_TENSOR || (flags == GS_PATH_AUTO && tc_ok && big_gemm(N, M, r));
     if (tensor && !tc_ok) return h->has_split && r >= 1 ? GS_ERR_ALIGNMENT : GS_ERR_UNSUPPORTED;
-    if (!tensor && r >= 1 && r <= gs::kMaxCoeffsWarpR)  // small r: one fused launch, no scratch
-        return from_cuda(gs::launch_coeffs_warp(Y, N, ldy, r, h->R, h->ldr, M, h->cnorm, mode, scale, S, lds, argmax,
-                                                maxval, s));
+    if (!tensor && r >= 1 && r <= gs::kMaxScoresR) {  // small r: one fused launch, no scratch
+        gs::ScoreArgs q{};
+        q.Y = Y; q.ldy = ldy;
+        q.N = N; q.r = r; q.R = h->R; q.ldr = h->ldr; q.M = M; q.cnorm = h->cnorm;
+        q.mode = mode; q.scale = scale;
+        q.S = S; q.lds = lds; q.argmax = argmax; q.maxval = maxval;
+        return from_cuda(gs::launch_scores(q, s));
+    }
     // scratch per row: ||y|| (cosine) and the score row when S is not an output
     const long long per_row = (mode == GS_SCORE_COSINE ? 1 : 0) + (S ? 0 : M);
     const long long chunk = std::min(per_row ? h->scratch_floats / per_row : N, kMaxGemmRows);
@@ -566,6 +608,19 @@ gs_status gs_prob_vectorize(const gs_basis* h, const float* P, long long N, int 
     return GS_OK;
 }
 
+// whether reconstruct_rows may and will take the fp16 tensor-core path
+static bool reconstruct_tc_ok(const gs_basis* h, const void* T, int t_dtype, int ldt) {
+    // one fp16 rounding of T and of Q: each output sums r rounding errors weighted by entries of Q of
+    // size ~1/sqrt(D), so the error's spread is ~2^-11 ||t|| / sqrt(D); from D = 1024 on its worst
+    // case over a large output stays well inside 1e-4 ||t||, shorter rows take the fp32 path
+    return h->has_split && h->r >= 1 && t_dtype == GS_F32 && h->D >= gs::kMinF16Depth && (uintptr_t)T % 16 == 0 &&
+           ldt % 4 == 0;
+}
+static bool reconstruct_on_tensor(const gs_basis* h, const void* T, int t_dtype, long long N, int ldt, unsigned flags) {
+    const bool tc_ok = reconstruct_tc_ok(h, T, t_dtype, ldt);
+    return tc_ok && (flags == GS_PATH_TENSOR || (flags == GS_PATH_AUTO && big_gemm(N, h->D, h->r)));
+}
+
 // Xhat = T B with the fp16 copy of T (tensor-core path) in `work` (work_floats floats).  B is the
 // basis (Qb = h->Q, ldqb = D, Qtb = h->Q16t) or, for the one-partner reconstruct + bind, the basis
 // rows bound with the partner (fp32 r x D rows, ld ldqb, and their transposed fp16 copy).
@@ -577,14 +632,10 @@ static gs_status reconstruct_rows(const gs_basis* h, const void* T, int t_dtype,
         ldqb = h->D;
         Qtb = h->Q16t;
     }
-    // one fp16 rounding of T and of Q: each output sums r rounding errors weighted by entries of Q of
-    // size ~1/sqrt(D), so the error's spread is ~2^-11 ||t|| / sqrt(D); from D = 1024 on its worst
-    // case over a large output stays well inside 1e-4 ||t||, shorter rows take the fp32 path
-    const bool deep = h->D >= gs::kMinF16Depth;
-    const bool tc_ok = h->has_split && h->r >= 1 && t_dtype == GS_F32 && deep && (uintptr_t)T % 16 == 0 &&
-                       ldt % 4 == 0;
-    if (flags == GS_PATH_TENSOR || (flags == GS_PATH_AUTO && tc_ok && big_gemm(N, h->D, h->r))) {
-        if (!tc_ok) return t_dtype != GS_F32 || !h->has_split || !deep ? GS_ERR_UNSUPPORTED : GS_ERR_ALIGNMENT;
+    const bool tc_ok = reconstruct_tc_ok(h, T, t_dtype, ldt);
+    if (flags == GS_PATH_TENSOR && !tc_ok)
+        return t_dtype != GS_F32 || !h->has_split || h->D < gs::kMinF16Depth ? GS_ERR_UNSUPPORTED : GS_ERR_ALIGNMENT;
+    if (reconstruct_on_tensor(h, T, t_dtype, N, ldt, flags)) {
         // Xhat = T Q: T rounded once to fp16 into the handle's scratch (every column tile of
         // Xhat re-reads it) after an exact power-of-two scale per row, the basis' dithered fp16
         // Q^T, fp32 accumulation, the row scales undone in the epilogue; rows in chunks that
@@ -693,7 +744,7 @@ static gs_status reconstruct_bind_one_partner(const gs_basis* h, const void* T, 
     float* work = h->scratch + qy_floats + qt_floats;
     gs_status st = bind_rows(h->Q, r, D, D, Y, 0, L, op, Qy, Dp, s);
     if (st != GS_OK) return st;
-    if (h->has_split) {  // the tensor-core reconstruction's operand (the fp32 path reads Qy)
+    if (reconstruct_on_tensor(h, T, t_dtype, N, ldt, flags)) {  // its operand (the fp32 path reads Qy)
         st = from_cuda(gs::launch_f16t_dither(Qy, r, D, Dp, Qyt, ld16, s));
         if (st != GS_OK) return st;
     }

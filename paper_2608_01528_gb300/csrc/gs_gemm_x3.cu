@@ -570,24 +570,27 @@ static cudaError_t launch_gemm_x3(const GemmArgs& g, int sms, int device, cudaSt
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_gemm_fp32(const GemmArgs& g, bool simt, int device, cudaStream_t s) {
+bool gemm_fp32_on_tensor(const GemmArgs& g, bool simt, int device) {
     const bool takes = !simt && g.b_type == MAT_F32 && (g.a_type == MAT_F32 || !g.b_trans) && !g.gate_xn2 && g.k >= 1 &&
                        g.k <= 32768 && g.lda <= 1 << 22 &&
                        (g.b_trans ? g.ldb <= 1 << 22 : (double)g.ldb * g.k < 1e9) && g.m > 0 && g.n > 0 && g.batch > 0;
     // times of both kernels, fitted to measured ones: a wave of tiles takes ~0.9 us per K-block and ~6 us
-    // around it (m = 1000, n = 5000, k = 100: 31 us against 42 us on the CUDA cores; 512 x 3001 x 257:
-    // 21 / 35; 3000 x 1000 x 300: 31 / 65; 20,000 x 777 x 131: 94 / 146; 34,304 x 448 x 62: 70 / 67, not
-    // taken); the CUDA-core GEMM runs at 28 to 37 TFLOP/s
+    // around it (512 x 3001 x 257: 21 us against 35 on the CUDA cores; 3000 x 1000 x 300: 31 / 65; 20,000 x
+    // 777 x 131: 94 / 146; 34,304 x 448 x 62: 70 / 67, not taken); the CUDA-core GEMM runs at 28 to 37
+    // TFLOP/s
     const double simt_us = 2e-6 * g.m * g.n * g.k * g.batch / 30.0;
-    if (takes && simt_us > 15.0 && tc_available(device)) {
-        int sms = 0;
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
-        sms = std::max(sms, 1);
-        const double tiles = (double)((g.m + kBM - 1) / kBM) * ((g.n + kBN - 1) / kBN) * g.batch;
-        const double x3_us = 8.0 + std::ceil(tiles / sms) * (0.9 * ((g.k + kBK - 1) / kBK) + 6.0);
-        if (x3_us < simt_us) return launch_gemm_x3(g, sms, device, s);
-    }
-    return launch_gemm_simt(g, s);
+    if (!takes || simt_us <= 15.0 || !tc_available(device)) return false;
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+    const double tiles = (double)((g.m + kBM - 1) / kBM) * ((g.n + kBN - 1) / kBN) * g.batch;
+    return 8.0 + std::ceil(tiles / std::max(sms, 1)) * (0.9 * ((g.k + kBK - 1) / kBK) + 6.0) < simt_us;
+}
+
+cudaError_t launch_gemm_fp32(const GemmArgs& g, bool simt, int device, cudaStream_t s) {
+    if (!gemm_fp32_on_tensor(g, simt, device)) return launch_gemm_simt(g, s);
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+    return launch_gemm_x3(g, std::max(sms, 1), device, s);
 }
 
 }  // namespace gs

@@ -100,17 +100,29 @@ gs_status import_basis(const float* Q, int ldq, const float* R, int ldr_in, cons
 // ----------------------------------------------------------------- SIMT kernels (gs_simt.cu)
 enum { MAT_F32 = 0, MAT_BF16 = 1 };
 
-// fused small-r project + similarity, one warp per query (r <= 32)
-cudaError_t launch_ps_warp(const float* X, long long N, int ldx, int D, const float* Q, int r,
-                           const float* R, int ldr, int M, const float* cnorm, int mode, float scale,
-                           float* Y, int ldy, float* S, int lds, int* argmax, float* maxval,
-                           cudaStream_t s);
+// fused small-r project + similarity, four queries per block (r <= 32)
+cudaError_t launch_ps_small(const float* X, long long N, int ldx, int D, const float* Q, int r,
+                            const float* R, int ldr, int M, const float* cnorm, int mode, float scale,
+                            float* Y, int ldy, float* S, int lds, int* argmax, float* maxval,
+                            cudaStream_t s);
 
-// similarity of Gram-loc queries Y (N x r, r <= 64), one warp per query; every mode, S optional
-constexpr int kMaxCoeffsWarpR = 64;
-cudaError_t launch_coeffs_warp(const float* Y, long long N, int ldy, int r, const float* R, int ldr, int M,
-                               const float* cnorm, int mode, float scale, float* S, int lds, int* argmax,
-                               float* maxval, cudaStream_t s);
+// scores, argmax and max of Gram-loc rows, 1 <= r <= kMaxScoresR, one warp per row; every mode, outputs
+// optional.  The rows are Y, or the sums over z < ks (in order) of part[z] (ks x N x r, written to Yout
+// when given; xx: ||x||^2 in ks parts, for the cosine).  With Y, xnorm (optional) holds ||x_n||;
+// otherwise ||y_n|| stands for it (Eq. 3).
+constexpr int kMaxScoresR = 64;
+struct ScoreArgs {
+    const float* Y; int ldy;
+    const float* part; const float* xx; int ks;
+    const float* xnorm;
+    float* Yout; int ldyo;
+    long long N; int r;
+    const float* R; int ldr; int M;
+    const float* cnorm;
+    int mode; float scale;
+    float* S; int lds; int* argmax; float* maxval;
+};
+cudaError_t launch_scores(const ScoreArgs& a, cudaStream_t s);
 
 // C = alpha * A * op(B), batched over `batch` with element strides.
 //   A: m x k (lda), B: trans ? n x k : k x n (ldb); types MAT_F32 / MAT_BF16.
@@ -133,11 +145,18 @@ struct GemmArgs {
                           // (ksplit x m x n floats, caller's workspace) and a second kernel
                           // sums the chunks in a fixed order into C (deterministic)
     float* kpart;
+    // optional (batch 1): every K chunk's part of A's rows' squared norms (ksplit x m floats)
+    float* xx_part;
+    int a_vec, b_vec;     // set by the launch: rows of four-element groups on 16-byte boundaries
 };
 cudaError_t launch_gemm_simt(const GemmArgs& g, cudaStream_t s);
+// sum = false: the partial products stay in kpart (also for one chunk) and C is not written
+cudaError_t launch_gemm_simt_parts(const GemmArgs& g, cudaStream_t s, bool sum);
 // the same product at fp32 accuracy: on the tensor cores when it is large (gs_gemm_x3.cu: operands
 // split into three bf16 parts), else (and always with simt) launch_gemm_simt
 cudaError_t launch_gemm_fp32(const GemmArgs& g, bool simt, int device, cudaStream_t s);
+// whether launch_gemm_fp32 takes the tensor cores
+bool gemm_fp32_on_tensor(const GemmArgs& g, bool simt, int device);
 
 // per-row ||x||
 cudaError_t launch_rownorm(const float* X, long long N, int ldx, int D, float* out, cudaStream_t s);

@@ -5,9 +5,10 @@
 // shape can take (GS_PATH_SIMT).  The large-batch hot path is on tcgen05 in
 // gs_tc.cu.
 //
-//  k_ps_warp      fused project + similarity, one warp per query, r <= 32
+//  k_ps_small     fused project + similarity, four queries per block, r <= 32
 //                 (Sec. 3.1 t = U^T x; Sec. 2.2 similarity; Eq. 2-3)
-//  k_coeffs_warp  similarity of Gram-loc queries, one warp per query, r <= 64 (Sec. 3.2, Eq. 2)
+//  k_scores       similarity of Gram-loc queries (or of K-split partial sums of them), one warp per
+//                 query, r <= 64 (Sec. 3.2, Eq. 2)
 //  k_gemm         tiled fp32 GEMM with scale / cosine / bf16 epilogues; used for
 //                 Y = X Q^T, S = Y R^T, V = P R (Sec. 2.2 / 3.3), Xhat = T Q
 //                 (Sec. 3.1 / 3.3) and batched attention logits (Sec. 2.2)
@@ -49,117 +50,274 @@ __device__ __forceinline__ void warp_argmax(float& v, int& i) {
     }
 }
 
-// ----------------------------------------------------------------- fused small-r kernel
-constexpr int kWarpR = 32;
+// ----------------------------------------------------------------- scores of Gram-loc rows, r <= 64
+constexpr int kCoefR = 64;
+constexpr int kCoefWarps = 8;
+constexpr int kRSmemFloats = 12 * 1024;  // codeword rows staged at a time: 48 KB
 
-__global__ void __launch_bounds__(256) k_ps_warp(const float* __restrict__ X, long long N, int ldx,
-                                                  int D, const float* __restrict__ Q, int r,
-                                                  const float* __restrict__ R, int ldr, int M,
-                                                  const float* __restrict__ cnorm, int mode,
-                                                  float scale, float* __restrict__ Y, int ldy,
-                                                  float* __restrict__ S, int lds,
-                                                  int* __restrict__ argmax,
-                                                  float* __restrict__ maxval) {
-    const int lane = threadIdx.x & 31;
-    const long long n = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (n >= N) return;
-    const float* x = X + (size_t)n * ldx;
-    float y[kWarpR];
+struct ScoreParams {
+    const float* Y;       // N x r (ld ldy), or null: y_j = sum over z < ks (in order) of part[z][n][j]
+    int ldy;
+    const float* part;
+    const float* xx;      // with part: ||x||^2 in ks parts (ks x N), or null
+    int ks;
+    const float* xnorm;   // with Y (optional): ||x_n||; otherwise ||y_n|| stands for it (Eq. 3)
+    float* Yout;          // with part (optional): the Gram-loc rows
+    int ldyo;
+    long long N;
+    int r;
+    const float* R;
+    int ldr, M;
+    const float* cnorm;
+    int mode;
+    float scale;
+    float* S;
+    int lds;
+    int* argmax;
+    float* maxval;
+    int chunk, pitch;     // codewords staged at a time, floats between their rows
+};
+
+// One warp per Gram-loc row, lane l scoring codewords l, l + 32, ...  R is staged in shared memory once
+// per block (pitch: whole float4s, an odd number of them, so that a float4 from 32 consecutive rows
+// falls in disjoint banks), the warp's row beside it: per codeword r / 4 conflict-free 16-byte reads and
+// as many broadcasts.  Reading R's rows from global memory, a row per lane, took r loads of 32 lines
+// each per codeword (1,024 rows x 40 codewords, r = 40: 8.1 us, now 5; r = 30, M = 22, 10,844 rows: 22.6 us,
+// now 8).  A codebook past 48 KB goes through in chunks; softmax rows are then scored twice.
+__global__ void __launch_bounds__(kCoefWarps * 32) k_scores(const ScoreParams p) {
+    extern __shared__ float4 coef_sm[];
+    float* Rs = reinterpret_cast<float*>(coef_sm);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float* ys = Rs + (size_t)p.chunk * p.pitch + warp * kCoefR;
+    const int r4 = (p.r + 3) / 4;
+    const bool whole = p.chunk >= p.M;  // one chunk: staged once, kept
+    auto stage = [&](int i0) {
+        const int n = min(p.chunk, p.M - i0);
+        for (int e = threadIdx.x; e < n * 4 * r4; e += kCoefWarps * 32) {
+            const int i = e / (4 * r4), j = e - i * 4 * r4;
+            Rs[i * p.pitch + j] = j < p.r ? __ldg(p.R + (size_t)(i0 + i) * p.ldr + j) : 0.f;
+        }
+    };
+    if (whole) {
+        stage(0);
+        __syncthreads();
+    }
+    const long long step = (long long)gridDim.x * kCoefWarps;
+    const long long rounds = (p.N + step - 1) / step;
+    for (long long it = 0; it < rounds; ++it) {
+        const long long n = it * step + (long long)blockIdx.x * kCoefWarps + warp;
+        const bool in = n < p.N;
+        float ynorm = 0.f;
+        __syncwarp();
+        if (in) {
+            float yy = 0.f;
+            for (int j = lane; j < 4 * r4; j += 32) {
+                float y = 0.f;
+                if (j < p.r) {
+                    if (p.part) {
+                        for (int z = 0; z < p.ks; ++z) y += p.part[((size_t)z * p.N + n) * p.r + j];
+                        if (p.Yout) p.Yout[(size_t)n * p.ldyo + j] = y;
+                    } else {
+                        y = __ldg(p.Y + (size_t)n * p.ldy + j);
+                    }
+                }
+                ys[j] = y;
+                yy = fmaf(y, y, yy);
+            }
+            if (p.mode == GS_SCORE_COSINE) {
+                if (p.part) {
+                    float xx = 0.f;
+                    for (int z = 0; z < p.ks; ++z) xx += p.xx[(size_t)z * p.N + n];
+                    ynorm = sqrtf(xx);
+                } else {
+                    ynorm = p.xnorm ? p.xnorm[n] : sqrtf(warp_sum(yy));
+                }
+            }
+        }
+        __syncwarp();
+        const bool wanted = p.S || p.argmax || p.maxval;
+        float bv = -FLT_MAX, m = -FLT_MAX, z = 0.f;
+        int bi = 0x7fffffff;
+        const bool soft = p.mode == GS_SCORE_SOFTMAX;
+        const int sweeps = soft && p.S ? 2 : 1;
+        float inv = 0.f;
+        for (int sweep = 0; sweep < sweeps && wanted; ++sweep) {
+            for (int i0 = 0; i0 < p.M; i0 += p.chunk) {
+                if (!whole) {
+                    __syncthreads();
+                    stage(i0);
+                    __syncthreads();
+                }
+                if (!in) continue;
+                const int i1 = min(p.M, i0 + p.chunk);
+                for (int i = i0 + lane; i < i1; i += 32) {
+                    const float4* Ri = reinterpret_cast<const float4*>(Rs + (i - i0) * p.pitch);
+                    const float4* yv = reinterpret_cast<const float4*>(ys);
+                    float g = 0.f;
+#pragma unroll 4
+                    for (int q = 0; q < r4; ++q) {
+                        const float4 a = yv[q], b = Ri[q];
+                        g = fmaf(a.x, b.x, g);
+                        g = fmaf(a.y, b.y, g);
+                        g = fmaf(a.z, b.z, g);
+                        g = fmaf(a.w, b.w, g);
+                    }
+                    g *= p.scale;
+                    if (p.mode == GS_SCORE_COSINE) {
+                        const float den = ynorm * p.cnorm[i];
+                        g = den > 0.f ? g / den : 0.f;
+                    }
+                    if (sweep == 1) {
+                        p.S[(size_t)n * p.lds + i] = __expf(g - m) * inv;
+                        continue;
+                    }
+                    if (g > bv) {
+                        bv = g;
+                        bi = i;
+                    }
+                    if (soft) {
+                        const float nm = fmaxf(m, g);
+                        z = z * __expf(m - nm) + __expf(g - nm);
+                        m = nm;
+                    } else if (p.S) {
+                        p.S[(size_t)n * p.lds + i] = g;
+                    }
+                }
+            }
+            if (sweep == 0 && soft && in) {  // the lanes' maxima and sums, merged
+                const float mm = warp_max(m);
+                inv = 1.f / warp_sum(z * __expf(m - mm));
+                m = mm;
+            }
+        }
+        if (!in || !wanted) continue;
+        warp_argmax(bv, bi);
+        if (bi == 0x7fffffff) bi = 0;
+        if (lane == 0) {
+            if (p.argmax) p.argmax[n] = bi;
+            if (p.maxval) p.maxval[n] = soft ? inv : bv;  // the largest score's share is 1 / sum
+        }
+    }
+}
+
+// ----------------------------------------------------------------- fused project + score, r <= 32
+// A block takes kSmallQ queries; its warps split the D dimension (chunks of 128, dealt in turn), a lane
+// four dimensions of a chunk, and keeps all kSmallQ x r partial products in registers: per chunk a lane
+// reads kSmallQ + r vectors for 4 kSmallQ r FMAs.  The lanes' sums fold in a butterfly that leaves
+// entry l in lane l, the warps' meet in shared memory; warp t then scores query t.  Bound by the
+// latency of the loads on the usual few hundred queries.  (One warp per query read all of Q per
+// query, 4 bytes a lane: 2,048 queries of D = 1024, r = 30: 96 us, now 9.)
+constexpr int kSmallR = 32;
+constexpr int kSmallQ = 4;
+
+// entry idx of v[RM] summed over the warp: lane l returns the sum of entry l % RM
+template <int RM>
+__device__ __forceinline__ float fold_entries(float (&v)[RM], int lane) {
 #pragma unroll
-    for (int j = 0; j < kWarpR; ++j) y[j] = 0.f;
-    float xx = 0.f;
-    for (int d = lane; d < D; d += 32) {
-        const float xv = x[d];
-        xx = fmaf(xv, xv, xx);
+    for (int w = RM / 2; w >= 1; w >>= 1) {
+        const bool up = (lane & w) != 0;
 #pragma unroll
-        for (int j = 0; j < kWarpR; ++j)
-            if (j < r) y[j] = fmaf(xv, __ldg(Q + (size_t)j * D + d), y[j]);
+        for (int j = 0; j < w; ++j) {
+            const float send = up ? v[j] : v[j + w], keep = up ? v[j + w] : v[j];
+            v[j] = keep + __shfl_xor_sync(0xffffffffu, send, w);
+        }
+    }
+    float x = v[0];
+#pragma unroll
+    for (int w = RM; w < 32; w <<= 1) x += __shfl_xor_sync(0xffffffffu, x, w);
+    return x;
+}
+
+template <int RM, bool VEC>
+__global__ void __launch_bounds__(256) k_ps_small(const float* __restrict__ X, long long N, int ldx, int D,
+                                                  const float* __restrict__ Q, int r, const float* __restrict__ R,
+                                                  int ldr, int M, const float* __restrict__ cnorm, int mode,
+                                                  float scale, float* __restrict__ Y, int ldy, float* __restrict__ S,
+                                                  int lds, int* __restrict__ argmax, float* __restrict__ maxval) {
+    __shared__ float red[8][kSmallQ][kSmallR + 1];
+    __shared__ float ysm[kSmallQ][kSmallR];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    const long long n0 = (long long)blockIdx.x * kSmallQ;
+    const float* x[kSmallQ];
+#pragma unroll
+    for (int t = 0; t < kSmallQ; ++t) x[t] = X + (size_t)(n0 + t < N ? n0 + t : N - 1) * ldx;
+    float acc[kSmallQ][RM], xx[kSmallQ];
+#pragma unroll
+    for (int t = 0; t < kSmallQ; ++t) {
+        xx[t] = 0.f;
+#pragma unroll
+        for (int j = 0; j < RM; ++j) acc[t][j] = 0.f;
+    }
+    for (int c = warp; c * 128 < D; c += nw) {
+        if (VEC) {  // D % 4 == 0, rows 16-byte aligned: a lane four consecutive dimensions
+            const int d = c * 128 + 4 * lane;
+            if (d >= D) continue;
+            float4 xv[kSmallQ];
+#pragma unroll
+            for (int t = 0; t < kSmallQ; ++t) {
+                xv[t] = __ldg(reinterpret_cast<const float4*>(x[t] + d));
+                xx[t] = fmaf(xv[t].x, xv[t].x, fmaf(xv[t].y, xv[t].y, fmaf(xv[t].z, xv[t].z, fmaf(xv[t].w, xv[t].w, xx[t]))));
+            }
+#pragma unroll
+            for (int j = 0; j < RM; ++j) {
+                if (j >= r) break;
+                const float4 q = __ldg(reinterpret_cast<const float4*>(Q + (size_t)j * D + d));
+#pragma unroll
+                for (int t = 0; t < kSmallQ; ++t)
+                    acc[t][j] = fmaf(xv[t].x, q.x, fmaf(xv[t].y, q.y, fmaf(xv[t].z, q.z, fmaf(xv[t].w, q.w, acc[t][j]))));
+            }
+        } else {
+            for (int u = 0; u < 4; ++u) {
+                const int d = c * 128 + 32 * u + lane;
+                if (d >= D) break;
+                float xv[kSmallQ];
+#pragma unroll
+                for (int t = 0; t < kSmallQ; ++t) {
+                    xv[t] = __ldg(x[t] + d);
+                    xx[t] = fmaf(xv[t], xv[t], xx[t]);
+                }
+#pragma unroll
+                for (int j = 0; j < RM; ++j) {
+                    if (j >= r) break;
+                    const float q = __ldg(Q + (size_t)j * D + d);
+#pragma unroll
+                    for (int t = 0; t < kSmallQ; ++t) acc[t][j] = fmaf(xv[t], q, acc[t][j]);
+                }
+            }
+        }
     }
 #pragma unroll
-    for (int j = 0; j < kWarpR; ++j)
-        if (j < r) y[j] = warp_sum(y[j]);
-    xx = warp_sum(xx);
-    if (Y) {
-        float mine = 0.f;
-#pragma unroll
-        for (int j = 0; j < kWarpR; ++j)
-            if (j == lane) mine = y[j];
-        if (lane < r) Y[(size_t)n * ldy + lane] = mine;
+    for (int t = 0; t < kSmallQ; ++t) {
+        const float y = fold_entries<RM>(acc[t], lane);
+        const float s = warp_sum(xx[t]);
+        if (lane < RM) red[warp][t][lane] = y;
+        if (lane == 0) red[warp][t][kSmallR] = s;
     }
-    const float xnorm = sqrtf(xx);
+    __syncthreads();
+    const long long n = n0 + warp;
+    if (warp >= kSmallQ || n >= N) return;
+    float yl = 0.f, x2 = 0.f;
+    for (int w = 0; w < nw; ++w) {
+        if (lane < r) yl += red[w][warp][lane];
+        x2 += red[w][warp][kSmallR];
+    }
+    if (Y && lane < r) Y[(size_t)n * ldy + lane] = yl;
+    ysm[warp][lane] = yl;
+    __syncwarp();
+    float y[RM];
+#pragma unroll
+    for (int j = 0; j < RM; ++j) y[j] = ysm[warp][j];
+    const float xnorm = sqrtf(x2);
     // scores: lane handles codewords i = lane, lane + 32, ...
     auto score = [&](int i) {
         const float* Ri = R + (size_t)i * ldr;
         float g = 0.f;
 #pragma unroll
-        for (int j = 0; j < kWarpR; ++j)
+        for (int j = 0; j < RM; ++j)
             if (j < r) g = fmaf(y[j], __ldg(Ri + j), g);
         g *= scale;
         if (mode == GS_SCORE_COSINE) {
             const float den = xnorm * cnorm[i];
-            g = den > 0.f ? g / den : 0.f;
-        }
-        return g;
-    };
-    float bv = -FLT_MAX;
-    int bi = 0x7fffffff;
-    for (int i = lane; i < M; i += 32) {
-        const float g = score(i);
-        if (g > bv) {
-            bv = g;
-            bi = i;
-        }
-        if (S && mode != GS_SCORE_SOFTMAX) S[(size_t)n * lds + i] = g;
-    }
-    warp_argmax(bv, bi);
-    if (bi == 0x7fffffff) bi = 0;
-    float outmax = bv;
-    if (mode == GS_SCORE_SOFTMAX) {
-        float z = 0.f;
-        for (int i = lane; i < M; i += 32) z += __expf(score(i) - bv);
-        z = warp_sum(z);
-        const float inv = 1.f / z;
-        if (S)
-            for (int i = lane; i < M; i += 32) S[(size_t)n * lds + i] = __expf(score(i) - bv) * inv;
-        outmax = inv;
-    }
-    if (lane == 0) {
-        if (argmax) argmax[n] = M > 0 ? bi : 0;
-        if (maxval) maxval[n] = M > 0 ? outmax : 0.f;
-    }
-}
-
-// Scores of queries given by their Gram-loc rows y (r <= 64): every lane holds the whole row
-// (broadcast loads), lane l scores codewords l, l + 32, ...; ||y|| stands for ||x|| in the
-// cosine mode (Eq. 3: equal for x in span(C)).  One launch for a small-batch lookup.
-constexpr int kCoefR = 64;
-
-__global__ void __launch_bounds__(256) k_coeffs_warp(const float* __restrict__ Yg, long long N, int ldy, int r,
-                                                      const float* __restrict__ R, int ldr, int M,
-                                                      const float* __restrict__ cnorm, int mode, float scale,
-                                                      float* __restrict__ S, int lds, int* __restrict__ argmax,
-                                                      float* __restrict__ maxval) {
-    const int lane = threadIdx.x & 31;
-    const long long n = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (n >= N) return;
-    const float* yr = Yg + (size_t)n * ldy;
-    float y[kCoefR];
-    float yy = 0.f;
-#pragma unroll
-    for (int j = 0; j < kCoefR; ++j) {
-        y[j] = j < r ? __ldg(yr + j) : 0.f;
-        yy = fmaf(y[j], y[j], yy);
-    }
-    const float ynorm = sqrtf(yy);
-    auto score = [&](int i) {
-        const float* Ri = R + (size_t)i * ldr;
-        float g = 0.f;
-#pragma unroll
-        for (int j = 0; j < kCoefR; ++j)
-            if (j < r) g = fmaf(y[j], __ldg(Ri + j), g);
-        g *= scale;
-        if (mode == GS_SCORE_COSINE) {
-            const float den = ynorm * cnorm[i];
             g = den > 0.f ? g / den : 0.f;
         }
         return g;
@@ -201,11 +359,25 @@ __device__ __forceinline__ float ld_elem(const void* p, long long i) {
     return __bfloat162float(((const __nv_bfloat16*)p)[i]);
 }
 
+// Four consecutive elements i .. i + 3 of a row, those at or past `left` zero; vec: one 16-byte load
+template <int T>
+__device__ __forceinline__ void ld4(const void* p, long long i, int left, bool vec, float (&v)[4]) {
+    if (T == MAT_F32 && vec && left >= 4) {
+        const float4 x = __ldg(reinterpret_cast<const float4*>((const float*)p + i));
+        v[0] = x.x, v[1] = x.y, v[2] = x.z, v[3] = x.w;
+        return;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] = u < left ? ld_elem<T>(p, i + u) : 0.f;
+}
+
 // One 64 x 64 output tile (rows m0.., columns n0..) of batch b, or of K chunk kz with ksplit;
-// called by every thread of the block.
+// called by every thread of the block.  A thread loads four consecutive elements of each operand per
+// K step (one 16-byte load where rows are aligned), the next step's while the current one is multiplied
+// (two shared buffers, one barrier a step): 1,024 x 40 over K = 8192 in 16 chunks went from 52 to 24 us.
 template <int TA, int TB, int TC, bool BT>
 __device__ __forceinline__ void gemm_tile(const GemmArgs& g, long long m0, int n0, int kz,
-                                          float (&As)[kTK][kTM + 4], float (&Bs)[kTK][kTN + 4]) {
+                                          float (&As)[2][kTK][kTM + 4], float (&Bs)[2][kTK][kTN + 4]) {
     const int tid = threadIdx.x;
     const int tx = tid % 16, ty = tid / 16;
     const bool split = g.ksplit > 1;
@@ -232,58 +404,76 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs& g, long long m0, int n
         kbeg = kz * chunk;
         kend = min(kend, kbeg + chunk);
     }
-    float acc[4][4] = {};
-    for (int k0 = kbeg; k0 < kend; k0 += kTK) {
+    // A: row lr, k lk .. lk + 3 of the step; B the same (K-major), or k br, columns bc .. bc + 3
+    const int lr = tid / 4, lk = tid % 4 * 4, br = tid / 16, bc = tid % 16 * 4;
+    const long long gm = m0 + lr;
+    const long long arow = (gm < g.m ? gm : g.m - 1) * g.lda;
+    const bool a_in = gm < g.m, b_in = n0 + lr < g.n;
+    const long long brow = BT ? (long long)(b_in ? n0 + lr : g.n - 1) * g.ldb : 0;
+    float av[4], bv[4], xx = 0.f;
+    auto load = [&](int k0) {
+        ld4<TA>(Ab, arow + k0 + lk, a_in ? kend - (k0 + lk) : 0, g.a_vec, av);
+        if (BT)
+            ld4<TB>(Bb, brow + k0 + lk, b_in ? kend - (k0 + lk) : 0, g.b_vec, bv);
+        else
+            ld4<TB>(Bb, (long long)(k0 + br) * g.ldb + n0 + bc, k0 + br < kend ? g.n - (n0 + bc) : 0, g.b_vec, bv);
+    };
+    auto store = [&](int buf) {
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const int e = tid + 256 * t;
-            const int row = e / kTK, kk = e % kTK;
-            const long long gm = m0 + row;
-            const int gk = k0 + kk;
-            As[kk][row] = (gm < g.m && gk < kend) ? ld_elem<TA>(Ab, gm * g.lda + gk) : 0.f;
-            if (BT) {
-                const int gn = n0 + row;
-                Bs[kk][row] = (gn < g.n && gk < kend) ? ld_elem<TB>(Bb, (long long)gn * g.ldb + gk) : 0.f;
-            } else {
-                const int kk2 = e / kTN, col = e % kTN;
-                const int gk2 = k0 + kk2, gn = n0 + col;
-                Bs[kk2][col] = (gn < g.n && gk2 < kend) ? ld_elem<TB>(Bb, (long long)gk2 * g.ldb + gn) : 0.f;
-            }
+        for (int u = 0; u < 4; ++u) {
+            As[buf][lk + u][lr] = av[u];
+            if (BT) Bs[buf][lk + u][lr] = bv[u];
+            xx = fmaf(av[u], av[u], xx);
         }
-        __syncthreads();
+        if (!BT) *reinterpret_cast<float4*>(&Bs[buf][br][bc]) = make_float4(bv[0], bv[1], bv[2], bv[3]);
+    };
+    float acc[4][4] = {};
+    if (kbeg < kend) {
+        load(kbeg);
+        store(0);
+    }
+    __syncthreads();
+    int buf = 0;
+    for (int k0 = kbeg; k0 < kend; k0 += kTK, buf ^= 1) {
+        const bool more = k0 + kTK < kend;
+        if (more) load(k0 + kTK);
 #pragma unroll
         for (int kk = 0; kk < kTK; ++kk) {
-            float a[4], bb[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
-            const float4 bv = *reinterpret_cast<const float4*>(&Bs[kk][tx * 4]);
-            bb[0] = bv.x; bb[1] = bv.y; bb[2] = bv.z; bb[3] = bv.w;
+            const float4 a4 = *reinterpret_cast<const float4*>(&As[buf][kk][ty * 4]);
+            const float4 b4 = *reinterpret_cast<const float4*>(&Bs[buf][kk][tx * 4]);
+            const float a[4] = {a4.x, a4.y, a4.z, a4.w}, bb[4] = {b4.x, b4.y, b4.z, b4.w};
 #pragma unroll
             for (int i = 0; i < 4; ++i)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], bb[j], acc[i][j]);
         }
+        if (more) store(buf ^ 1);
         __syncthreads();
+    }
+    if (g.xx_part && n0 == 0) {  // this chunk's part of each row's squared norm
+        xx += __shfl_xor_sync(0xffffffffu, xx, 1);
+        xx += __shfl_xor_sync(0xffffffffu, xx, 2);
+        if (lk == 0 && a_in) g.xx_part[(size_t)kz * g.m + gm] = xx;
     }
     char* Cb = (char*)g.C + (size_t)b * g.c_bstride * (TC == MAT_F32 ? 4 : 2);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        const long long gm = m0 + ty * 4 + i;
-        if (gm >= g.m) continue;
+        const long long gi = m0 + ty * 4 + i;
+        if (gi >= g.m) continue;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int gn = n0 + tx * 4 + j;
             if (gn >= g.n) continue;
             float v = g.alpha * acc[i][j];
             if (g.rownorm) {
-                const float den = g.rownorm[gm] * g.colnorm[gn];
+                const float den = g.rownorm[gi] * g.colnorm[gn];
                 v = den > 0.f ? v / den : 0.f;
             }
             if (TC == MAT_F32) {
-                if (split) g.kpart[((size_t)kz * g.m + gm) * g.n + gn] = v;
-                else ((float*)Cb)[gm * g.ldc + gn] = v;
+                if (g.kpart) g.kpart[((size_t)kz * g.m + gi) * g.n + gn] = v;
+                else ((float*)Cb)[gi * g.ldc + gn] = v;
             } else {
-                ((__nv_bfloat16*)Cb)[gm * g.ldc + gn] = __float2bfloat16_rn(v);
+                ((__nv_bfloat16*)Cb)[gi * g.ldc + gn] = __float2bfloat16_rn(v);
             }
         }
     }
@@ -291,8 +481,8 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs& g, long long m0, int n
 
 template <int TA, int TB, int TC, bool BT>
 __global__ void __launch_bounds__(256) k_gemm(GemmArgs g) {
-    __shared__ float As[kTK][kTM + 4];
-    __shared__ __align__(16) float Bs[kTK][kTN + 4];
+    __shared__ __align__(16) float As[2][kTK][kTM + 4];
+    __shared__ __align__(16) float Bs[2][kTK][kTN + 4];
     gemm_tile<TA, TB, TC, BT>(g, (long long)blockIdx.y * kTM, blockIdx.x * kTN, blockIdx.z, As, Bs);
 }
 
@@ -302,8 +492,8 @@ __global__ void __launch_bounds__(256) k_gemm(GemmArgs g) {
 // barrier per tile: 16,384 x 922).
 template <int TA, int TB, int TC, bool BT>
 __global__ void __launch_bounds__(256) k_gemm_gated(GemmArgs g, long long per) {
-    __shared__ float As[kTK][kTM + 4];
-    __shared__ __align__(16) float Bs[kTK][kTN + 4];
+    __shared__ __align__(16) float As[2][kTK][kTM + 4];
+    __shared__ __align__(16) float Bs[2][kTK][kTN + 4];
     const int tiles_n = (g.n + kTN - 1) / kTN;
     const long long tiles = (g.m + kTM - 1) / kTM * tiles_n;
     const long long t0 = (long long)blockIdx.x * per, t1 = t0 + per < tiles ? t0 + per : tiles;
@@ -632,27 +822,56 @@ inline unsigned rows_grid(long long n) { return (unsigned)((n + 7) / 8); }
 
 }  // namespace
 
-cudaError_t launch_ps_warp(const float* X, long long N, int ldx, int D, const float* Q, int r,
-                           const float* R, int ldr, int M, const float* cnorm, int mode, float scale,
-                           float* Y, int ldy, float* S, int lds, int* argmax, float* maxval,
-                           cudaStream_t s) {
-    k_ps_warp<<<rows_grid(N), 256, 0, s>>>(X, N, ldx, D, Q, r, R, ldr, M, cnorm, mode, scale, Y, ldy,
-                                           S, lds, argmax, maxval);
+cudaError_t launch_ps_small(const float* X, long long N, int ldx, int D, const float* Q, int r,
+                            const float* R, int ldr, int M, const float* cnorm, int mode, float scale,
+                            float* Y, int ldy, float* S, int lds, int* argmax, float* maxval,
+                            cudaStream_t s) {
+    const bool vec = (uintptr_t)X % 16 == 0 && ldx % 4 == 0 && D % 4 == 0 && (uintptr_t)Q % 16 == 0;
+    const long long blocks = (N + kSmallQ - 1) / kSmallQ;
+    // eight warps share D while every block has an SM of its own (a block holds ~170 registers a
+    // thread), four once blocks queue
+    const int threads = blocks <= 152 ? 256 : 128;
+    auto kern = r <= 8 ? (vec ? k_ps_small<8, true> : k_ps_small<8, false>)
+                : r <= 16 ? (vec ? k_ps_small<16, true> : k_ps_small<16, false>)
+                          : (vec ? k_ps_small<32, true> : k_ps_small<32, false>);
+    kern<<<(unsigned)blocks, threads, 0, s>>>(X, N, ldx, D, Q, r, R, ldr, M, cnorm, mode, scale, Y, ldy, S, lds,
+                                              argmax, maxval);
     return cudaGetLastError();
 }
 
-cudaError_t launch_coeffs_warp(const float* Y, long long N, int ldy, int r, const float* R, int ldr, int M,
-                               const float* cnorm, int mode, float scale, float* S, int lds, int* argmax,
-                               float* maxval, cudaStream_t s) {
-    if (N <= 0) return cudaSuccess;
-    if (r > kCoefR) return cudaErrorInvalidValue;
-    k_coeffs_warp<<<rows_grid(N), 256, 0, s>>>(Y, N, ldy, r, R, ldr, M, cnorm, mode, scale, S, lds, argmax,
-                                               maxval);
+cudaError_t launch_scores(const ScoreArgs& a, cudaStream_t s) {
+    if (a.N <= 0) return cudaSuccess;
+    if (a.r < 1 || a.r > kCoefR) return cudaErrorInvalidValue;
+    ScoreParams p;
+    p.Y = a.Y, p.ldy = a.ldy;
+    p.part = a.part, p.xx = a.xx, p.ks = a.ks;
+    p.xnorm = a.xnorm;
+    p.Yout = a.Yout, p.ldyo = a.ldyo;
+    p.N = a.N, p.r = a.r;
+    p.R = a.R, p.ldr = a.ldr, p.M = a.M, p.cnorm = a.cnorm;
+    p.mode = a.mode, p.scale = a.scale;
+    p.S = a.S, p.lds = a.lds, p.argmax = a.argmax, p.maxval = a.maxval;
+    const int r4 = (a.r + 3) / 4;
+    p.pitch = 4 * (r4 | 1);
+    p.chunk = std::min(a.M, (kRSmemFloats - kCoefWarps * kCoefR) / p.pitch);
+    const size_t smem = sizeof(float) * ((size_t)p.chunk * p.pitch + kCoefWarps * kCoefR);
+    // a block stages R once, so at most about two blocks' worth of rounds per SM of a large batch
+    const long long blocks = std::min<long long>((a.N + kCoefWarps - 1) / kCoefWarps, 152LL * 8);
+    k_scores<<<(unsigned)blocks, kCoefWarps * 32, smem, s>>>(p);
     return cudaGetLastError();
 }
 
 cudaError_t launch_gemm_simt(const GemmArgs& g, cudaStream_t s) {
+    return launch_gemm_simt_parts(g, s, true);
+}
+
+cudaError_t launch_gemm_simt_parts(const GemmArgs& args, cudaStream_t s, bool sum) {
+    GemmArgs g = args;
     if (g.m <= 0 || g.n <= 0 || g.batch <= 0) return cudaSuccess;
+    if (g.ksplit <= 1 && sum) g.kpart = nullptr;
+    // 16-byte loads of four elements: rows (and batches) of fp32 operands on 16-byte boundaries
+    g.a_vec = g.a_type == MAT_F32 && (uintptr_t)g.A % 16 == 0 && g.lda % 4 == 0 && g.a_bstride % 4 == 0;
+    g.b_vec = g.b_type == MAT_F32 && (uintptr_t)g.B % 16 == 0 && g.ldb % 4 == 0 && g.b_bstride % 4 == 0;
     if (g.ksplit > 1 && (g.batch != 1 || g.c_type != MAT_F32 || !g.kpart)) return cudaErrorInvalidValue;
     if (g.gate_xn2) {
         if (g.batch != 1 || g.ksplit > 1 || g.a_type != MAT_F32 || g.b_type != MAT_F32 || g.c_type != MAT_F32 ||
@@ -672,7 +891,7 @@ cudaError_t launch_gemm_simt(const GemmArgs& g, cudaStream_t s) {
 #define GS_GEMM_CASE(TA, TB, TC, BT)                                                        \
     if (g.a_type == TA && g.b_type == TB && g.c_type == TC && g.b_trans == BT) {            \
         k_gemm<TA, TB, TC, BT><<<grid, 256, 0, s>>>(g);                                     \
-        if (g.ksplit > 1) {                                                                 \
+        if (g.ksplit > 1 && sum) {                                                          \
             const long long mn = g.m * g.n;                                                 \
             k_ksum<<<(unsigned)((mn + 255) / 256), 256, 0, s>>>(g.kpart, g.ksplit, g.m, g.n, \
                                                                  (float*)g.C, g.ldc);       \
