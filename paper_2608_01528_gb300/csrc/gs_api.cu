@@ -158,13 +158,14 @@ gs_status ps_two_gemm(const gs_basis* h, const float* X, long long N, int ldx, i
 }
 
 // K chunks for the fp32 GEMM of m x n outputs over depth k: enough 64 x 64 tiles x chunks to
-// give every SM about two blocks, chunks of at least 512.
+// give every SM four blocks (each keeps one 16-deep step of loads in flight, so the blocks hide the
+// memory's latency; four are resident at once), chunks of at least 128.
 int gemm_ksplit(long long m, int n, int k, int dev) {
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const long long tiles = ((m + 63) / 64) * ((n + 63) / 64);
-    const long long want = (2LL * std::max(sms, 1) + tiles - 1) / tiles;
-    const long long most = std::max(1, k / 512);
+    const long long want = 4LL * std::max(sms, 1) / tiles;
+    const long long most = std::max(1, k / 128);
     return (int)std::max(1LL, std::min(want, most));
 }
 

@@ -100,7 +100,7 @@ gs_status import_basis(const float* Q, int ldq, const float* R, int ldr_in, cons
 // ----------------------------------------------------------------- SIMT kernels (gs_simt.cu)
 enum { MAT_F32 = 0, MAT_BF16 = 1 };
 
-// fused small-r project + similarity, four queries per block (r <= 32)
+// fused small-r project + similarity, 4 to 16 queries per block (r <= 32)
 cudaError_t launch_ps_small(const float* X, long long N, int ldx, int D, const float* Q, int r,
                             const float* R, int ldr, int M, const float* cnorm, int mode, float scale,
                             float* Y, int ldy, float* S, int lds, int* argmax, float* maxval,

@@ -5,7 +5,7 @@
 // shape can take (GS_PATH_SIMT).  The large-batch hot path is on tcgen05 in
 // gs_tc.cu.
 //
-//  k_ps_small     fused project + similarity, four queries per block, r <= 32
+//  k_ps_small     fused project + similarity, 4 to 16 queries per block, r <= 32
 //                 (Sec. 3.1 t = U^T x; Sec. 2.2 similarity; Eq. 2-3)
 //  k_scores       similarity of Gram-loc queries (or of K-split partial sums of them), one warp per
 //                 query, r <= 64 (Sec. 3.2, Eq. 2)
@@ -201,157 +201,180 @@ __global__ void __launch_bounds__(kCoefWarps * 32) k_scores(const ScoreParams p)
 }
 
 // ----------------------------------------------------------------- fused project + score, r <= 32
-// A block takes kSmallQ queries; its warps split the D dimension (chunks of 128, dealt in turn), a lane
-// four dimensions of a chunk, and keeps all kSmallQ x r partial products in registers: per chunk a lane
-// reads kSmallQ + r vectors for 4 kSmallQ r FMAs.  The lanes' sums fold in a butterfly that leaves
-// entry l in lane l, the warps' meet in shared memory; warp t then scores query t.  Bound by the
-// latency of the loads on the usual few hundred queries.  (One warp per query read all of Q per
-// query, 4 bytes a lane: 2,048 queries of D = 1024, r = 30: 96 us, now 9.)
+// A block takes QB queries against the whole basis (RB >= r rows): chunks of 128 dimensions of both go
+// through a cp.async ring, each of the eight warps takes 16 dimensions of a chunk for all
+// QB x RB products (a lane QB / 4 x RB / 8 of them, 16-byte shared reads without conflicts), the warps'
+// sums meet in shared memory, and the warps score the queries.  Bound by the loads' latency at the usual
+// few hundred queries.  One warp per query read all of Q per query, 4 bytes a lane (2,048 queries of D =
+// 1024, r = 30: 45 us); four queries' products in one warp's registers left few for loads in flight (19).
 constexpr int kSmallR = 32;
-constexpr int kSmallQ = 4;
+constexpr int kSmallM = 64;   // codewords kept in shared memory
+constexpr int kSmallKC = 128, kSmallPitch = kSmallKC + 4;
+// ring depth: the few-query blocks have an SM each and are bound by latency alone
+constexpr int small_stages(int qb) { return qb == 4 ? 8 : 4; }
 
-// entry idx of v[RM] summed over the warp: lane l returns the sum of entry l % RM
-template <int RM>
-__device__ __forceinline__ float fold_entries(float (&v)[RM], int lane) {
-#pragma unroll
-    for (int w = RM / 2; w >= 1; w >>= 1) {
-        const bool up = (lane & w) != 0;
-#pragma unroll
-        for (int j = 0; j < w; ++j) {
-            const float send = up ? v[j] : v[j + w], keep = up ? v[j + w] : v[j];
-            v[j] = keep + __shfl_xor_sync(0xffffffffu, send, w);
-        }
-    }
-    float x = v[0];
-#pragma unroll
-    for (int w = RM; w < 32; w <<= 1) x += __shfl_xor_sync(0xffffffffu, x, w);
-    return x;
+__device__ __forceinline__ void cp_async_zfill16(float* dst, const float* src, int bytes) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+                 "r"(bytes)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async_zfill4(float* dst, const float* src, int bytes) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+                 "r"(bytes)
+                 : "memory");
 }
 
-template <int RM, bool VEC>
+template <int QB, int RB, bool VEC>
 __global__ void __launch_bounds__(256) k_ps_small(const float* __restrict__ X, long long N, int ldx, int D,
                                                   const float* __restrict__ Q, int r, const float* __restrict__ R,
                                                   int ldr, int M, const float* __restrict__ cnorm, int mode,
                                                   float scale, float* __restrict__ Y, int ldy, float* __restrict__ S,
                                                   int lds, int* __restrict__ argmax, float* __restrict__ maxval) {
-    __shared__ float red[8][kSmallQ][kSmallR + 1];
-    __shared__ float ysm[kSmallQ][kSmallR];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    const long long n0 = (long long)blockIdx.x * kSmallQ;
-    const float* x[kSmallQ];
-#pragma unroll
-    for (int t = 0; t < kSmallQ; ++t) x[t] = X + (size_t)(n0 + t < N ? n0 + t : N - 1) * ldx;
-    float acc[kSmallQ][RM], xx[kSmallQ];
-#pragma unroll
-    for (int t = 0; t < kSmallQ; ++t) {
-        xx[t] = 0.f;
-#pragma unroll
-        for (int j = 0; j < RM; ++j) acc[t][j] = 0.f;
+    constexpr int NQ = QB / 4, NJ = RB / 8, kRows = QB + RB, kSmallStages = small_stages(QB);
+    extern __shared__ float4 small_sm[];
+    float* ring = reinterpret_cast<float*>(small_sm);  // kSmallStages x kRows rows: the queries, then Q
+    __shared__ float ysm[QB][kSmallR], xsm[QB];
+    __shared__ float Rs[kSmallM][kSmallR + 1];  // codewords (up to kSmallM), odd pitch: a row per lane
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const long long n0 = (long long)blockIdx.x * QB;
+    const int nch = (D + kSmallKC - 1) / kSmallKC;
+    auto fetch = [&](int c) {
+        float* st = ring + (size_t)(c % kSmallStages) * kRows * kSmallPitch;
+        constexpr int W = VEC ? 4 : 1, kPer = kSmallKC / W;
+        for (int e = threadIdx.x; e < kRows * kPer; e += 256) {
+            const int row = e / kPer, d = e % kPer * W, gd = c * kSmallKC + d;
+            // rows past the end: any valid one, whose sums nobody reads; past D: zeros
+            const float* src = row < QB ? X + (size_t)(n0 + row < N ? n0 + row : N - 1) * ldx
+                                        : Q + (size_t)(row - QB < r ? row - QB : 0) * D;
+            const int left = min(W, max(0, D - gd));
+            float* dst = st + row * kSmallPitch + d;
+            if (VEC)
+                cp_async_zfill16(dst, src + (left ? gd : 0), 4 * left);
+            else
+                cp_async_zfill4(dst, src + (left ? gd : 0), 4 * left);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    for (int c = 0; c < kSmallStages - 1; ++c) {
+        if (c < nch) fetch(c);
+        else asm volatile("cp.async.commit_group;" ::: "memory");
     }
-    for (int c = warp; c * 128 < D; c += nw) {
-        if (VEC) {  // D % 4 == 0, rows 16-byte aligned: a lane four consecutive dimensions
-            const int d = c * 128 + 4 * lane;
-            if (d >= D) continue;
-            float4 xv[kSmallQ];
+    const bool staged = M <= kSmallM;
+    if (staged)  // in flight under the projection
+        for (int e = threadIdx.x; e < M * RB; e += 256) {
+            const int i = e / RB, j = e % RB;
+            Rs[i][j] = j < r ? __ldg(R + (size_t)i * ldr + j) : 0.f;
+        }
+    const int jg = lane & 7, qg = lane >> 3;  // queries qg + 4 v, basis rows jg + 8 u
+    float acc[NQ][NJ] = {}, xx[NQ] = {};
+    for (int c = 0; c < nch; ++c) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(kSmallStages - 2) : "memory");
+        __syncthreads();  // chunk c is here for every thread, and chunk c - 1's stage has been read
+        if (c + kSmallStages - 1 < nch) fetch(c + kSmallStages - 1);
+        else asm volatile("cp.async.commit_group;" ::: "memory");
+        const float* st = ring + (size_t)(c % kSmallStages) * kRows * kSmallPitch + 16 * warp;
 #pragma unroll
-            for (int t = 0; t < kSmallQ; ++t) {
-                xv[t] = __ldg(reinterpret_cast<const float4*>(x[t] + d));
-                xx[t] = fmaf(xv[t].x, xv[t].x, fmaf(xv[t].y, xv[t].y, fmaf(xv[t].z, xv[t].z, fmaf(xv[t].w, xv[t].w, xx[t]))));
-            }
+        for (int k = 0; k < 16; k += 4) {
+            float4 x[NQ], q[NJ];
 #pragma unroll
-            for (int j = 0; j < RM; ++j) {
-                if (j >= r) break;
-                const float4 q = __ldg(reinterpret_cast<const float4*>(Q + (size_t)j * D + d));
+            for (int v = 0; v < NQ; ++v) x[v] = *reinterpret_cast<const float4*>(st + (qg + 4 * v) * kSmallPitch + k);
 #pragma unroll
-                for (int t = 0; t < kSmallQ; ++t)
-                    acc[t][j] = fmaf(xv[t].x, q.x, fmaf(xv[t].y, q.y, fmaf(xv[t].z, q.z, fmaf(xv[t].w, q.w, acc[t][j]))));
-            }
-        } else {
-            for (int u = 0; u < 4; ++u) {
-                const int d = c * 128 + 32 * u + lane;
-                if (d >= D) break;
-                float xv[kSmallQ];
+            for (int u = 0; u < NJ; ++u) q[u] = *reinterpret_cast<const float4*>(st + (QB + jg + 8 * u) * kSmallPitch + k);
 #pragma unroll
-                for (int t = 0; t < kSmallQ; ++t) {
-                    xv[t] = __ldg(x[t] + d);
-                    xx[t] = fmaf(xv[t], xv[t], xx[t]);
-                }
+            for (int v = 0; v < NQ; ++v) {
+                xx[v] = fmaf(x[v].x, x[v].x, fmaf(x[v].y, x[v].y, fmaf(x[v].z, x[v].z, fmaf(x[v].w, x[v].w, xx[v]))));
 #pragma unroll
-                for (int j = 0; j < RM; ++j) {
-                    if (j >= r) break;
-                    const float q = __ldg(Q + (size_t)j * D + d);
-#pragma unroll
-                    for (int t = 0; t < kSmallQ; ++t) acc[t][j] = fmaf(xv[t], q, acc[t][j]);
-                }
+                for (int u = 0; u < NJ; ++u)
+                    acc[v][u] = fmaf(x[v].x, q[u].x, fmaf(x[v].y, q[u].y, fmaf(x[v].z, q[u].z, fmaf(x[v].w, q[u].w, acc[v][u]))));
             }
         }
     }
+    // the warps' sums, through the ring's memory: [warp][query][RB + 1], the last the squared norm
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    float* red = ring;
 #pragma unroll
-    for (int t = 0; t < kSmallQ; ++t) {
-        const float y = fold_entries<RM>(acc[t], lane);
-        const float s = warp_sum(xx[t]);
-        if (lane < RM) red[warp][t][lane] = y;
-        if (lane == 0) red[warp][t][kSmallR] = s;
+    for (int v = 0; v < NQ; ++v) {
+        float* row = red + ((size_t)warp * QB + qg + 4 * v) * (RB + 1);
+#pragma unroll
+        for (int u = 0; u < NJ; ++u) row[jg + 8 * u] = acc[v][u];
+        if (jg == 0) row[RB] = xx[v];
     }
     __syncthreads();
-    const long long n = n0 + warp;
-    if (warp >= kSmallQ || n >= N) return;
-    float yl = 0.f, x2 = 0.f;
-    for (int w = 0; w < nw; ++w) {
-        if (lane < r) yl += red[w][warp][lane];
-        x2 += red[w][warp][kSmallR];
-    }
-    if (Y && lane < r) Y[(size_t)n * ldy + lane] = yl;
-    ysm[warp][lane] = yl;
-    __syncwarp();
-    float y[RM];
+    for (int e = threadIdx.x; e < QB * (RB + 1); e += 256) {
+        const int qi = e / (RB + 1), j = e - qi * (RB + 1);
+        float t = 0.f;
 #pragma unroll
-    for (int j = 0; j < RM; ++j) y[j] = ysm[warp][j];
-    const float xnorm = sqrtf(x2);
-    // scores: lane handles codewords i = lane, lane + 32, ...
-    auto score = [&](int i) {
-        const float* Ri = R + (size_t)i * ldr;
-        float g = 0.f;
+        for (int w = 0; w < 8; ++w) t += red[((size_t)w * QB + qi) * (RB + 1) + j];
+        if (j == RB) {
+            xsm[qi] = t;
+        } else {
+            ysm[qi][j] = t;
+            if (Y && j < r && n0 + qi < N) Y[(size_t)(n0 + qi) * ldy + j] = t;
+        }
+    }
+    __syncthreads();
+    for (int qi = warp; qi < QB; qi += 8) {
+        const long long n = n0 + qi;
+        if (n >= N) break;
+        float y[RB];
 #pragma unroll
-        for (int j = 0; j < RM; ++j)
-            if (j < r) g = fmaf(y[j], __ldg(Ri + j), g);
-        g *= scale;
-        if (mode == GS_SCORE_COSINE) {
-            const float den = xnorm * cnorm[i];
-            g = den > 0.f ? g / den : 0.f;
+        for (int j = 0; j < RB; ++j) y[j] = j < r ? ysm[qi][j] : 0.f;
+        const float x2 = xsm[qi];
+        const float xnorm = sqrtf(x2);
+        // scores: lane handles codewords i = lane, lane + 32, ...
+        auto score = [&](int i) {
+            float g = 0.f;
+            if (staged) {
+#pragma unroll
+                for (int j = 0; j < RB; ++j) g = fmaf(y[j], Rs[i][j], g);
+            } else {
+                const float* Ri = R + (size_t)i * ldr;
+#pragma unroll
+                for (int j = 0; j < RB; ++j)
+                    if (j < r) g = fmaf(y[j], __ldg(Ri + j), g);
+            }
+            g *= scale;
+            if (mode == GS_SCORE_COSINE) {
+                const float den = xnorm * cnorm[i];
+                g = den > 0.f ? g / den : 0.f;
+            }
+            return g;
+        };
+        float bv = -FLT_MAX;
+        int bi = 0x7fffffff;
+        for (int i = lane; i < M; i += 32) {
+            const float g = score(i);
+            if (g > bv) {
+                bv = g;
+                bi = i;
+            }
+            if (S && mode != GS_SCORE_SOFTMAX) S[(size_t)n * lds + i] = g;
         }
-        return g;
-    };
-    float bv = -FLT_MAX;
-    int bi = 0x7fffffff;
-    for (int i = lane; i < M; i += 32) {
-        const float g = score(i);
-        if (g > bv) {
-            bv = g;
-            bi = i;
+        warp_argmax(bv, bi);
+        if (bi == 0x7fffffff) bi = 0;
+        float outmax = bv;
+        if (mode == GS_SCORE_SOFTMAX) {
+            float z = 0.f;
+            for (int i = lane; i < M; i += 32) z += __expf(score(i) - bv);
+            z = warp_sum(z);
+            const float inv = 1.f / z;
+            if (S)
+                for (int i = lane; i < M; i += 32) S[(size_t)n * lds + i] = __expf(score(i) - bv) * inv;
+            outmax = inv;
         }
-        if (S && mode != GS_SCORE_SOFTMAX) S[(size_t)n * lds + i] = g;
-    }
-    warp_argmax(bv, bi);
-    if (bi == 0x7fffffff) bi = 0;
-    float outmax = bv;
-    if (mode == GS_SCORE_SOFTMAX) {
-        float z = 0.f;
-        for (int i = lane; i < M; i += 32) z += __expf(score(i) - bv);
-        z = warp_sum(z);
-        const float inv = 1.f / z;
-        if (S)
-            for (int i = lane; i < M; i += 32) S[(size_t)n * lds + i] = __expf(score(i) - bv) * inv;
-        outmax = inv;
-    }
-    if (lane == 0) {
-        if (argmax) argmax[n] = M > 0 ? bi : 0;
-        if (maxval) maxval[n] = M > 0 ? outmax : 0.f;
+        if (lane == 0) {
+            if (argmax) argmax[n] = M > 0 ? bi : 0;
+            if (maxval) maxval[n] = M > 0 ? outmax : 0.f;
+        }
     }
 }
 
 // ----------------------------------------------------------------- tiled GEMM
-constexpr int kTM = 64, kTN = 64, kTK = 16;
+// 256 threads, each MT x 4 outputs: tiles of 16 MT x 64 (MT = 8 reads 3 shared vectors per 32 FMAs, MT = 4
+// two per 16; the smaller tile where the larger would leave SMs without work)
+constexpr int kTN = 64, kTK = 16;
+constexpr int kTM = 64;  // MT = 4
 
 template <int T>
 __device__ __forceinline__ float ld_elem(const void* p, long long i) {
@@ -375,9 +398,9 @@ __device__ __forceinline__ void ld4(const void* p, long long i, int left, bool v
 // called by every thread of the block.  A thread loads four consecutive elements of each operand per
 // K step (one 16-byte load where rows are aligned), the next step's while the current one is multiplied
 // (two shared buffers, one barrier a step): 1,024 x 40 over K = 8192 in 16 chunks went from 52 to 24 us.
-template <int TA, int TB, int TC, bool BT>
+template <int TA, int TB, int TC, bool BT, int MT>
 __device__ __forceinline__ void gemm_tile(const GemmArgs& g, long long m0, int n0, int kz,
-                                          float (&As)[2][kTK][kTM + 4], float (&Bs)[2][kTK][kTN + 4]) {
+                                          float (&As)[2][kTK][16 * MT + 4], float (&Bs)[2][kTK][kTN + 4]) {
     const int tid = threadIdx.x;
     const int tx = tid % 16, ty = tid / 16;
     const bool split = g.ksplit > 1;
@@ -406,13 +429,21 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs& g, long long m0, int n
     }
     // A: row lr, k lk .. lk + 3 of the step; B the same (K-major), or k br, columns bc .. bc + 3
     const int lr = tid / 4, lk = tid % 4 * 4, br = tid / 16, bc = tid % 16 * 4;
-    const long long gm = m0 + lr;
-    const long long arow = (gm < g.m ? gm : g.m - 1) * g.lda;
-    const bool a_in = gm < g.m, b_in = n0 + lr < g.n;
+    constexpr int AR = MT / 4;  // rows lr, lr + 64 of A
+    long long arow[AR];
+    bool a_in[AR];
+#pragma unroll
+    for (int h = 0; h < AR; ++h) {
+        const long long gm = m0 + lr + 64 * h;
+        a_in[h] = gm < g.m;
+        arow[h] = (a_in[h] ? gm : g.m - 1) * g.lda;
+    }
+    const bool b_in = n0 + lr < g.n;
     const long long brow = BT ? (long long)(b_in ? n0 + lr : g.n - 1) * g.ldb : 0;
-    float av[4], bv[4], xx = 0.f;
+    float av[AR][4], bv[4], xx[AR] = {};
     auto load = [&](int k0) {
-        ld4<TA>(Ab, arow + k0 + lk, a_in ? kend - (k0 + lk) : 0, g.a_vec, av);
+#pragma unroll
+        for (int h = 0; h < AR; ++h) ld4<TA>(Ab, arow[h] + k0 + lk, a_in[h] ? kend - (k0 + lk) : 0, g.a_vec, av[h]);
         if (BT)
             ld4<TB>(Bb, brow + k0 + lk, b_in ? kend - (k0 + lk) : 0, g.b_vec, bv);
         else
@@ -421,13 +452,16 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs& g, long long m0, int n
     auto store = [&](int buf) {
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            As[buf][lk + u][lr] = av[u];
+#pragma unroll
+            for (int h = 0; h < AR; ++h) {
+                As[buf][lk + u][lr + 64 * h] = av[h][u];
+                xx[h] = fmaf(av[h][u], av[h][u], xx[h]);
+            }
             if (BT) Bs[buf][lk + u][lr] = bv[u];
-            xx = fmaf(av[u], av[u], xx);
         }
         if (!BT) *reinterpret_cast<float4*>(&Bs[buf][br][bc]) = make_float4(bv[0], bv[1], bv[2], bv[3]);
     };
-    float acc[4][4] = {};
+    float acc[MT][4] = {};
     if (kbeg < kend) {
         load(kbeg);
         store(0);
@@ -439,11 +473,14 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs& g, long long m0, int n
         if (more) load(k0 + kTK);
 #pragma unroll
         for (int kk = 0; kk < kTK; ++kk) {
-            const float4 a4 = *reinterpret_cast<const float4*>(&As[buf][kk][ty * 4]);
-            const float4 b4 = *reinterpret_cast<const float4*>(&Bs[buf][kk][tx * 4]);
-            const float a[4] = {a4.x, a4.y, a4.z, a4.w}, bb[4] = {b4.x, b4.y, b4.z, b4.w};
+            float a[MT];
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int h = 0; h < AR; ++h)
+                *reinterpret_cast<float4*>(a + 4 * h) = *reinterpret_cast<const float4*>(&As[buf][kk][ty * 4 + 64 * h]);
+            const float4 b4 = *reinterpret_cast<const float4*>(&Bs[buf][kk][tx * 4]);
+            const float bb[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+            for (int i = 0; i < MT; ++i)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], bb[j], acc[i][j]);
         }
@@ -451,14 +488,18 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs& g, long long m0, int n
         __syncthreads();
     }
     if (g.xx_part && n0 == 0) {  // this chunk's part of each row's squared norm
-        xx += __shfl_xor_sync(0xffffffffu, xx, 1);
-        xx += __shfl_xor_sync(0xffffffffu, xx, 2);
-        if (lk == 0 && a_in) g.xx_part[(size_t)kz * g.m + gm] = xx;
+#pragma unroll
+        for (int h = 0; h < AR; ++h) {
+            float x = xx[h];
+            x += __shfl_xor_sync(0xffffffffu, x, 1);
+            x += __shfl_xor_sync(0xffffffffu, x, 2);
+            if (lk == 0 && a_in[h]) g.xx_part[(size_t)kz * g.m + m0 + lr + 64 * h] = x;
+        }
     }
     char* Cb = (char*)g.C + (size_t)b * g.c_bstride * (TC == MAT_F32 ? 4 : 2);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const long long gi = m0 + ty * 4 + i;
+    for (int i = 0; i < MT; ++i) {
+        const long long gi = m0 + ty * 4 + 64 * (i / 4) + i % 4;
         if (gi >= g.m) continue;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
@@ -479,11 +520,11 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs& g, long long m0, int n
     }
 }
 
-template <int TA, int TB, int TC, bool BT>
-__global__ void __launch_bounds__(256) k_gemm(GemmArgs g) {
-    __shared__ __align__(16) float As[2][kTK][kTM + 4];
+template <int TA, int TB, int TC, bool BT, int MT>
+__global__ void __launch_bounds__(256, MT == 8 ? 3 : 4) k_gemm(GemmArgs g) {
+    __shared__ __align__(16) float As[2][kTK][16 * MT + 4];
     __shared__ __align__(16) float Bs[2][kTK][kTN + 4];
-    gemm_tile<TA, TB, TC, BT>(g, (long long)blockIdx.y * kTM, blockIdx.x * kTN, blockIdx.z, As, Bs);
+    gemm_tile<TA, TB, TC, BT, MT>(g, (long long)blockIdx.y * (16 * MT), blockIdx.x * kTN, blockIdx.z, As, Bs);
 }
 
 // The gated product (gate_xn2): each block takes a run of consecutive 64 x 64 tiles, n fastest, and
@@ -515,7 +556,7 @@ __global__ void __launch_bounds__(256) k_gemm_gated(GemmArgs g, long long per) {
             any = __syncthreads_or(mine) != 0;
             last_m0 = m0;
         }
-        if (any) gemm_tile<TA, TB, TC, BT>(g, m0, (int)(t % tiles_n) * kTN, 0, As, Bs);
+        if (any) gemm_tile<TA, TB, TC, BT, 4>(g, m0, (int)(t % tiles_n) * kTN, 0, As, Bs);
     }
 }
 
@@ -827,15 +868,37 @@ cudaError_t launch_ps_small(const float* X, long long N, int ldx, int D, const f
                             float* Y, int ldy, float* S, int lds, int* argmax, float* maxval,
                             cudaStream_t s) {
     const bool vec = (uintptr_t)X % 16 == 0 && ldx % 4 == 0 && D % 4 == 0 && (uintptr_t)Q % 16 == 0;
-    const long long blocks = (N + kSmallQ - 1) / kSmallQ;
-    // eight warps share D while every block has an SM of its own (a block holds ~170 registers a
-    // thread), four once blocks queue
-    const int threads = blocks <= 152 ? 256 : 128;
-    auto kern = r <= 8 ? (vec ? k_ps_small<8, true> : k_ps_small<8, false>)
-                : r <= 16 ? (vec ? k_ps_small<16, true> : k_ps_small<16, false>)
-                          : (vec ? k_ps_small<32, true> : k_ps_small<32, false>);
-    kern<<<(unsigned)blocks, threads, 0, s>>>(X, N, ldx, D, Q, r, R, ldr, M, cnorm, mode, scale, Y, ldy, S, lds,
-                                              argmax, maxval);
+    // queries per block: few while blocks are fewer than the SMs, more once they queue (each block
+    // reads all of Q)
+    const int qb = N <= 4 * 152 ? 4 : N <= 16 * 152 ? 8 : 16;
+    const int rb = r <= 8 ? 8 : r <= 16 ? 16 : 32;
+    const size_t smem = sizeof(float) * std::max((size_t)small_stages(qb) * (qb + rb) * kSmallPitch, (size_t)8 * qb * (rb + 1));
+    const unsigned blocks = (unsigned)((N + qb - 1) / qb);
+    static bool opted[64];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+#define GS_SMALL_CASE(QB, RB)                                                                          \
+    if (!opted[dev])                                                                                   \
+        for (auto fn : {k_ps_small<QB, RB, true>, k_ps_small<QB, RB, false>}) {                        \
+            e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);     \
+            if (e != cudaSuccess) return e;                                                            \
+        }                                                                                              \
+    if (qb == QB && rb == RB) kern = vec ? k_ps_small<QB, RB, true> : k_ps_small<QB, RB, false>;
+    auto kern = k_ps_small<4, 8, true>;
+    GS_SMALL_CASE(4, 8)
+    GS_SMALL_CASE(4, 16)
+    GS_SMALL_CASE(4, 32)
+    GS_SMALL_CASE(8, 8)
+    GS_SMALL_CASE(8, 16)
+    GS_SMALL_CASE(8, 32)
+    GS_SMALL_CASE(16, 8)
+    GS_SMALL_CASE(16, 16)
+    GS_SMALL_CASE(16, 32)
+#undef GS_SMALL_CASE
+    opted[dev] = true;
+    kern<<<blocks, 256, smem, s>>>(X, N, ldx, D, Q, r, R, ldr, M, cnorm, mode, scale, Y, ldy, S, lds, argmax, maxval);
     return cudaGetLastError();
 }
 
@@ -885,12 +948,15 @@ cudaError_t launch_gemm_simt_parts(const GemmArgs& args, cudaStream_t s, bool su
         k_gemm_gated<MAT_F32, MAT_F32, MAT_F32, true><<<(unsigned)((tiles + per - 1) / per), 256, 0, s>>>(g, per);
         return cudaGetLastError();
     }
-    dim3 grid((unsigned)((g.n + kTN - 1) / kTN), (unsigned)((g.m + kTM - 1) / kTM),
-              (unsigned)(g.ksplit > 1 ? g.ksplit : g.batch));
+    const long long z = g.ksplit > 1 ? g.ksplit : g.batch, tn = (g.n + kTN - 1) / kTN;
+    const bool tall = (g.m + 127) / 128 * tn * z >= 300;  // about two 128-row tiles for every SM
+    const int tm = tall ? 128 : kTM;
+    dim3 grid((unsigned)tn, (unsigned)((g.m + tm - 1) / tm), (unsigned)z);
     if (grid.y > 65535u) return cudaErrorInvalidConfiguration;
 #define GS_GEMM_CASE(TA, TB, TC, BT)                                                        \
     if (g.a_type == TA && g.b_type == TB && g.c_type == TC && g.b_trans == BT) {            \
-        k_gemm<TA, TB, TC, BT><<<grid, 256, 0, s>>>(g);                                     \
+        if (tall) k_gemm<TA, TB, TC, BT, 8><<<grid, 256, 0, s>>>(g);                        \
+        else k_gemm<TA, TB, TC, BT, 4><<<grid, 256, 0, s>>>(g);                             \
         if (g.ksplit > 1 && sum) {                                                          \
             const long long mn = g.m * g.n;                                                 \
             k_ksum<<<(unsigned)((mn + 255) / 256), 256, 0, s>>>(g.kpart, g.ksplit, g.m, g.n, \
