@@ -103,7 +103,8 @@ struct PanelState {
     int slow;    // a rank decision needs the row-by-row kernel
     int nacc;    // accepted rows, in order
     int acc[kPanel];
-    double L[kPanel][kPanel];  // V = L V' (V': nacc rows)
+    double G[kPanel][kPanel];  // V V^T
+    double T[kPanel][kPanel];  // V' = T V (nacc rows)
 };
 
 __device__ __forceinline__ void cp_async8(double* dst, const double* src) {
@@ -344,23 +345,31 @@ __global__ void __launch_bounds__(256) k_panel_reduce(const double* __restrict__
     }
 }
 
-// 3. Inside the panel: Cholesky QR, twice.  G = V V^T (summed over the slices) = L L^T, V' = L^-1 V has
-//    rows orthonormal up to the loss of forming G (eps times the panel's condition squared); a second
-//    round on V' brings that to eps, and V = (L L2) V''.  Each round is one pass over the slices with
-//    every CTA doing the 16 x 16 factorisation itself, against three cluster-wide sums per row
-//    (k_panel_gs2: 326 us a panel at D = 4096, of which ~65 us were arithmetic; two rounds take ~25 us).
+// 3. Inside the panel: Cholesky QR, twice.  G = V V^T (summed over the slices) = L L^T, V' = T V with T ~
+//    L^-1 has rows orthonormal up to the rounding of T and G times the panel's condition squared; a
+//    second round on V' brings that to eps: V'' = T2 V', and the panel's rows of R are V V''^T =
+//    G T^T T2^T.  Each round is one pass over the slices with every CTA doing the 16 x 16 factorisation
+//    itself, against three cluster-wide sums per row (k_panel_gs2: 326 us a panel at D = 4096, of which
+//    ~65 us were arithmetic).
+//    T need not be exact, V' = T V only has to be taken in fp64 with the T that is used: the first
+//    round's factorisation runs in fp32, one warp, a row per lane (rows scaled by powers of two), where
+//    every pivot stays above 1e-3 of its row and certain of its rank decision; otherwise in fp64.  The
+//    second round's Gram matrix is then I + E with |E| ~ 1e-7, whose Cholesky factor I + X and T2 come
+//    from their series (X = lower(E - X X^T) iterated, T2 = I - X + X^2 - X^3: errors below |E|^4) in four
+//    16 x 16 products; otherwise by the fp64 factorisation.  (fp64 runs at 2 FMAs per clock and SM here,
+//    16 dependent steps of it cost ~20 us: the two rounds took 57 us a panel with both in fp64.)
 //    Row k is accepted exactly as the row-by-row kernel would: its norm against what came before it,
-//    sqrt(pivot), > tau ||c_k||.  A pivot taken from G is only known to ~1e-14 ||v_k||^2, so a panel
-//    with a decision that this could touch (a pivot below 1e-6 ||v_k||^2 that is not certain to fall
-//    below the tolerance, or one within 1e-6 of it) is left to k_panel_gs2.
+//    sqrt(pivot), > tau ||c_k||.  A pivot taken from G in fp64 is only known to ~1e-14 ||v_k||^2, so a
+//    panel with a decision that this could touch (a pivot below 1e-6 ||v_k||^2 that is not certain to
+//    fall below the tolerance, or one within 1e-6 of it) is left to k_panel_gs2.
 //
-// The factorisation in one CTA (all threads): A (the Gram matrix, overwritten), T: rows of L^-1 for the
-// accepted rows (T[a] over the panel's rows), L as in PanelState.  first: the rank decisions are taken;
-// otherwise every row is accepted.  rsqrt of a pivot runs in one thread, the 16 x 16 updates in one
-// FMA per thread (256 of A, 256 of T with 512 threads).
+// The factorisation in one CTA (all threads): A (the Gram matrix; the fp64 form overwrites it), T: rows of
+// the transform for the accepted rows (T[k] over the panel's rows).
 struct Chol {
     double A[kPanel][kPanel + 1], T[kPanel][kPanel + 1], L[kPanel][kPanel], diag[kPanel], nv[kPanel], rs;
-    int acc[kPanel], nacc, slow, take;
+    double W[kPanel][kPanel + 1];
+    float Af[kPanel][kPanel + 1];
+    int acc[kPanel], nacc, slow, take, quick;
 };
 
 __device__ __forceinline__ void chol_load(Chol& c, const double* Gp, int ncl) {
@@ -436,6 +445,128 @@ __device__ __forceinline__ void chol_factor(Chol& c, int n, bool first, const do
     }
 }
 
+// 2^-e for a squared norm in [4^e, 4^(e+1)) (1 when it is not a positive finite number)
+__device__ __forceinline__ double row_unscale(double n2) {
+    if (!(n2 > 0.0) || !(n2 <= DBL_MAX)) return 1.0;
+    const int e = (((__double2hiint(n2) >> 20) & 0x7ff) - 1023) >> 1;
+    return __hiloint2double((1023 - e) << 20, 0);
+}
+
+// The first round's factorisation in fp32 on warp 0 (all threads call it): sets T, acc, nacc and quick when
+// every decision is certain.
+__device__ __forceinline__ void chol_quick(Chol& c, int n, const double* cn, double tau, int room) {
+    for (int e = threadIdx.x; e < kPanel * kPanel; e += blockDim.x) {
+        const int i = e / kPanel, j = e % kPanel;
+        c.Af[i][j] = (float)(c.A[i][j] * row_unscale(c.diag[i]) * row_unscale(c.diag[j]));
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x, i = lane & 15;
+        float a[kPanel], t[kPanel];
+#pragma unroll
+        for (int j = 0; j < kPanel; ++j) {
+            a[j] = c.Af[i][j];
+            t[j] = i == j ? 1.f : 0.f;
+        }
+        const float d = c.Af[i][i];
+        // rows below the tolerance already are dependent; the others' tolerance in the scaled units
+        bool out = true;
+        float lim = 0.f;
+        bool sure = true;
+        if (i < n) {
+            const double l = tau * cn[i], l2 = l * l, v2 = c.diag[i], u = row_unscale(v2);
+            out = !(v2 > l2 * (1.0 - 1e-6));
+            lim = (float)(l2 * u * u);
+            sure = v2 == v2 && v2 <= DBL_MAX && (out || (d >= 1.f && d < 4.1f));
+        }
+        bool ok = __all_sync(0xffffffffu, sure);
+        int na = 0;
+        unsigned taken = 0;
+#pragma unroll
+        for (int k = 0; k < kPanel; ++k) {
+            const bool skip = __shfl_sync(0xffffffffu, (int)out, k) != 0;
+            const float piv = __shfl_sync(0xffffffffu, a[k], k), dk = __shfl_sync(0xffffffffu, d, k),
+                        lk = __shfl_sync(0xffffffffu, lim, k);
+            if (k >= n || skip || na >= room) continue;  // (warp-uniform)
+            ok = ok && piv > 1e-3f * dk && piv > 1.001f * lk;
+            const float rs = rsqrtf(piv), l = a[k] * rs;
+#pragma unroll
+            for (int j = 0; j < kPanel; ++j) {
+                if (j > k) {
+                    const float lj = __shfl_sync(0xffffffffu, l, j);
+                    if (i > k) a[j] = fmaf(-l, lj, a[j]);
+                } else {
+                    const float tj = __shfl_sync(0xffffffffu, t[j], k) * rs;
+                    if (i > k) t[j] = fmaf(-l, tj, t[j]);
+                    if (i == k) t[j] = tj;
+                }
+            }
+            if (lane == 0) c.acc[na] = k;
+            taken |= 1u << k;
+            ++na;
+        }
+        // T's rounding reaches V' V'^T times (sum_j |t_j| ||v_j||)^2
+        float amp = 0.f;
+#pragma unroll
+        for (int j = 0; j < kPanel; ++j) amp += fabsf(t[j]) * 2.f;
+        ok = ok && __all_sync(0xffffffffu, !((taken >> i) & 1u) || amp < 60.f);
+        if (ok && lane < kPanel) {
+#pragma unroll
+            for (int j = 0; j < kPanel; ++j) c.T[i][j] = (double)t[j] * row_unscale(c.diag[j]);
+        }
+        if (lane == 0) {
+            c.quick = ok;
+            if (ok) c.nacc = na;
+        }
+    }
+    __syncthreads();
+}
+
+// The second round's transform from the series, when the Gram matrix is that close to I: T[0..n).  Entry
+// (i, j <= i) of each 16 x 16 product in one thread, ordered so that a warp's sums have about one length.
+__device__ __forceinline__ bool chol_series(Chol& c, int n) {
+    bool far = false;
+    for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
+        const int i = e / n, j = e % n;
+        far |= !(fabs(c.A[i][j] - (i == j ? 1.0 : 0.0)) < 4e-6);
+    }
+    if (__syncthreads_or(far)) return false;
+    // entries by column (sum length j + 1) and by diagonal (sum length i - j + 1)
+    int ci = -1, cj = 0, di = -1, dj = 0;
+    if (threadIdx.x < kPairs) {
+        int e = threadIdx.x, len = kPanel;
+        while (e >= len) e -= len--;
+        cj = kPanel - len, ci = cj + e;
+        di = kPanel - len + e, dj = e;
+    }
+    const bool con = ci >= 0 && ci < n, don = di >= 0 && di < n;
+    const double eij = con ? (ci == cj ? 0.5 * (c.A[ci][cj] - 1.0) : c.A[ci][cj]) : 0.0;
+    if (con) c.L[ci][cj] = eij;
+    __syncthreads();
+    for (int it = 0; it < 2; ++it) {  // X = lower(E - X X^T), the diagonal halved
+        double s = 0.0;
+        if (con)
+            for (int m = 0; m <= cj; ++m) s += c.L[ci][m] * c.L[cj][m];
+        __syncthreads();
+        if (con) c.L[ci][cj] = eij - (ci == cj ? 0.5 * s : s);
+        __syncthreads();
+    }
+    if (don) c.T[di][dj] = (di == dj ? 1.0 : 0.0) - c.L[di][dj];
+    __syncthreads();
+    for (int it = 0; it < 2; ++it) {  // T = I - X T
+        double s = 0.0;
+        if (don)
+            for (int m = dj; m <= di; ++m) s += c.L[di][m] * c.T[m][dj];
+        __syncthreads();
+        if (don) c.T[di][dj] = (di == dj ? 1.0 : 0.0) - s;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) c.nacc = n;
+    if (threadIdx.x < n) c.acc[threadIdx.x] = threadIdx.x;
+    __syncthreads();
+    return true;
+}
+
 struct CholParams {
     double* V;
     double* Qw;
@@ -467,18 +598,25 @@ __global__ void __launch_bounds__(512) k_panel_chol(const CholParams p) {
     const int n = ROUND == 1 ? p.bp : p.st->nacc;
     for (int e = tid; e < n * w; e += nt) Vs[(e / w) * vl + e % w] = p.V[(size_t)(e / w) * p.D + c0 + e % w];
     chol_load(c, p.Gp, p.ncl);
-    chol_factor(c, n, ROUND == 1, p.cn, p.tau, p.rmax - r0);
     if (ROUND == 1) {
-        // V' = T V multiplies G's rounding by (sum_j |T_kj| ||v_j||)^2: beyond 1e8 the second round would
-        // not bring it back to eps
-        if (tid < p.bp && !c.slow) {
-            double amp = 0.0;
-            for (int j = 0; j <= tid; ++j) amp += fabs(c.T[tid][j]) * c.nv[j];
-            bool taken = false;
-            for (int a = 0; a < c.nacc; ++a) taken |= c.acc[a] == tid;
-            if (taken && !(amp < 1e4)) c.slow = 1;
+        if (blockIdx.x == 0)
+            for (int e = tid; e < kPanel * kPanel; e += nt) p.st->G[e / kPanel][e % kPanel] = c.A[e / kPanel][e % kPanel];
+        chol_quick(c, n, p.cn, p.tau, p.rmax - r0);
+        if (!c.quick) {
+            chol_factor(c, n, true, p.cn, p.tau, p.rmax - r0);
+            // V' = T V multiplies G's rounding by (sum_j |T_kj| ||v_j||)^2: beyond 1e8 the second round would
+            // not bring it back to eps
+            if (tid < p.bp && !c.slow) {
+                double amp = 0.0;
+                for (int j = 0; j <= tid; ++j) amp += fabs(c.T[tid][j]) * c.nv[j];
+                bool taken = false;
+                for (int a = 0; a < c.nacc; ++a) taken |= c.acc[a] == tid;
+                if (taken && !(amp < 1e4)) c.slow = 1;
+            }
+            __syncthreads();
         }
-        __syncthreads();
+    } else if (!chol_series(c, n)) {
+        chol_factor(c, n, false, p.cn, p.tau, p.rmax - r0);
     }
     const bool slow = ROUND == 1 && c.slow != 0;
     if (ROUND == 1 && blockIdx.x == 0) {
@@ -487,7 +625,10 @@ __global__ void __launch_bounds__(512) k_panel_chol(const CholParams p) {
             p.st->nacc = c.nacc;
         }
         for (int e = tid; e < kPanel; e += nt) p.st->acc[e] = c.acc[e];
-        for (int e = tid; e < kPanel * kPanel; e += nt) p.st->L[e / kPanel][e % kPanel] = c.L[e / kPanel][e % kPanel];
+        for (int e = tid; e < c.nacc * kPanel; e += nt) {
+            const int a = e / kPanel, j = e % kPanel;
+            p.st->T[a][j] = j <= c.acc[a] ? c.T[c.acc[a]][j] : 0.0;
+        }
     }
     if (slow) return;  // the same data and so the same answer in every CTA of the grid
     const int na = c.nacc;
@@ -510,11 +651,19 @@ __global__ void __launch_bounds__(512) k_panel_chol(const CholParams p) {
         gram_slice(Vs, vl, w, part);
         cluster_add_pairs(part, p.Gp2 + (size_t)(blockIdx.x / kSliceCluster) * kPairs);
     } else if (blockIdx.x == 0) {
-        // R's new columns: L1 L2
+        // R's new columns, V V''^T = (G T^T) T2^T; entry (k, a) is zero where row k comes before accepted row a
         for (int e = tid; e < p.bp * na; e += nt) {
             const int k = e / na, a = e - k * na;
             double v = 0.0;
-            for (int b = a; b < na; ++b) v += p.st->L[k][b] * c.L[b][a];
+            for (int j = 0; j <= p.st->acc[a]; ++j) v += p.st->G[k][j] * p.st->T[a][j];
+            c.W[k][a] = v;
+        }
+        __syncthreads();
+        for (int e = tid; e < p.bp * na; e += nt) {
+            const int k = e / na, a = e - k * na;
+            if (p.st->acc[a] > k) continue;
+            double v = 0.0;
+            for (int b = 0; b <= a; ++b) v += c.W[k][b] * c.T[a][b];
             p.R64[(size_t)k * p.ldr + r0 + a] = v;
         }
         if (tid == 0) *p.r_next = r0 + na;
