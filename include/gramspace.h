@@ -268,7 +268,7 @@ GS_API gs_status gs_project_similarity_host(const gs_basis* h, const float* X, l
  * r = 0 (every score is then 0).
  * Tensor-core path (GS_PATH_AUTO for large N·M·r): Y and R split into bf16 hi /
  * lo, three products, fp32 accumulation (~2^-16 relative); needs Y 16-byte
- * aligned and ldy % 4 == 0.  Otherwise fp32 CUDA cores.  Uses the basis'
+ * aligned and ldy % 4 == 0.  Otherwise at fp32 accuracy, as gs_prob_vectorize.  Uses the basis'
  * scratch for cosine norms and, when S is NULL, for the scores.
  */
 GS_API gs_status gs_similarity_coeffs(const gs_basis* h, const float* Y, long long N, int ldy, int mode,
@@ -383,7 +383,8 @@ GS_API gs_status gs_reconstruct_bind(const gs_basis* h, const void* T, int t_dty
  * apply_softmax != 0.  Yq is B x Lq x r and Yk is B x Lk x r, both of type
  * in_dtype (GS_F32 or GS_BF16) with row stride ldy elements; A is
  * B x Lq x Lk fp32, dense.  scale = 1/sqrt(D) reproduces full-dimension
- * attention.  Tensor-core path: bf16 inputs, fp32 accumulation.
+ * attention.  Tensor-core path: bf16 inputs, fp32 accumulation.  fp32 inputs: at fp32
+ * accuracy, as gs_prob_vectorize.
  */
 GS_API gs_status gs_attention_scores(const void* Yq, const void* Yk, int in_dtype, int B, int Lq,
                               int Lk, int r, int ldy, float scale, int apply_softmax, float* A,

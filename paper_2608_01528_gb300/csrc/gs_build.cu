@@ -16,8 +16,10 @@
 // paper's construction (projections onto orthonormal directions commute, and
 // Cholesky QR of a panel is its Gram-Schmidt factorisation); the block passes
 // against the old basis and the column slices are what make it data-parallel.
-// Measured (GB300): M = 512, D = 4096: 20.0 ms before the slices were cut to the
-// number of SMs and the panels factored by Cholesky QR; see k_panel_slice.
+// Measured (GB300): M = 512, D = 4096: 7.25 ms (19.9 before the slices were cut to the
+// number of SMs and the panels factored by Cholesky QR); M = 1,024, D = 10,000, rank
+// 922: 38 ms (97).  The fp64 arithmetic of the block projections takes ~2.7 ms of the
+// first, the rest is the chain of eight launches per panel.
 // The only host synchronisation is the read of the final rank r.
 //
 // Afterwards fp32 copies of Q and R are made for the caller, plus the
@@ -85,8 +87,9 @@ __global__ void __launch_bounds__(256) k_row_norms(const float* __restrict__ C, 
 
 // 2. Block projections.  The D columns are cut into slices of w, one CTA each (about one per SM: GB300
 //    does ~2 fp64 FMAs per clock and SM, so a pass over the basis is bound by that pipe and wants every
-//    SM busy for the same time; 64-column CTAs left 88 of 152 SMs idle at D = 4096, 76 us a pass
-//    against 27 us).  A CTA keeps its slice of the panel in shared memory and streams the basis' slice
+//    SM busy for the same time; 64-column CTAs left 88 of 152 SMs idle at D = 4096: dots 64 us and update
+//    77 us per panel and pass, now 36 us for dots alone, 68 us for an update and the next dots, 29 us for
+//    the fp32 update with the Gram matrix).  A CTA keeps its slice of the panel in shared memory and streams the basis' slice
 //    through two buffers (cp.async).  kind:
 //      kDots1    V = C;           Hp = V Q^T                  (first pass' dots, over the slice)
 //      kUpdDots  V = C - H Q;     Hp = V Q^T                  (first pass' update, second's dots)
@@ -357,7 +360,7 @@ __global__ void __launch_bounds__(256) k_panel_reduce(const double* __restrict__
 //    second round's Gram matrix is then I + E with |E| ~ 1e-7, whose Cholesky factor I + X and T2 come
 //    from their series (X = lower(E - X X^T) iterated, T2 = I - X + X^2 - X^3: errors below |E|^4) in four
 //    16 x 16 products; otherwise by the fp64 factorisation.  (fp64 runs at 2 FMAs per clock and SM here,
-//    16 dependent steps of it cost ~20 us: the two rounds took 57 us a panel with both in fp64.)
+//    16 dependent steps of it cost ~20 us: the two rounds took 57 us a panel with both in fp64, 39 now.)
 //    Row k is accepted exactly as the row-by-row kernel would: its norm against what came before it,
 //    sqrt(pivot), > tau ||c_k||.  A pivot taken from G in fp64 is only known to ~1e-14 ||v_k||^2, so a
 //    panel with a decision that this could touch (a pivot below 1e-6 ||v_k||^2 that is not certain to

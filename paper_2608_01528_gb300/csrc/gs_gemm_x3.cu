@@ -27,7 +27,10 @@
 // 1125 clk at 128 B/clk against 768 clk of MMA.  Tried: one group of eleven converter warps (3,670 to
 // 4,000 us: every load's latency exposed, and code long enough to miss the instruction cache), one pair
 // of k per lane with four-byte stores (1,785 us), loading A's next K-block before the hand-over
-// (2,000 us: the hand-over's arrive waits for it).
+// (2,000 us: the hand-over's arrive waits for it), B's parts kept in memory and loaded by TMA (1,650 us, for
+// 6 more bytes an entry of the basis).  Timing copies of that form say that no single part holds it: 4 to
+// 17 % less time without A's loads, without the split's arithmetic, without stores, or with a third of the
+// MMAs; the converters issue at 0.33 instructions a clock and sub-partition, two warps each.
 //
 // No workspace and no pass over the operands beforehand: rows that start anywhere are read with plain
 // loads (no TMA), so nothing is allocated and calls on different streams share nothing.
@@ -575,9 +578,8 @@ bool gemm_fp32_on_tensor(const GemmArgs& g, bool simt, int device) {
                        g.k <= 32768 && g.lda <= 1 << 22 &&
                        (g.b_trans ? g.ldb <= 1 << 22 : (double)g.ldb * g.k < 1e9) && g.m > 0 && g.n > 0 && g.batch > 0;
     // times of both kernels, fitted to measured ones: a wave of tiles takes ~0.9 us per K-block and ~6 us
-    // around it (512 x 3001 x 257: 21 us against 35 on the CUDA cores; 3000 x 1000 x 300: 31 / 65; 20,000 x
-    // 777 x 131: 94 / 146; 34,304 x 448 x 62: 70 / 67, not taken); the CUDA-core GEMM runs at 28 to 37
-    // TFLOP/s
+    // around it (512 x 3001 x 257: 21 us against 36 on the CUDA cores; 3000 x 1000 x 300: 32 / 56; 20,000 x
+    // 777 x 131: 95 / 128; 1,300 x 13,823 x 130: 84 / 154); the CUDA-core GEMM runs at 28 to 45 TFLOP/s
     const double simt_us = 2e-6 * g.m * g.n * g.k * g.batch / 30.0;
     if (!takes || simt_us <= 15.0 || !tc_available(device)) return false;
     int sms = 0;

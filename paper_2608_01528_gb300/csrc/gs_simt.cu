@@ -82,8 +82,7 @@ struct ScoreParams {
 // per block (pitch: whole float4s, an odd number of them, so that a float4 from 32 consecutive rows
 // falls in disjoint banks), the warp's row beside it: per codeword r / 4 conflict-free 16-byte reads and
 // as many broadcasts.  Reading R's rows from global memory, a row per lane, took r loads of 32 lines
-// each per codeword (1,024 rows x 40 codewords, r = 40: 8.1 us, now 5; r = 30, M = 22, 10,844 rows: 22.6 us,
-// now 8).  A codebook past 48 KB goes through in chunks; softmax rows are then scored twice.
+// each per codeword (8,000 rows x 16 codewords: 11.1 us, now 6.5; 1,024 x 40: 5.3, now 4.6).  A codebook past 48 KB goes through in chunks; softmax rows are then scored twice.
 __global__ void __launch_bounds__(kCoefWarps * 32) k_scores(const ScoreParams p) {
     extern __shared__ float4 coef_sm[];
     float* Rs = reinterpret_cast<float*>(coef_sm);
@@ -206,7 +205,8 @@ __global__ void __launch_bounds__(kCoefWarps * 32) k_scores(const ScoreParams p)
 // QB x RB products (a lane QB / 4 x RB / 8 of them, 16-byte shared reads without conflicts), the warps'
 // sums meet in shared memory, and the warps score the queries.  Bound by the loads' latency at the usual
 // few hundred queries.  One warp per query read all of Q per query, 4 bytes a lane (2,048 queries of D =
-// 1024, r = 30: 45 us); four queries' products in one warp's registers left few for loads in flight (19).
+// 1024, r = 30: 45 us, now 14; of D = 2560: 103, now 28); four queries' products in one warp's registers left
+// few for loads in flight (19 and 57 us; at 512 queries, r = 10, it was the faster one, 5 us against 8).
 constexpr int kSmallR = 32;
 constexpr int kSmallM = 64;   // codewords kept in shared memory
 constexpr int kSmallKC = 128, kSmallPitch = kSmallKC + 4;
@@ -397,7 +397,8 @@ __device__ __forceinline__ void ld4(const void* p, long long i, int left, bool v
 // One 64 x 64 output tile (rows m0.., columns n0..) of batch b, or of K chunk kz with ksplit;
 // called by every thread of the block.  A thread loads four consecutive elements of each operand per
 // K step (one 16-byte load where rows are aligned), the next step's while the current one is multiplied
-// (two shared buffers, one barrier a step): 1,024 x 40 over K = 8192 in 16 chunks went from 52 to 24 us.
+// (two shared buffers, one barrier a step).  16,384 x 922 -> 10,000: 8,240 us with scalar loads and nothing in
+// flight (37 TFLOP/s), 6,750 us here (45); 1,024 x 40 over K = 8192, summed and scored: 51, now 38.
 template <int TA, int TB, int TC, bool BT, int MT>
 __device__ __forceinline__ void gemm_tile(const GemmArgs& g, long long m0, int n0, int kz,
                                           float (&As)[2][kTK][16 * MT + 4], float (&Bs)[2][kTK][kTN + 4]) {
@@ -530,7 +531,7 @@ __global__ void __launch_bounds__(256, MT == 8 ? 3 : 4) k_gemm(GemmArgs g) {
 // The gated product (gate_xn2): each block takes a run of consecutive 64 x 64 tiles, n fastest, and
 // computes only those whose 64 rows hold a selected row.  It looks at all its rows first (a run spans few
 // row blocks), so with no such row the launch is one round of loads and a barrier (12 us before, with a
-// barrier per tile: 16,384 x 922).
+// barrier per tile: 16,384 x 922; 3.6 now).
 template <int TA, int TB, int TC, bool BT>
 __global__ void __launch_bounds__(256) k_gemm_gated(GemmArgs g, long long per) {
     __shared__ __align__(16) float As[2][kTK][kTM + 4];

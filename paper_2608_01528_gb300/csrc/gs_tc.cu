@@ -197,7 +197,8 @@ __device__ __forceinline__ bool walk_tiles(const CtaRows& cr, Ctl& c, Wait wait,
 // owns (rows [q 128 / ks, (q + 1) 128 / ks)) into q's shared memory; q adds the parts in a fixed order
 // and goes on alone with its rows (GEMM2 over all 128 TMEM lanes, of which its own are read).  Without
 // it a 4,096-query batch ran on 32 of 152 SMs, each streaming its X tile and all of Q: 150 us at D =
-// 8192, r = M = 256 (softmax, scores out) against 58 us on 38 clusters of 4.  Splitting the rows
+// 8192, r = M = 256 (softmax, scores out) against 59 us on 36 clusters of 4 (92 and 50
+// us for raw argmax).  Splitting the rows
 // instead would have every SM stream all of Q (4 MB each, 620 MB of L2 reads).  The exchange reuses the
 // X staging and A stages, after every CTA of the cluster has finished GEMM1 (peer_ready).
 // FULL = false: raw scores with only argmax / maxval out (the large-batch lookup); true: every
