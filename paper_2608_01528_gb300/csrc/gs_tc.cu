@@ -88,6 +88,7 @@ constexpr int kTmemCols = 512;
 constexpr int kMaxKR = 4;            // K-blocks of 64 in r <= 256
 constexpr int kSCol = 256;           // first TMEM column of the score accumulator
 constexpr int kMaxKS = 8;            // CTAs that may share a tile's K range
+constexpr int kSendLd = 36;          // floats between the rows of a sending warp's 32 x 32 scratch
 
 // ----------------------------------------------------------------- work split
 struct TileRange {
@@ -123,6 +124,7 @@ struct PsParams {
     int nh, half_rows, nkr_h[2];  // GEMM2: halves of codewords, K-blocks of R each half needs
     int ks;                 // SPLIT: CTAs of a cluster that share a tile's K range
     int xch_ld;             // SPLIT: floats between exchanged Y rows (npad + 4)
+    int xch_bytes;          // SPLIT: bytes of the exchanged rows (the senders' scratch lies behind them)
     int bs_off;             // bytes from the X staging to the B ring
     int sx, sa, sb;         // ring depths: fp32 X staging, fp16 A, B operand tiles
     int box_rows;           // rows of each X TMA box (>= every tile's rows)
@@ -197,9 +199,8 @@ __device__ __forceinline__ bool walk_tiles(const CtaRows& cr, Ctl& c, Wait wait,
 // owns (rows [q 128 / ks, (q + 1) 128 / ks)) into q's shared memory; q adds the parts in a fixed order
 // and goes on alone with its rows (GEMM2 over all 128 TMEM lanes, of which its own are read).  Without
 // it a 4,096-query batch ran on 32 of 152 SMs, each streaming its X tile and all of Q: 150 us at D =
-// 8192, r = M = 256 (softmax, scores out) against 59 us on 36 clusters of 4 (92 and 50
-// us for raw argmax).  Splitting the rows
-// instead would have every SM stream all of Q (4 MB each, 620 MB of L2 reads).  The exchange reuses the
+// 8192, r = M = 256 (softmax, scores out) against 52 us on 36 clusters of 4 (92 and 46 us for raw
+// argmax).  Splitting the rows instead would have every SM stream all of Q (4 MB each, 620 MB of L2 reads).  The exchange reuses the
 // X staging and A stages, after every CTA of the cluster has finished GEMM1 (peer_ready).
 // FULL = false: raw scores with only argmax / maxval out (the large-batch lookup); true: every
 // mode and output.  A template parameter, so the lookup kernel carries none of the other paths.
@@ -498,19 +499,47 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (warp == 0 && lane < ks) mbar_arrive_cluster(mapa_shared(smem_u32(&c.peer_ready), (uint32_t)lane));
                 if (!__all_sync(0xffffffffu, mbar_wait_cluster(&c.peer_ready, pt, abort_flag, &g_err_tc))) return false;
                 const int src = rank < owner ? rank : rank - 1;
-                const uint32_t dst = mapa_shared(smem_u32(Xs) + 4u * (uint32_t)((src * own_rows + i % own_rows) * p.xch_ld),
-                                                 (uint32_t)owner);
-                for (int jc = 0; jc < p.npad; jc += 16) {
-                    float y[16];
-                    tmem_ld16(ty + (uint32_t)jc, y);
-                    if (!mine) {
+                // 32 columns at a time through this warp's scratch behind the exchanged rows, so that a store
+                // takes 128 contiguous bytes of each of four rows (a row per lane: 32 pieces of 16 bytes,
+                // 5.9 against 4.1 us for 96 rows of 256 columns)
+                float* tile = reinterpret_cast<float*>(Xs + p.xch_bytes) + warp * 32 * kSendLd;
+                const bool none_mine = __ballot_sync(0xffffffffu, mine) == 0u;
+                const int u0 = lane >> 3, c4 = (lane & 7) * 4;  // rows u0 + 4 u of the warp, four columns
+                uint32_t half_dst[2];  // rows u0 of the warp's two halves (which have an owner each at ks = 8)
+                bool half_out[2];
 #pragma unroll
-                        for (int u = 0; u < 4; ++u)
-                            st_cluster_f32x4(dst + 4u * (uint32_t)(jc + 4 * u), y[4 * u], y[4 * u + 1], y[4 * u + 2],
-                                             y[4 * u + 3]);
+                for (int h = 0; h < 2; ++h) {
+                    const int ri = warp * 32 + 16 * h, own = ri / own_rows, from = rank < own ? rank : rank - 1;
+                    half_out[h] = own != rank;
+                    half_dst[h] = mapa_shared(smem_u32(Xs) + 4u * (uint32_t)((from * own_rows + ri % own_rows + u0) * p.xch_ld + c4),
+                                              (uint32_t)own);
+                }
+                const float* sent_from = tile + u0 * kSendLd + c4;
+                if (none_mine || own_rows < 32) {
+                    for (int jc = 0; jc < p.npad; jc += 32) {
+                        const int w = p.npad - jc >= 32 ? 32 : 16;
+                        for (int e = 0; e < w; e += 16) {
+                            float y[16];
+                            tmem_ld16(ty + (uint32_t)(jc + e), y);
+#pragma unroll
+                            for (int j = 0; j < 4; ++j)
+                                *reinterpret_cast<float4*>(tile + lane * kSendLd + e + 4 * j) =
+                                    make_float4(y[4 * j], y[4 * j + 1], y[4 * j + 2], y[4 * j + 3]);
+                        }
+                        __syncwarp();
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) {
+                            const float4 f = *reinterpret_cast<const float4*>(sent_from + 4 * u * kSendLd);
+                            if (half_out[u >> 2] && c4 < w)
+                                st_cluster_f32x4(half_dst[u >> 2] + 4u * (uint32_t)(4 * (u & 3) * p.xch_ld + jc), f.x, f.y,
+                                                 f.z, f.w);
+                        }
+                        __syncwarp();
                     }
                 }
-                if (!mine) st_cluster_f32x4(dst + 4u * (uint32_t)p.npad, xn2, 0.f, 0.f, 0.f);
+                if (!mine)
+                    st_cluster_f32x4(mapa_shared(smem_u32(Xs) + 4u * (uint32_t)((src * own_rows + i % own_rows) * p.xch_ld + p.npad),
+                                                 (uint32_t)owner), xn2, 0.f, 0.f, 0.f);
                 __syncwarp();
                 // one arrival per group of rows of one owner (a release: the lanes' stores come before it)
                 if (!mine && lane % std::min(32, own_rows) == 0)
@@ -647,26 +676,49 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int ic = 0; ic < p.mpad; ic += 16) {
                 float sv[16];
                 scores(ic, sv);
-                if (FULL && p.mode == GS_SCORE_SOFTMAX) {
-                    // online, sixteen at a time: one rescaling exponential per chunk, one per score
-                    float nm = run_max, add = 0.f;
+                if (ic + 16 > p.M) {  // columns past M never win and add nothing
 #pragma unroll
                     for (int j = 0; j < 16; ++j)
-                        if (ic + j < p.M) nm = fmaxf(nm, sv[j]);
+                        if (ic + j >= p.M) sv[j] = -INFINITY;
+                }
+                // the chunk's first largest score by a tree, left before right (one compare after the other
+                // took 4.6 against 2.5 us a tile of 256 scores, 11.2 against 5.8 with the softmax); a NaN never wins
+                float tv[16];
+                int ti[8];
 #pragma unroll
-                    for (int j = 0; j < 16; ++j)
-                        if (ic + j < p.M) add += __expf(sv[j] - nm);
-                    run_sum = run_sum * __expf(run_max - nm) + add;
-                    run_max = nm;
+                for (int j = 0; j < 16; ++j) tv[j] = fmaxf(sv[j], -FLT_MAX);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const bool g = tv[2 * j + 1] > tv[2 * j];
+                    ti[j] = g ? 2 * j + 1 : 2 * j;
+                    tv[j] = g ? tv[2 * j + 1] : tv[2 * j];
                 }
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const int ci = ic + j;
-                    if (ci >= p.M) break;
-                    if (sv[j] > best) {
-                        best = sv[j];
-                        besti = ci;
+                for (int n = 4; n > 0; n >>= 1) {
+#pragma unroll
+                    for (int j = 0; j < n; ++j) {
+                        const bool g = tv[2 * j + 1] > tv[2 * j];
+                        ti[j] = g ? ti[2 * j + 1] : ti[2 * j];
+                        tv[j] = g ? tv[2 * j + 1] : tv[2 * j];
                     }
+                }
+                if (tv[0] > best) {
+                    best = tv[0];
+                    besti = ic + ti[0];
+                }
+                if (FULL && p.mode == GS_SCORE_SOFTMAX) {
+                    // online, sixteen at a time: one rescaling exponential per chunk, one per score
+                    const float nm = best;
+                    float e[16];
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) e[j] = __expf(sv[j] - nm);
+#pragma unroll
+                    for (int n = 8; n > 0; n >>= 1) {
+#pragma unroll
+                        for (int j = 0; j < n; ++j) e[j] += e[j + n];
+                    }
+                    run_sum = run_sum * __expf(run_max - nm) + e[0];
+                    run_max = nm;
                 }
                 if (FULL && p.S && valid && p.mode != GS_SCORE_SOFTMAX) store(ic, sv);
             }
@@ -927,7 +979,8 @@ cudaError_t launch_ps_tc(const gs_basis* h, const float* X, long long N, int ldx
                       CU_TENSOR_MAP_SWIZZLE_NONE))
         return cudaErrorInvalidValue;
     const int xch_ld = h->tc_npad + 4;  // 16 bytes of shift per row: the row-per-thread accesses spread over the banks
-    const size_t xch = ks > 1 ? sizeof(float) * (size_t)(ks - 1) * (kBM / ks) * xch_ld : 0;
+    const size_t xch_rows = ks > 1 ? sizeof(float) * (size_t)(ks - 1) * (kBM / ks) * xch_ld : 0;
+    const size_t xch = ks > 1 ? xch_rows + sizeof(float) * kBM * kSendLd : 0;
     const Rings g = ps_rings(box_rows, xch);
     if (g.sx % kCvtGroups != 0 || g.sa % kCvtGroups != 0) return cudaErrorInvalidConfiguration;
     PsParams p;
@@ -949,6 +1002,7 @@ cudaError_t launch_ps_tc(const gs_basis* h, const float* X, long long N, int ldx
     p.xstage = ps_xstage(box_rows);
     p.ks = ks;
     p.xch_ld = xch_ld;
+    p.xch_bytes = (int)xch_rows;
     p.bs_off = (int)ps_bs_off(g, p.xstage, xch);
     p.s_vec = (uintptr_t)S % 16 == 0 && lds % 4 == 0;
     // one fp16 rounding of a row is accurate for 2^-8 sqrt(D) <= ||x|| <= 2^15; other rows are redone
