@@ -88,7 +88,10 @@ constexpr int kTmemCols = 512;
 constexpr int kMaxKR = 4;            // K-blocks of 64 in r <= 256
 constexpr int kSCol = 256;           // first TMEM column of the score accumulator
 constexpr int kMaxKS = 8;            // CTAs that may share a tile's K range
-constexpr int kSendLd = 36;          // floats between the rows of a sending warp's 32 x 32 scratch
+constexpr int kSendLd = 36;          // SPLIT: floats between the rows of a sending warp's 32 x 32 scratch
+constexpr int kTailRoles = 1 + kCvtGroups;            // SPLIT: warps of a lane quadrant that share its columns
+constexpr int kTailWarps = kEpiWarps * kTailRoles;    // SPLIT: warps that share the rows to be scored
+static_assert(kCvtGroupWarps == 4, "every converter group has a warp in each lane quadrant");
 
 // ----------------------------------------------------------------- work split
 struct TileRange {
@@ -124,7 +127,8 @@ struct PsParams {
     int nh, half_rows, nkr_h[2];  // GEMM2: halves of codewords, K-blocks of R each half needs
     int ks;                 // SPLIT: CTAs of a cluster that share a tile's K range
     int xch_ld;             // SPLIT: floats between exchanged Y rows (npad + 4)
-    int xch_bytes;          // SPLIT: bytes of the exchanged rows (the senders' scratch lies behind them)
+    int send_off;           // SPLIT: the senders' scratch, behind the exchanged rows and the rows to be scored, then ||x||
+    int s_ld;               // SPLIT: floats between the rows to be scored (mpad + 4)
     int bs_off;             // bytes from the X staging to the B ring
     int sx, sa, sb;         // ring depths: fp32 X staging, fp16 A, B operand tiles
     int box_rows;           // rows of each X TMA box (>= every tile's rows)
@@ -151,6 +155,7 @@ struct Ctl {
     uint64_t xn_full[2], xn_empty[2];
     uint64_t dec_full[2];     // redo decision of regular tile t published in slot t % 2
     uint64_t peer_ready, xch_full;  // SPLIT: every CTA's GEMM1 is done; the peers' parts of my rows are here
+    uint64_t sent_full, rows_full, tail_done;  // SPLIT: other owners' lanes are sent; S is in shared memory; scored
     uint64_t mma_done;
     float xn[2][kBM];  // ||x||^2 per row, both converter groups add into it
     int8_t rsc[2][kBM];      // per-row exponent s of the redo's scale 2^s, for the tile in that slot
@@ -169,6 +174,41 @@ __device__ __forceinline__ float pow2f(int k) { return __int_as_float((127 + k) 
 __device__ __forceinline__ int row_scale_exp(float xn2) {
     if (!(xn2 > 0.f) || !(xn2 <= FLT_MAX)) return 0;
     return 14 - (ilogbf(xn2) >> 1);  // ilogbf(xn2) >> 1 = floor(log2 ||x||)
+}
+
+// one fp16 rounding of x is accurate when every element is inside fp16's range
+// (||x|| <= 2^15) and the row's mass is far above its subnormals (||x|| >= 2^-8
+// sqrt(D): the subnormals' absolute errors, at most 2^-25 each, then add at most
+// 2^-19 ||x|| to the error of <x, q_j>); any other nonzero row has its tile redone
+// with an exact power-of-two scale (a norm that is not a number keeps scale 1)
+__device__ __forceinline__ bool out_of_range(float xn2, const PsParams& p) {
+    return xn2 > 0.f && !(xn2 >= p.xn2_lo && xn2 <= p.xn2_hi);
+}
+
+// w (16 or 32) columns of Y at TMEM address ty, split in place: a chunk of 16 fp32 columns -> 8 columns of
+// packed bf16(Y) + 8 columns of packed bf16(Y - bf16(Y)).
+__device__ __forceinline__ void split_y(uint32_t ty, int w, const float (&y)[32]) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        if (h * 16 >= w) break;
+        uint32_t hl[16];  // 8 columns of packed hi, then 8 of packed lo
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const float a = y[16 * h + 2 * j], b = y[16 * h + 2 * j + 1];
+            const float ah = __bfloat162float(__float2bfloat16_rn(a));
+            const float bh = __bfloat162float(__float2bfloat16_rn(b));
+            hl[j] = pack_bf16(ah, bh);
+            hl[8 + j] = pack_bf16(a - ah, b - bh);
+        }
+        tmem_st16(ty + (uint32_t)(16 * h), hl);
+    }
+}
+
+// Largest value over the warp's lanes (no NaN among them).
+__device__ __forceinline__ float warp_max(float v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
 }
 
 // Processing order of a CTA's tiles: regular tile t, and once tile t + 1 has been handed on, the
@@ -199,9 +239,11 @@ __device__ __forceinline__ bool walk_tiles(const CtaRows& cr, Ctl& c, Wait wait,
 // owns (rows [q 128 / ks, (q + 1) 128 / ks)) into q's shared memory; q adds the parts in a fixed order
 // and goes on alone with its rows (GEMM2 over all 128 TMEM lanes, of which its own are read).  Without
 // it a 4,096-query batch ran on 32 of 152 SMs, each streaming its X tile and all of Q: 150 us at D =
-// 8192, r = M = 256 (softmax, scores out) against 52 us on 36 clusters of 4 (92 and 46 us for raw
-// argmax).  Splitting the rows instead would have every SM stream all of Q (4 MB each, 620 MB of L2 reads).  The exchange reuses the
-// X staging and A stages, after every CTA of the cluster has finished GEMM1 (peer_ready).
+// 8192, r = M = 256 (softmax, scores out) against 46.5 us on 36 clusters of 4 (92 and 44 us for raw
+// argmax): 23.5 until GEMM1's last K-block, 1.7 until every CTA is there, 4.1 for the exchange, 3.2 for the
+// split, 2.3 for GEMM2, 2.5 for scores and rows, the rest launch and exit.  Splitting the rows instead would
+// have every SM stream all of Q (4 MB each, 620 MB of L2 reads).  The exchange reuses the X staging and A
+// stages, after every CTA of the cluster has finished GEMM1 (peer_ready).
 // FULL = false: raw scores with only argmax / maxval out (the large-batch lookup); true: every
 // mode and output.  A template parameter, so the lookup kernel carries none of the other paths.
 template <bool FULL, bool SPLIT>
@@ -224,6 +266,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int rank = SPLIT ? (int)cluster_ctarank() : 0;
     const CtaRows cr(p.N, gridDim.x / ks, blockIdx.x / ks);
     const int kb0 = SPLIT ? p.nkb * rank / ks : 0, kb1 = SPLIT ? p.nkb * (rank + 1) / ks : p.nkb;
+    constexpr int kRoles = SPLIT ? kTailRoles : 1;
     const int own_rows = kBM / ks;                                    // rows this CTA carries on with
     const int own_warps = SPLIT ? std::max(1, kEpiWarps / ks) : kEpiWarps;  // epilogue warps that hold them
 
@@ -241,19 +284,22 @@ __global__ void __launch_bounds__(kThreads, 1)
             mbar_init(&c.b_empty[s], 1);
         }
         mbar_init(&c.y_full, 1);
-        for (int k = 0; k < kMaxKR; ++k) mbar_init(&c.ysplit[k], own_warps);
+        for (int k = 0; k < kMaxKR; ++k) mbar_init(&c.ysplit[k], own_warps * kRoles);
         mbar_init(&c.s_full, 1);
-        mbar_init(&c.s_empty, own_warps);
+        mbar_init(&c.s_empty, own_warps * kRoles);
         mbar_init(&c.gemm2_done, 1);
         for (int b = 0; b < 2; ++b) {
             mbar_init(&c.xn_full[b], kCvtWarps);
             mbar_init(&c.xn_empty[b], kEpiWarps);
-            mbar_init(&c.dec_full[b], SPLIT ? ks * own_warps : kEpiWarps);
+            mbar_init(&c.dec_full[b], SPLIT ? ks * own_warps * kRoles : kEpiWarps);
             for (int w = 0; w < kMaxKS; ++w) c.redo[b][w] = 0;
         }
         if (SPLIT) {
             mbar_init(&c.peer_ready, ks);
             mbar_init(&c.xch_full, (ks - 1) * own_warps);
+            mbar_init(&c.sent_full, own_warps);
+            mbar_init(&c.rows_full, own_warps * kRoles);
+            mbar_init(&c.tail_done, kTailWarps);
         }
         mbar_init(&c.mma_done, 1);
         c.abort_flag = 0;
@@ -280,6 +326,247 @@ __global__ void __launch_bounds__(kThreads, 1)
                      : wait_warp(bar, par);
     };
 
+    // SPLIT: what follows GEMM1 of a tile, on the epilogue's and the converters' twelve warps.  Three warps
+    // (`role`) share a lane quadrant: the first sends the rows that peers own, then all three add the
+    // peers' parts of this CTA's own rows and split them for GEMM2, column chunks in turn.  S goes through shared memory, from
+    // which every warp (`wi`) scores whole rows: the own rows are 32 TMEM lanes at ks = 4, so that one
+    // scheduler's warps did all the arithmetic (9.7 us for 32 rows of 256 scores with the softmax against 1.9),
+    // and the rows left 16 bytes at a time.
+    auto split_tail = [&](int role, int qd, int wi, int t, bool redo, int q) {
+        const uint32_t pt = (uint32_t)q & 1u;
+        const int b = q & 1;
+        const int i = qd * 32 + lane;  // row within the tile = TMEM lane
+        const uint32_t ty = tmem + ((uint32_t)(qd * 32) << 16), ts = ty + kSCol;
+        const TileRange tr = cr.tile(t);
+        const int owner = i / own_rows;  // the CTA that carries on with this row
+        const bool mine = owner == rank;
+        float* fin = reinterpret_cast<float*>(Xs + p.send_off) + kBM * kSendLd;  // ||x|| per row
+        float* rows = reinterpret_cast<float*>(Xs);  // S of the own rows, once their parts are read
+        if (!wait_warp(&c.y_full, pt)) return false;
+        tc_fence_after();
+        float xn2 = 0.f;
+        if (role == 0) {
+            if (!wait_warp(&c.xn_full[b], (uint32_t)(q >> 1) & 1u)) return false;
+            xn2 = c.xn[b][i];
+            c.xn[b][i] = 0.f;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&c.xn_empty[b]);
+            // the peers may write over this CTA's X and A stages, and it over theirs
+            if (qd == 0 && lane < ks) mbar_arrive_cluster(mapa_shared(smem_u32(&c.peer_ready), (uint32_t)lane));
+        }
+        if (!__all_sync(0xffffffffu, mbar_wait_cluster(&c.peer_ready, pt, abort_flag, &g_err_tc))) return false;
+        const unsigned own_lanes = __ballot_sync(0xffffffffu, mine);
+        if (role == 0 && own_lanes != 0xffffffffu) {
+            // 32 columns at a time through this warp's scratch, so that a store takes 128 contiguous bytes of
+            // each of four rows: 4.1 us for 96 rows of 256 columns, 24 bytes/ns, which is what the SM-to-SM
+            // network carries (5.9 with a row per lane, 5.1 with 64 bytes of a row from three warps)
+            float* tile = reinterpret_cast<float*>(Xs + p.send_off) + qd * 32 * kSendLd;
+            const int u0 = lane >> 3, c4 = (lane & 7) * 4;  // rows u0 + 4 u of the warp, four columns
+            uint32_t half_dst[2];  // rows u0 of the warp's two halves (which have an owner each at ks = 8)
+            bool half_out[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int ri = qd * 32 + 16 * h, own = ri / own_rows, from = rank < own ? rank : rank - 1;
+                half_out[h] = own != rank;
+                half_dst[h] = mapa_shared(smem_u32(Xs) + 4u * (uint32_t)((from * own_rows + ri % own_rows + u0) * p.xch_ld + c4),
+                                          (uint32_t)own);
+            }
+            const float* sent_from = tile + u0 * kSendLd + c4;
+            for (int jc = 0; jc < p.npad; jc += 32) {
+                const int w = p.npad - jc >= 32 ? 32 : 16;
+                for (int e = 0; e < w; e += 16) {
+                    float y[16];
+                    tmem_ld16(ty + (uint32_t)(jc + e), y);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        *reinterpret_cast<float4*>(tile + lane * kSendLd + e + 4 * j) =
+                            make_float4(y[4 * j], y[4 * j + 1], y[4 * j + 2], y[4 * j + 3]);
+                }
+                __syncwarp();
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const float4 f = *reinterpret_cast<const float4*>(sent_from + 4 * u * kSendLd);
+                    if (half_out[u >> 2] && c4 < w)
+                        st_cluster_f32x4(half_dst[u >> 2] + 4u * (uint32_t)(4 * (u & 3) * p.xch_ld + jc), f.x, f.y, f.z,
+                                         f.w);
+                }
+                __syncwarp();
+            }
+            const int src = rank < owner ? rank : rank - 1;
+            if (!mine)
+                st_cluster_f32x4(mapa_shared(smem_u32(Xs) + 4u * (uint32_t)((src * own_rows + i % own_rows) * p.xch_ld + p.npad),
+                                             (uint32_t)owner),
+                                 xn2, 0.f, 0.f, 0.f);
+            __syncwarp();
+            // one arrival per group of rows of one owner (a release: the lanes' stores come before it)
+            if (!mine && lane % std::min(32, own_rows) == 0)
+                mbar_arrive_cluster(mapa_shared(smem_u32(&c.xch_full), (uint32_t)owner));
+        }
+        if (own_lanes != 0u) {
+            if (own_rows < 32) {  // the split overwrites the other owners' lanes too, which role 0 sends
+                tc_fence_before();
+                if (role == 0 && lane == 0) mbar_arrive(&c.sent_full);
+                if (!wait_warp(&c.sent_full, pt)) return false;
+                tc_fence_after();
+            }
+            if (!__all_sync(0xffffffffu, mbar_wait_cluster(&c.xch_full, pt, abort_flag, &g_err_tc))) return false;
+            // this row's parts from the peers, in CTA order
+            const float* parts = reinterpret_cast<const float*>(Xs) + (size_t)(i % own_rows) * p.xch_ld;
+            // a redone tile ran on x 2^s: Y and ||x|| come back multiplied by 2^s
+            const float unscale = redo ? pow2f(-c.rsc[t & 1][i]) : 1.f;
+            if (role == 0) {
+                if (mine) {
+                    for (int u = 0; u < ks - 1; ++u) xn2 += parts[(size_t)u * own_rows * p.xch_ld + p.npad];
+                    fin[i] = sqrtf(xn2) * unscale;
+                }
+                if (!redo) {  // the redo's data, to every CTA of the cluster (this one among them)
+                    const int slot = t & 1;
+                    const uint32_t e = (uint32_t)(uint8_t)(int8_t)row_scale_exp(xn2);
+                    const unsigned any = __ballot_sync(0xffffffffu, mine && out_of_range(xn2, p));
+                    const uint32_t a_rsc = smem_u32(&c.rsc[slot][i]);
+                    const uint32_t a_redo = smem_u32(&c.redo[slot][own_warps > 1 ? qd : rank]);
+                    for (int d = 0; d < ks; ++d)
+                        if (mine) st_cluster_u8(mapa_shared(a_rsc, (uint32_t)d), e);
+                    if (lane < ks) st_cluster_u32(mapa_shared(a_redo, (uint32_t)lane), any != 0u);
+                }
+            }
+            for (int jc = 0; jc < p.npad; jc += 32) {
+                if ((jc >> 5) % kRoles == role) {
+                    const int w = p.npad - jc >= 32 ? 32 : 16;
+                    float y[32];
+                    if (w == 32)
+                        tmem_ld32(ty + (uint32_t)jc, y);
+                    else
+                        tmem_ld16(ty + (uint32_t)jc, y);
+                    if (mine) {
+                        for (int u = 0; u < ks - 1; ++u) {
+                            const float4* src = reinterpret_cast<const float4*>(parts + (size_t)u * own_rows * p.xch_ld + jc);
+#pragma unroll
+                            for (int j = 0; j < 8; ++j) {
+                                if (4 * j >= w) break;
+                                const float4 f = src[j];
+                                y[4 * j] += f.x;
+                                y[4 * j + 1] += f.y;
+                                y[4 * j + 2] += f.z;
+                                y[4 * j + 3] += f.w;
+                            }
+                        }
+                    }
+                    if (redo) {
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) y[j] *= unscale;
+                    }
+                    if (FULL && p.Y && mine && i < tr.nrows) {
+                        float* dst = p.Y + (size_t)(tr.row0 + i) * p.ldy + jc;
+#pragma unroll
+                        for (int j = 0; j < 32; ++j)
+                            if (j < w && jc + j < p.r) dst[j] = y[j];
+                    }
+                    split_y(ty + (uint32_t)jc, w, y);
+                }
+                if (((jc + 32) & 63) == 0 || jc + 32 >= p.npad) {  // this role's part of K-block jc / 64 is split
+                    tmem_wait_st();
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&c.ysplit[jc >> 6]);
+                }
+            }
+            // the parts are read and the redo's data sent
+            if (!redo && lane < ks) mbar_arrive_cluster(mapa_shared(smem_u32(&c.dec_full[t & 1]), (uint32_t)lane));
+            if (!wait_warp(&c.s_full, pt)) return false;
+            tc_fence_after();
+            for (int ic = 16 * role; ic < p.mpad; ic += 16 * kRoles) {
+                float sv[16];
+                tmem_ld16(ts + (uint32_t)ic, sv);
+                if (p.nkr_h[ic >= p.half_rows ? 1 : 0] == 0) {  // a half with no nonzero R: S = 0
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) sv[j] = 0.f;
+                }
+                if (mine) {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        *reinterpret_cast<float4*>(rows + (i % own_rows) * p.s_ld + ic + 4 * j) =
+                            make_float4(sv[4 * j], sv[4 * j + 1], sv[4 * j + 2], sv[4 * j + 3]);
+                }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) {
+                mbar_arrive(&c.s_empty);
+                mbar_arrive(&c.rows_full);
+            }
+        }
+        if (!wait_warp(&c.rows_full, pt)) return false;
+        const bool softmax = FULL && p.mode == GS_SCORE_SOFTMAX;
+        for (int il = wi; il < own_rows && rank * own_rows + il < tr.nrows; il += kTailWarps) {
+            const long long row = tr.row0 + rank * own_rows + il;
+            float v[8];  // columns 4 lane + j and 128 + 4 lane + j
+            float best = -FLT_MAX;
+            int besti = 0;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int col = 128 * h + 4 * lane;
+                const float4 f = col < p.mpad ? *reinterpret_cast<const float4*>(rows + il * p.s_ld + col)
+                                              : make_float4(0.f, 0.f, 0.f, 0.f);
+                v[4 * h] = f.x;
+                v[4 * h + 1] = f.y;
+                v[4 * h + 2] = f.z;
+                v[4 * h + 3] = f.w;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    float& x = v[4 * h + j];
+                    x *= p.scale;
+                    if (FULL && p.mode == GS_SCORE_COSINE) {
+                        const float den = col + j < p.M ? fin[rank * own_rows + il] * p.cnorm[col + j] : 0.f;
+                        x = den > 0.f ? x / den : 0.f;
+                    }
+                    if (col + j >= p.M) x = -INFINITY;  // columns past M never win and add nothing
+                    if (x > best) {
+                        best = x;
+                        besti = col + j;
+                    }
+                }
+            }
+            const float top = warp_max(best);
+            // the first of equal scores, and entry 0 where none is above the type's lowest value
+            const int idx = top > -FLT_MAX ? (int)__reduce_min_sync(0xffffffffu, best == top ? (unsigned)besti : 0x7fffffffu) : 0;
+            float outmax = top;
+            if (softmax) {
+                float sum = 0.f;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    v[j] = __expf(v[j] - top);
+                    sum += v[j];
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+                const float inv = 1.f / sum;
+                outmax = __expf(top - top) * inv;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) v[j] *= inv;
+            }
+            if (FULL && p.S) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int col = 128 * h + 4 * lane;
+                    float* dst = p.S + (size_t)row * p.lds + col;
+                    if (p.s_vec && col + 4 <= p.M) {
+                        *reinterpret_cast<float4*>(dst) = make_float4(v[4 * h], v[4 * h + 1], v[4 * h + 2], v[4 * h + 3]);
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            if (col + j < p.M) dst[j] = v[4 * h + j];
+                    }
+                }
+            }
+            if (lane == 0 && p.argmax) p.argmax[row] = idx;
+            if (lane == 0 && p.maxval) p.maxval[row] = outmax;
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&c.tail_done);
+        return true;
+    };
+
     if (warp == kXWarp) {
         // ------------------------------------------------------------- X tiles via TMA
         if (lane == 0) {
@@ -287,9 +574,12 @@ __global__ void __launch_bounds__(kThreads, 1)
             const uint32_t bytes = (uint32_t)p.box_rows * kBK * 4;
             int it = 0;
             RingPos xs;
-            walk_tiles(cr, c, dec_1t, [&](int t, bool redo, int) {
+            walk_tiles(cr, c, dec_1t, [&](int t, bool redo, int q) {
                 const TileRange tr = cr.tile(t);
-                if (SPLIT && redo) fence_proxy_async();  // the exchanged rows lay where X lands again
+                if (SPLIT && redo) {  // the exchanged rows and the scores lay where X lands again
+                    if (!wait_1t(&c.tail_done, (uint32_t)(q - 1) & 1u)) return false;
+                    fence_proxy_async();
+                }
                 for (int kb = kb0; kb < kb1; ++kb, ++it, xs.next(p.sx)) {
                     if (!wait_1t(&c.x_empty[xs.idx], xs.phase ^ 1u)) return false;
                     mbar_arrive_expect_tx(&c.x_full[xs.idx], bytes);
@@ -468,7 +758,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (lane == 0) mbar_arrive(&c.xn_full[b]);
 #pragma unroll
             for (int u = 0; u < kCvtRows; ++u) nrm[u] = 0.f;
-            return true;
+            return SPLIT ? split_tail(1 + g, warp & 3, kEpiWarps + warp - kCvt0, t, redo, q) : true;
         });
         // only a redone row can still leave fp16's range (a norm that is not a finite fp32 number)
         if (amax > 65504.f) atomicOr(&g_err_tc, GS_DEV_ERR_RANGE);
@@ -478,78 +768,14 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
         const uint32_t ty = tmem + lane_base, ts = tmem + lane_base + kSCol;
         walk_tiles(cr, c, dec_warp, [&](int t, bool redo, int q) {
+            if (SPLIT) return split_tail(0, warp, warp, t, redo, q);
             const uint32_t pt = (uint32_t)q & 1u;
             const int b = q & 1;
             if (!wait_warp(&c.y_full, pt)) return false;
             tc_fence_after();
             const TileRange tr = cr.tile(t);
             const long long row = tr.row0 + i;
-            const int owner = SPLIT ? i / own_rows : 0;  // the CTA that carries on with this row
-            const bool mine = owner == rank;
-            const bool valid = i < tr.nrows && mine;
-            float xn2 = 0.f;
-            const float* parts = nullptr;  // SPLIT: this row's parts from the peers, in CTA order
-            if (SPLIT) {
-                if (!wait_warp(&c.xn_full[b], (uint32_t)(q >> 1) & 1u)) return false;
-                xn2 = c.xn[b][i];
-                c.xn[b][i] = 0.f;
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&c.xn_empty[b]);
-                // the peers may write over this CTA's X and A stages, and it over theirs
-                if (warp == 0 && lane < ks) mbar_arrive_cluster(mapa_shared(smem_u32(&c.peer_ready), (uint32_t)lane));
-                if (!__all_sync(0xffffffffu, mbar_wait_cluster(&c.peer_ready, pt, abort_flag, &g_err_tc))) return false;
-                const int src = rank < owner ? rank : rank - 1;
-                // 32 columns at a time through this warp's scratch behind the exchanged rows, so that a store
-                // takes 128 contiguous bytes of each of four rows (a row per lane: 32 pieces of 16 bytes,
-                // 5.9 against 4.1 us for 96 rows of 256 columns)
-                float* tile = reinterpret_cast<float*>(Xs + p.xch_bytes) + warp * 32 * kSendLd;
-                const bool none_mine = __ballot_sync(0xffffffffu, mine) == 0u;
-                const int u0 = lane >> 3, c4 = (lane & 7) * 4;  // rows u0 + 4 u of the warp, four columns
-                uint32_t half_dst[2];  // rows u0 of the warp's two halves (which have an owner each at ks = 8)
-                bool half_out[2];
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int ri = warp * 32 + 16 * h, own = ri / own_rows, from = rank < own ? rank : rank - 1;
-                    half_out[h] = own != rank;
-                    half_dst[h] = mapa_shared(smem_u32(Xs) + 4u * (uint32_t)((from * own_rows + ri % own_rows + u0) * p.xch_ld + c4),
-                                              (uint32_t)own);
-                }
-                const float* sent_from = tile + u0 * kSendLd + c4;
-                if (none_mine || own_rows < 32) {
-                    for (int jc = 0; jc < p.npad; jc += 32) {
-                        const int w = p.npad - jc >= 32 ? 32 : 16;
-                        for (int e = 0; e < w; e += 16) {
-                            float y[16];
-                            tmem_ld16(ty + (uint32_t)(jc + e), y);
-#pragma unroll
-                            for (int j = 0; j < 4; ++j)
-                                *reinterpret_cast<float4*>(tile + lane * kSendLd + e + 4 * j) =
-                                    make_float4(y[4 * j], y[4 * j + 1], y[4 * j + 2], y[4 * j + 3]);
-                        }
-                        __syncwarp();
-#pragma unroll
-                        for (int u = 0; u < 8; ++u) {
-                            const float4 f = *reinterpret_cast<const float4*>(sent_from + 4 * u * kSendLd);
-                            if (half_out[u >> 2] && c4 < w)
-                                st_cluster_f32x4(half_dst[u >> 2] + 4u * (uint32_t)(4 * (u & 3) * p.xch_ld + jc), f.x, f.y,
-                                                 f.z, f.w);
-                        }
-                        __syncwarp();
-                    }
-                }
-                if (!mine)
-                    st_cluster_f32x4(mapa_shared(smem_u32(Xs) + 4u * (uint32_t)((src * own_rows + i % own_rows) * p.xch_ld + p.npad),
-                                                 (uint32_t)owner), xn2, 0.f, 0.f, 0.f);
-                __syncwarp();
-                // one arrival per group of rows of one owner (a release: the lanes' stores come before it)
-                if (!mine && lane % std::min(32, own_rows) == 0)
-                    mbar_arrive_cluster(mapa_shared(smem_u32(&c.xch_full), (uint32_t)owner));
-                if (__ballot_sync(0xffffffffu, mine) == 0u) return true;  // none of this warp's rows stay here
-                if (!__all_sync(0xffffffffu, mbar_wait_cluster(&c.xch_full, pt, abort_flag, &g_err_tc))) return false;
-                parts = reinterpret_cast<const float*>(Xs) + (size_t)(i % own_rows) * p.xch_ld;
-                if (mine)
-                    for (int u = 0; u < ks - 1; ++u) xn2 += parts[(size_t)u * own_rows * p.xch_ld + p.npad];
-            }
+            const bool valid = i < tr.nrows;
             // a redone tile ran on x 2^s: Y and ||x|| come back multiplied by 2^s
             const float unscale = redo ? pow2f(-c.rsc[t & 1][i]) : 1.f;
             // split Y in place: chunk of 16 fp32 columns -> 8 columns bf16(Y) + 8 columns
@@ -563,20 +789,6 @@ __global__ void __launch_bounds__(kThreads, 1)
                     tmem_ld32(ty + (uint32_t)jc, y);
                 else
                     tmem_ld16(ty + (uint32_t)jc, y);
-                if (SPLIT && mine) {
-                    for (int u = 0; u < ks - 1; ++u) {
-                        const float4* src = reinterpret_cast<const float4*>(parts + (size_t)u * own_rows * p.xch_ld + jc);
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) {
-                            if (4 * j >= w) break;
-                            const float4 f = src[j];
-                            y[4 * j] += f.x;
-                            y[4 * j + 1] += f.y;
-                            y[4 * j + 2] += f.z;
-                            y[4 * j + 3] += f.w;
-                        }
-                    }
-                }
                 if (redo) {
 #pragma unroll
                     for (int j = 0; j < 32; ++j) y[j] *= unscale;
@@ -587,20 +799,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     for (int j = 0; j < 32; ++j)
                         if (j < w && jc + j < p.r) dst[j] = y[j];
                 }
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    if (h * 16 >= w) break;
-                    uint32_t hl[16];  // 8 columns of packed hi, then 8 of packed lo
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const float a = y[16 * h + 2 * j], bb = y[16 * h + 2 * j + 1];
-                        const float ah = __bfloat162float(__float2bfloat16_rn(a));
-                        const float bh = __bfloat162float(__float2bfloat16_rn(bb));
-                        hl[j] = pack_bf16(ah, bh);
-                        hl[8 + j] = pack_bf16(a - ah, bb - bh);
-                    }
-                    tmem_st16(ty + (uint32_t)(jc + 16 * h), hl);
-                }
+                split_y(ty + (uint32_t)jc, w, y);
                 if (((jc + 32) & 63) == 0 || jc + 32 >= p.npad) {  // K-block jc / 64 is split
                     tmem_wait_st();
                     tc_fence_before();
@@ -608,38 +807,19 @@ __global__ void __launch_bounds__(kThreads, 1)
                     if (lane == 0) mbar_arrive(&c.ysplit[jc >> 6]);
                 }
             }
-            if (!SPLIT) {
-                if (!wait_warp(&c.xn_full[b], (uint32_t)(q >> 1) & 1u)) return false;
-                xn2 = c.xn[b][i];
-                c.xn[b][i] = 0.f;  // ready for the tile after next (both groups add into it)
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&c.xn_empty[b]);
-            }
+            if (!wait_warp(&c.xn_full[b], (uint32_t)(q >> 1) & 1u)) return false;
+            const float xn2 = c.xn[b][i];
+            c.xn[b][i] = 0.f;  // ready for the tile after next (both groups add into it)
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&c.xn_empty[b]);
             const float xnorm = sqrtf(xn2) * unscale;
             if (!redo) {
-                // one fp16 rounding of x is accurate when every element is inside fp16's range
-                // (||x|| <= 2^15) and the row's mass is far above its subnormals (||x|| >= 2^-8
-                // sqrt(D): the subnormals' absolute errors, at most 2^-25 each, then add at most
-                // 2^-19 ||x|| to the error of <x, q_j>); any other nonzero row has its tile redone
-                // with an exact power-of-two scale (a norm that is not a number keeps scale 1)
-                const bool bad = mine && xn2 > 0.f && !(xn2 >= p.xn2_lo && xn2 <= p.xn2_hi);
                 const int slot = t & 1;
-                const int8_t e = (int8_t)row_scale_exp(xn2);
-                const unsigned any = __ballot_sync(0xffffffffu, bad);
-                if (SPLIT) {  // to every CTA of the cluster (this one among them)
-                    const uint32_t a_rsc = smem_u32(&c.rsc[slot][i]);
-                    const uint32_t a_redo = smem_u32(&c.redo[slot][own_warps > 1 ? warp : rank]);
-                    for (int d = 0; d < ks; ++d)
-                        if (mine) st_cluster_u8(mapa_shared(a_rsc, (uint32_t)d), (uint32_t)(uint8_t)e);
-                    if (lane < ks) st_cluster_u32(mapa_shared(a_redo, (uint32_t)lane), any != 0u);
-                    __syncwarp();
-                    if (lane < ks) mbar_arrive_cluster(mapa_shared(smem_u32(&c.dec_full[slot]), (uint32_t)lane));
-                } else {
-                    c.rsc[slot][i] = e;
-                    if (lane == 0) c.redo[slot][warp] = any != 0u;
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&c.dec_full[slot]);
-                }
+                c.rsc[slot][i] = (int8_t)row_scale_exp(xn2);
+                const unsigned any = __ballot_sync(0xffffffffu, out_of_range(xn2, p));
+                if (lane == 0) c.redo[slot][warp] = any != 0u;
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&c.dec_full[slot]);
             }
             if (!wait_warp(&c.s_full, pt)) return false;
             tc_fence_after();
@@ -800,7 +980,8 @@ constexpr size_t kSmemCap = 227 * 1024;
 // bytes between fp32 X staging tiles of `box_rows` rows (SW128 operand areas follow: 1 KB aligned)
 int ps_xstage(int box_rows) { return (box_rows * kBK * 4 + 1023) / 1024 * 1024; }
 
-// xch: bytes of the exchanged rows (0: no K split), which share the X staging's and A stages' place
+// xch: bytes of the exchanged rows, the senders' scratch and the norms (0: no K split), which share the X
+// staging's and A stages' place
 size_t ps_bs_off(Rings g, int xstage, size_t xch) {
     return std::max((size_t)g.sx * xstage + (size_t)g.sa * kAStageBytes, (xch + 1023) / 1024 * 1024);
 }
@@ -962,9 +1143,9 @@ cudaError_t launch_ps_tc(const gs_basis* h, const float* X, long long N, int ldx
     const long long tiles = (N + kBM - 1) / kBM;
     // Fewer tiles than half the SMs: clusters of ks CTAs share each tile's K range, as many clusters as
     // the GPU holds (their rows even out).  A K-block takes a CTA ~0.65 us, the exchange and what only the
-    // row's owner does after it up to ~20 us at r = M = 256 (10 us at 32), so the K-blocks saved have
-    // to be worth 20 us.  Measured at r = M = 256, 4,096 queries: D = 4096: 39 us (50 without), 8192: 50
-    // (92), 16,384: 70; D = 2048 is left alone.
+    // row's owner does after it ~15 us at r = M = 256, so the K-blocks saved have to be worth 20 us.
+    // Measured at r = M = 256, 4,096 queries: D = 4096: 33 us (50 without), 8192: 44 (92), 16,384: 65;
+    // D = 2048 is left alone.
     const int nkb = (h->D + kBK - 1) / kBK;
     int ks = 1, clusters = 0;
     for (int i = 0; i < 3; ++i)
@@ -979,8 +1160,9 @@ cudaError_t launch_ps_tc(const gs_basis* h, const float* X, long long N, int ldx
                       CU_TENSOR_MAP_SWIZZLE_NONE))
         return cudaErrorInvalidValue;
     const int xch_ld = h->tc_npad + 4;  // 16 bytes of shift per row: the row-per-thread accesses spread over the banks
-    const size_t xch_rows = ks > 1 ? sizeof(float) * (size_t)(ks - 1) * (kBM / ks) * xch_ld : 0;
-    const size_t xch = ks > 1 ? xch_rows + sizeof(float) * kBM * kSendLd : 0;
+    const int s_ld = h->tc_mpad + 4;
+    const size_t send_off = sizeof(float) * (size_t)(kBM / ks) * std::max((ks - 1) * xch_ld, s_ld);
+    const size_t xch = ks > 1 ? send_off + sizeof(float) * (kBM * kSendLd + kBM) : 0;
     const Rings g = ps_rings(box_rows, xch);
     if (g.sx % kCvtGroups != 0 || g.sa % kCvtGroups != 0) return cudaErrorInvalidConfiguration;
     PsParams p;
@@ -1002,7 +1184,8 @@ cudaError_t launch_ps_tc(const gs_basis* h, const float* X, long long N, int ldx
     p.xstage = ps_xstage(box_rows);
     p.ks = ks;
     p.xch_ld = xch_ld;
-    p.xch_bytes = (int)xch_rows;
+    p.send_off = (int)send_off;
+    p.s_ld = s_ld;
     p.bs_off = (int)ps_bs_off(g, p.xstage, xch);
     p.s_vec = (uintptr_t)S % 16 == 0 && lds % 4 == 0;
     // one fp16 rounding of a row is accurate for 2^-8 sqrt(D) <= ||x|| <= 2^15; other rows are redone

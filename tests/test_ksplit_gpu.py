@@ -84,3 +84,31 @@ def test_unaligned_score_rows(gs):
     out = gs.project_similarity(b, X, mode="softmax", scale=8 / 4096, want_S=True, out={"S": S})
     gs.stream_status()
     assert float((out["S"].sum(1) - 1).abs().max()) <= 1e-5
+
+
+# clusters of 8, 4 and 2, no split: more codewords than the basis has rows, so that the scores of a row
+# take more shared memory than its coefficients
+@pytest.mark.parametrize("N", [500, 3000, 6000, 20000])
+def test_zero_and_nan_rows(gs, N):
+    """A zero query ties everywhere: the first entry wins.  A NaN query wins nowhere: entry 0, the lowest value."""
+    rng = np.random.default_rng(N)
+    B = torch.from_numpy((rng.integers(0, 2, size=(20, 4160)) * 2 - 1).astype(np.float32)).cuda()
+    mix = torch.from_numpy(rng.integers(-1, 2, size=(250, 20)).astype(np.float32)).cuda()
+    mix[:20] = torch.eye(20)
+    C = mix @ B  # small whole numbers: exact in fp32
+    X = torch.from_numpy(rng.standard_normal((N, 4160)).astype(np.float32)).cuda()
+    zero, nan = [0, 129, N - 1], [1, 131, N - 2]
+    X[zero] = 0
+    X[nan, 7] = float("nan")
+    b = gs.build_basis(C)
+    assert b.r == 20
+    out = gs.project_similarity(b, X, path="tensor", want_S=True)
+    gs.stream_status()
+    assert bool((out["argmax"][zero + nan] == 0).all()) and bool((out["maxval"][zero] == 0).all())
+    assert bool((out["maxval"][nan] == torch.finfo(torch.float32).min).all())
+    keep = torch.ones(N, dtype=torch.bool, device="cuda")
+    keep[nan] = False
+    S = X[keep].double() @ C.double().T
+    tol = TOL * X[keep].double().norm(dim=1)[:, None] * C.double().norm(dim=1)[None, :]
+    assert bool(((out["S"][keep].double() - S).abs() <= tol).all())
+    assert torch.equal(out["S"][keep].argmax(1), out["argmax"][keep].long())
