@@ -395,7 +395,8 @@ gs_status gs_project_similarity(const gs_basis* h, const float* X, long long N, 
             const long long used = (long long)(scr - h->scratch);
             const long long room = (h->scratch_floats - used) / std::max(1LL, nc * r);
             a.ksplit = (int)std::min<long long>(gemm_ksplit(nc, r, D, h->device), room);
-            a.kpart = a.ksplit > 1 ? scr : nullptr;
+            a.kpart = scr;
+            a.kpart_floats = h->scratch_floats - used;
         }
         cudaError_t e = gs::launch_gemm_fp32(a, simt, h->device, s);
         if (e != cudaSuccess) return from_cuda(e);

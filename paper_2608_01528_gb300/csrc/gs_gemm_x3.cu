@@ -71,6 +71,8 @@ struct X3Params {
     long long lda, ldb, ldc, a_bs, b_bs, c_bs;
     long long m, tiles_m, tiles;
     int n, k, nt, tiles_n, nkb;
+    int k_last;          // K of the last batch plane (a K split's planes are chunks of one product)
+    long long last;      // that plane
     int c_bf16, c_vec;
     float alpha;
     const float* rownorm;
@@ -91,6 +93,7 @@ struct Step {
     const char* A;   // first row of A (in its batch plane), first row or column of B
     const char* B;
     int rows, cols;  // valid rows of A and columns of C in the tile
+    int k;           // K of the tile's plane
 };
 
 template <int TA>
@@ -286,6 +289,7 @@ __global__ void __maxnreg__(96) k_gemm_x3(const __grid_constant__ X3Params p) {
             st.B = (const char*)(p.B + b * p.b_bs + (BT ? (long long)n0 * p.ldb : n0));
             st.rows = (int)(p.m - m0 < kBM ? p.m - m0 : kBM);
             st.cols = p.n - n0 < p.nt ? p.n - n0 : p.nt;
+            st.k = b == p.last ? p.k_last : p.k;
         };
         // to K-block `kb` of tile lt, or into the tiles after it; false past the CTA's last tile
         auto seek = [&]() {
@@ -308,7 +312,7 @@ __global__ void __maxnreg__(96) k_gemm_x3(const __grid_constant__ X3Params p) {
         };
         auto load = [&]() {
             const int k0 = st.kb * kBK, kc = k0 + 8 * cw;  // kc: this warp's eight k of a B stored K x n
-            if (k0 + kBK <= p.k) {
+            if (k0 + kBK <= st.k) {
 #pragma unroll
                 for (int i = 0; i < kSlots; ++i) ld8<TA, VEC>(row_a(i) + (k0 + 8 * ch) * ta_size, va[i]);
 #pragma unroll
@@ -330,18 +334,18 @@ __global__ void __maxnreg__(96) k_gemm_x3(const __grid_constant__ X3Params p) {
                 }
             } else {
 #pragma unroll
-                for (int i = 0; i < kSlots; ++i) ld8_end<TA>(row_a(i), k0 + 8 * ch, p.k, va[i]);
+                for (int i = 0; i < kSlots; ++i) ld8_end<TA>(row_a(i), k0 + 8 * ch, st.k, va[i]);
 #pragma unroll
                 for (int i = 0; i < kSlots; ++i) {
                     if (BT) {
-                        ld8_end<MAT_F32>(row_b(i), k0 + 8 * ch, p.k, vb[i]);
+                        ld8_end<MAT_F32>(row_b(i), k0 + 8 * ch, st.k, vb[i]);
                         continue;
                     }
                     const float* f = reinterpret_cast<const float*>(st.B) + min(32 * i + lane, st.cols - 1);
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
-                        vb[i][u].x = __ldg(f + (size_t)min(kc + 2 * u, p.k - 1) * p.ldb);
-                        vb[i][u].y = __ldg(f + (size_t)min(kc + 2 * u + 1, p.k - 1) * p.ldb);
+                        vb[i][u].x = __ldg(f + (size_t)min(kc + 2 * u, st.k - 1) * p.ldb);
+                        vb[i][u].y = __ldg(f + (size_t)min(kc + 2 * u + 1, st.k - 1) * p.ldb);
                     }
                 }
             }
@@ -481,6 +485,7 @@ __global__ void __maxnreg__(96) k_gemm_x3(const __grid_constant__ X3Params p) {
             if (bad) {  // this thread's outputs again, as plain fp32 dot products in K order
                 const char* Ab = (const char*)p.A + (size_t)(b * p.a_bs) * ta_size;
                 const float* Bb = p.B + b * p.b_bs;
+                const int kend = b == p.last ? p.k_last : p.k;
 #pragma unroll 1
                 for (int e = 0; e < 64; ++e) {
                     const int cl = 64 * half + 32 * (e >> 5) + 8 * ((e >> 3) & 3) + 2 * (lane & 3) + (e & 1);
@@ -489,7 +494,7 @@ __global__ void __maxnreg__(96) k_gemm_x3(const __grid_constant__ X3Params p) {
                     if (cl >= p.nt || col >= p.n || row >= p.m) continue;
                     float g = 0.f;
 #pragma unroll 4
-                    for (int k = 0; k < p.k; ++k)
+                    for (int k = 0; k < kend; ++k)
                         g = fmaf(lda1<TA>(Ab, row * p.lda + k),
                                  __ldg(Bb + (BT ? (long long)col * p.ldb + k : (long long)k * p.ldb + col)), g);
                     g = finish(g, row, col);
@@ -520,7 +525,7 @@ unsigned take_device_error_x3() {
     return v;
 }
 
-static cudaError_t launch_gemm_x3(const GemmArgs& g, int sms, int device, cudaStream_t s) {
+static cudaError_t launch_gemm_x3(const GemmArgs& g, int k_last, int sms, int device, cudaStream_t s) {
     X3Params p;
     p.A = g.A;
     p.B = (const float*)g.B;
@@ -528,6 +533,7 @@ static cudaError_t launch_gemm_x3(const GemmArgs& g, int sms, int device, cudaSt
     p.lda = g.lda, p.ldb = g.ldb, p.ldc = g.ldc;
     p.a_bs = g.a_bstride, p.b_bs = g.b_bstride, p.c_bs = g.c_bstride;
     p.m = g.m, p.n = g.n, p.k = g.k;
+    p.k_last = k_last, p.last = g.batch - 1;
     p.tiles_n = (g.n + kBN - 1) / kBN;
     p.nt = ((g.n + p.tiles_n - 1) / p.tiles_n + 15) / 16 * 16;
     p.tiles_m = (g.m + kBM - 1) / kBM;
@@ -573,7 +579,8 @@ static cudaError_t launch_gemm_x3(const GemmArgs& g, int sms, int device, cudaSt
     return cudaErrorInvalidValue;
 }
 
-bool gemm_fp32_on_tensor(const GemmArgs& g, bool simt, int device) {
+// K chunks for the product on the tensor cores; 0: it stays on the CUDA cores.
+static int x3_ksplit(const GemmArgs& g, bool simt, int device) {
     const bool takes = !simt && g.b_type == MAT_F32 && (g.a_type == MAT_F32 || !g.b_trans) && !g.gate_xn2 && g.k >= 1 &&
                        g.k <= 32768 && g.lda <= 1 << 22 &&
                        (g.b_trans ? g.ldb <= 1 << 22 : (double)g.ldb * g.k < 1e9) && g.m > 0 && g.n > 0 && g.batch > 0;
@@ -581,18 +588,45 @@ bool gemm_fp32_on_tensor(const GemmArgs& g, bool simt, int device) {
     // around it (512 x 3001 x 257: 21 us against 36 on the CUDA cores; 3000 x 1000 x 300: 32 / 56; 20,000 x
     // 777 x 131: 95 / 128; 1,300 x 13,823 x 130: 84 / 154); the CUDA-core GEMM runs at 28 to 45 TFLOP/s
     const double simt_us = 2e-6 * g.m * g.n * g.k * g.batch / 30.0;
-    if (!takes || simt_us <= 15.0 || !tc_available(device)) return false;
+    if (!takes || simt_us <= 15.0 || !tc_available(device)) return 0;
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
     const double tiles = (double)((g.m + kBM - 1) / kBM) * ((g.n + kBN - 1) / kBN) * g.batch;
-    return 8.0 + std::ceil(tiles / std::max(sms, 1)) * (0.9 * ((g.k + kBK - 1) / kBK) + 6.0) < simt_us;
+    const int nkb = (g.k + kBK - 1) / kBK;
+    // few tiles over a deep K: chunks of at least eight K-blocks to partial products in the caller's
+    // workspace, and their sum.  Whole scoring calls: 2,000 x 8192, r = M = 512: 239 -> 150 us; 1,000 x
+    // 4096, 512: 138 -> 74; 300 x 8192, 1,000: 250 -> 102; 500 x 16,384, 256: 125 -> 60
+    const bool may = g.kpart && g.batch == 1 && g.c_type == MAT_F32 && !g.rownorm && !g.colnorm && g.alpha == 1.f;
+    const long long most = may ? std::min<long long>(g.kpart_floats / (g.m * g.n), std::min(32, nkb / 8)) : 1;
+    int best = 0;
+    double best_us = simt_us;
+    for (int ks = 1; ks <= std::max(1LL, most); ++ks) {
+        const double us = 8.0 + std::ceil(tiles * ks / std::max(sms, 1)) * (0.9 * ((nkb + ks - 1) / ks) + 6.0) +
+                          (ks > 1 ? 4.0 + 4e-6 * g.m * g.n * (ks + 1) / 3.0 : 0.0);
+        if (us < best_us) best = ks, best_us = us;
+    }
+    return best;
 }
 
+bool gemm_fp32_on_tensor(const GemmArgs& g, bool simt, int device) { return x3_ksplit(g, simt, device) > 0; }
+
 cudaError_t launch_gemm_fp32(const GemmArgs& g, bool simt, int device, cudaStream_t s) {
-    if (!gemm_fp32_on_tensor(g, simt, device)) return launch_gemm_simt(g, s);
+    const int ks = x3_ksplit(g, simt, device);
+    if (ks == 0) return launch_gemm_simt(g, s);
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
-    return launch_gemm_x3(g, std::max(sms, 1), device, s);
+    if (ks == 1) return launch_gemm_x3(g, g.k, std::max(sms, 1), device, s);
+    GemmArgs q = g;  // the chunks as batch planes, the last one shorter
+    const int nkb = (g.k + kBK - 1) / kBK, each = (nkb + ks - 1) / ks;
+    q.k = each * kBK;
+    q.batch = (nkb + each - 1) / each;
+    q.a_bstride = q.k;
+    q.b_bstride = g.b_trans ? q.k : (long long)q.k * g.ldb;
+    q.C = g.kpart;
+    q.ldc = g.n;
+    q.c_bstride = g.m * g.n;
+    cudaError_t e = launch_gemm_x3(q, g.k - (q.batch - 1) * q.k, std::max(sms, 1), device, s);
+    return e != cudaSuccess ? e : launch_ksum(g, q.batch, s);
 }
 
 }  // namespace gs

@@ -145,11 +145,14 @@ struct GemmArgs {
                           // (ksplit x m x n floats, caller's workspace) and a second kernel
                           // sums the chunks in a fixed order into C (deterministic)
     float* kpart;
+    long long kpart_floats;  // optional: what kpart holds; launch_gemm_fp32 may then choose a split of its own
     // optional (batch 1): every K chunk's part of A's rows' squared norms (ksplit x m floats)
     float* xx_part;
     int a_vec, b_vec;     // set by the launch: rows of four-element groups on 16-byte boundaries
 };
 cudaError_t launch_gemm_simt(const GemmArgs& g, cudaStream_t s);
+// C = the sum of ks partial products in g.kpart, in order
+cudaError_t launch_ksum(const GemmArgs& g, int ks, cudaStream_t s);
 // sum = false: the partial products stay in kpart (also for one chunk) and C is not written
 cudaError_t launch_gemm_simt_parts(const GemmArgs& g, cudaStream_t s, bool sum);
 // the same product at fp32 accuracy: on the tensor cores when it is large (gs_gemm_x3.cu: operands

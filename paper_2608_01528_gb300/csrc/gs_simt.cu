@@ -925,6 +925,12 @@ cudaError_t launch_scores(const ScoreArgs& a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+cudaError_t launch_ksum(const GemmArgs& g, int ks, cudaStream_t s) {
+    const long long mn = g.m * g.n;
+    k_ksum<<<(unsigned)((mn + 255) / 256), 256, 0, s>>>(g.kpart, ks, g.m, g.n, (float*)g.C, g.ldc);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_gemm_simt(const GemmArgs& g, cudaStream_t s) {
     return launch_gemm_simt_parts(g, s, true);
 }
@@ -958,11 +964,7 @@ cudaError_t launch_gemm_simt_parts(const GemmArgs& args, cudaStream_t s, bool su
     if (g.a_type == TA && g.b_type == TB && g.c_type == TC && g.b_trans == BT) {            \
         if (tall) k_gemm<TA, TB, TC, BT, 8><<<grid, 256, 0, s>>>(g);                        \
         else k_gemm<TA, TB, TC, BT, 4><<<grid, 256, 0, s>>>(g);                             \
-        if (g.ksplit > 1 && sum) {                                                          \
-            const long long mn = g.m * g.n;                                                 \
-            k_ksum<<<(unsigned)((mn + 255) / 256), 256, 0, s>>>(g.kpart, g.ksplit, g.m, g.n, \
-                                                                 (float*)g.C, g.ldc);       \
-        }                                                                                   \
+        if (g.ksplit > 1 && sum) return launch_ksum(g, g.ksplit, s);                        \
         return cudaGetLastError();                                                          \
     }
     GS_GEMM_CASE(MAT_F32, MAT_F32, MAT_F32, true)

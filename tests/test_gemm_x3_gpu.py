@@ -105,3 +105,28 @@ def test_not_finite_as_on_the_cuda_cores(gs, bad):
     rows = [i for i in range(1100) if i not in (7, 1099)]
     ref = T.double() @ b.Q.double()
     assert bool(((X.double() - ref).abs() <= bound(b.r, T.double().abs() @ b.Q.double().abs()))[rows].all())
+
+
+# few output tiles over a deep K: chunks of K to partial products, the last one shorter; rows on and off
+# 16-byte boundaries, odd K
+@pytest.mark.parametrize("N,D,M", [(130, 8191, 300), (1000, 4100, 500), (257, 15999, 700), (640, 2048, 900), (1, 32768, 512)])
+def test_split_k(gs, N, D, M):
+    rng = np.random.default_rng([N, D])
+    C = torch.from_numpy((rng.integers(0, 2, size=(M, D)) * 2 - 1).astype(np.float32)).cuda()
+    lab = torch.from_numpy(rng.integers(0, M, size=N)).cuda()
+    X = C[lab] + torch.from_numpy(rng.standard_normal((N, D)).astype(np.float32)).cuda()
+    if N > 8:
+        X[3, D - 1], X[4, 0] = float("inf"), float("nan")
+    b = gs.build_basis(C)
+    out = gs.project_similarity(b, X, want_S=True, want_Y=True)
+    ref = gs.project_similarity(b, X, want_Y=True, path="simt")
+    again = gs.project_similarity(b, X, want_Y=True)
+    gs.stream_status()
+    fin = torch.isfinite(ref["Y"])
+    assert torch.equal(torch.isfinite(out["Y"]), fin) and torch.equal(again["Y"][fin], out["Y"][fin])
+    ok = torch.isfinite(X).all(1)
+    Xd = X[ok].double()
+    Y = Xd @ b.Q.double().T
+    # six bf16 products of the three-way split leave 2^-24 of |x||q|, the fp32 sums of 128 terms a few more
+    assert bool(((out["Y"][ok].double() - Y).abs() <= 1e-6 * Xd.norm(dim=1)[:, None]).all())
+    assert torch.equal(out["argmax"][ok].long(), lab[ok])
