@@ -55,8 +55,22 @@ constexpr int kCoefR = 64;
 constexpr int kCoefWarps = 8;
 constexpr int kRSmemFloats = 12 * 1024;  // codeword rows staged at a time: 48 KB
 
+// p[0] + p[stride] + ... + p[(ks - 1) stride] in eight sums of every eighth term: their loads are in flight
+// together, and the rounding grows with an eighth of the terms.
+__device__ __forceinline__ float sum_parts(const float* __restrict__ p, long long stride, int ks) {
+    float a[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) a[u] = u < ks ? p[u * stride] : 0.f;
+    for (int z = 8; z < ks; z += 8) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (z + u < ks) a[u] += p[(z + u) * stride];
+    }
+    return ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
+}
+
 struct ScoreParams {
-    const float* Y;       // N x r (ld ldy), or null: y_j = sum over z < ks (in order) of part[z][n][j]
+    const float* Y;       // N x r (ld ldy), or null: y_j = sum over z < ks (in a fixed order) of part[z][n][j]
     int ldy;
     const float* part;
     const float* xx;      // with part: ||x||^2 in ks parts (ks x N), or null
@@ -114,7 +128,7 @@ __global__ void __launch_bounds__(kCoefWarps * 32) k_scores(const ScoreParams p)
                 float y = 0.f;
                 if (j < p.r) {
                     if (p.part) {
-                        for (int z = 0; z < p.ks; ++z) y += p.part[((size_t)z * p.N + n) * p.r + j];
+                        y = sum_parts(p.part + n * p.r + j, p.N * p.r, p.ks);
                         if (p.Yout) p.Yout[(size_t)n * p.ldyo + j] = y;
                     } else {
                         y = __ldg(p.Y + (size_t)n * p.ldy + j);
@@ -125,9 +139,7 @@ __global__ void __launch_bounds__(kCoefWarps * 32) k_scores(const ScoreParams p)
             }
             if (p.mode == GS_SCORE_COSINE) {
                 if (p.part) {
-                    float xx = 0.f;
-                    for (int z = 0; z < p.ks; ++z) xx += p.xx[(size_t)z * p.N + n];
-                    ynorm = sqrtf(xx);
+                    ynorm = sqrtf(sum_parts(p.xx + n, p.N, p.ks));
                 } else {
                     ynorm = p.xnorm ? p.xnorm[n] : sqrtf(warp_sum(yy));
                 }
@@ -561,14 +573,12 @@ __global__ void __launch_bounds__(256) k_gemm_gated(GemmArgs g, long long per) {
     }
 }
 
-// C[i][j] = sum over z (in order) of part[z][i][j]: the split-K partials of k_gemm
+// C[i][j] = sum over z (in a fixed order) of part[z][i][j]: the split-K partials of k_gemm
 __global__ void k_ksum(const float* __restrict__ part, int ks, long long m, int n, float* __restrict__ C,
                        long long ldc) {
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= m * n) return;
-    float s = 0.f;
-    for (int z = 0; z < ks; ++z) s += part[(size_t)z * m * n + idx];
-    C[(idx / n) * ldc + idx % n] = s;
+    C[(idx / n) * ldc + idx % n] = sum_parts(part + idx, m * n, ks);
 }
 
 // ----------------------------------------------------------------- row kernels
