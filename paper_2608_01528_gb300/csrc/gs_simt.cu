@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(kCoefWarps * 32) k_scores(const ScoreParams p)
 // QB x RB products (a lane QB / 4 x RB / 8 of them, 16-byte shared reads without conflicts), the warps'
 // sums meet in shared memory, and the warps score the queries.  Bound by the loads' latency at the usual
 // few hundred queries.  One warp per query read all of Q per query, 4 bytes a lane (2,048 queries of D =
-// 1024, r = 30: 45 us, now 14; of D = 2560: 103, now 28); four queries' products in one warp's registers left
+// 1024, r = 30: 45 us, now 14.5; of D = 2560: 103, now 29); four queries' products in one warp's registers left
 // few for loads in flight (19 and 57 us; at 512 queries, r = 10, it was the faster one, 5 us against 8).
 constexpr int kSmallR = 32;
 constexpr int kSmallM = 64;   // codewords kept in shared memory
@@ -234,6 +234,10 @@ __device__ __forceinline__ void cp_async_zfill4(float* dst, const float* src, in
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
                  "r"(bytes)
                  : "memory");
+}
+
+__device__ __forceinline__ float dot4(const float4& a, const float4& b) {
+    return fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, a.w * b.w)));
 }
 
 template <int QB, int RB, bool VEC>
@@ -285,6 +289,9 @@ __global__ void __launch_bounds__(256) k_ps_small(const float* __restrict__ X, l
         if (c + kSmallStages - 1 < nch) fetch(c + kSmallStages - 1);
         else asm volatile("cp.async.commit_group;" ::: "memory");
         const float* st = ring + (size_t)(c % kSmallStages) * kRows * kSmallPitch + 16 * warp;
+        // a chunk's 16 terms are summed by themselves, by fours: chains of 4, 4 and D / 128 steps (one chain
+        // of D / 8 lost up to twice as much; 28.5 against 28.0 us for 2,048 queries of D = 2560)
+        float part[NQ][NJ] = {}, px[NQ] = {};
 #pragma unroll
         for (int k = 0; k < 16; k += 4) {
             float4 x[NQ], q[NJ];
@@ -294,11 +301,16 @@ __global__ void __launch_bounds__(256) k_ps_small(const float* __restrict__ X, l
             for (int u = 0; u < NJ; ++u) q[u] = *reinterpret_cast<const float4*>(st + (QB + jg + 8 * u) * kSmallPitch + k);
 #pragma unroll
             for (int v = 0; v < NQ; ++v) {
-                xx[v] = fmaf(x[v].x, x[v].x, fmaf(x[v].y, x[v].y, fmaf(x[v].z, x[v].z, fmaf(x[v].w, x[v].w, xx[v]))));
+                px[v] += dot4(x[v], x[v]);
 #pragma unroll
-                for (int u = 0; u < NJ; ++u)
-                    acc[v][u] = fmaf(x[v].x, q[u].x, fmaf(x[v].y, q[u].y, fmaf(x[v].z, q[u].z, fmaf(x[v].w, q[u].w, acc[v][u]))));
+                for (int u = 0; u < NJ; ++u) part[v][u] += dot4(x[v], q[u]);
             }
+        }
+#pragma unroll
+        for (int v = 0; v < NQ; ++v) {
+            xx[v] += px[v];
+#pragma unroll
+            for (int u = 0; u < NJ; ++u) acc[v][u] += part[v][u];
         }
     }
     // the warps' sums, through the ring's memory: [warp][query][RB + 1], the last the squared norm
@@ -315,9 +327,7 @@ __global__ void __launch_bounds__(256) k_ps_small(const float* __restrict__ X, l
     __syncthreads();
     for (int e = threadIdx.x; e < QB * (RB + 1); e += 256) {
         const int qi = e / (RB + 1), j = e - qi * (RB + 1);
-        float t = 0.f;
-#pragma unroll
-        for (int w = 0; w < 8; ++w) t += red[((size_t)w * QB + qi) * (RB + 1) + j];
+        const float t = sum_parts(red + qi * (RB + 1) + j, QB * (RB + 1), 8);
         if (j == RB) {
             xsm[qi] = t;
         } else {
