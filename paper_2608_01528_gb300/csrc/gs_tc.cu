@@ -46,7 +46,8 @@
 //   warp  5      TMEM allocator and MMA issuer (one elected lane)
 //   warp  6      TMA producer of the B operand tiles (Q per K-block, then Rh / Rl)
 //   warps 7-14   converters (fp32 -> fp16, row norms, range check), two groups of
-//                four warps taking alternate K-blocks so two blocks convert at once
+//                four warps taking alternate K-blocks so two blocks convert at once; with a
+//                K split they share the tile's tail with the epilogue (split_tail)
 // Every wait on an mbarrier is bounded (wall-clock limit): on expiry the CTA
 // records GS_DEV_ERR_TIMEOUT, raises a CTA-wide abort flag so the other roles
 // leave their loops, waits (bounded) for its own TMA copies and MMAs to land,
