@@ -362,9 +362,8 @@ __global__ void __launch_bounds__(256) k_panel_reduce(const double* __restrict__
 //    16 x 16 products; otherwise by the fp64 factorisation.  (fp64 runs at 2 FMAs per clock and SM here,
 //    16 dependent steps of it cost ~20 us: the two rounds took 57 us a panel with both in fp64, 39 now.)
 //    Row k is accepted exactly as the row-by-row kernel would: its norm against what came before it,
-//    sqrt(pivot), > tau ||c_k||.  A pivot taken from G in fp64 is only known to ~1e-14 ||v_k||^2, so a
-//    panel with a decision that this could touch (a pivot below 1e-6 ||v_k||^2 that is not certain to
-//    fall below the tolerance, or one within 1e-6 of it) is left to k_panel_gs2.
+//    sqrt(pivot), > tau ||c_k||.  A panel with a pivot that is closer to the tolerance than its own noise
+//    (see chol_factor), or within 1e-6 of it, is left to k_panel_gs2.
 //
 // The factorisation in one CTA (all threads): A (the Gram matrix; the fp64 form overwrites it), T: rows of
 // the transform for the accepted rows (T[k] over the panel's rows).
@@ -397,8 +396,20 @@ __device__ __forceinline__ void chol_load(Chol& c, const double* Gp, int ncl) {
     __syncthreads();
 }
 
-__device__ __forceinline__ void chol_factor(Chol& c, int n, bool first, const double* cn, double tau, int room) {
+// gerr: the first round's Gram matrix and its factorisation are off by at most gerr ||v_i|| ||v_j|| an entry, so
+// row k's pivot is by gerr (sum_j |t_j| ||v_j||)^2, t the combination of the panel's rows that it is the
+// squared norm of (a panel whose taken rows lie close to each other has large t: the noise can exceed the
+// tolerance although 1e-14 ||v_k||^2 does not)
+__device__ __forceinline__ void chol_factor(Chol& c, int n, bool first, const double* cn, double tau, int room,
+                                            double gerr) {
     for (int k = 0; k < n; ++k) {
+        double amp = 0.0;
+        if (first && threadIdx.x < 32) {
+            const int j = threadIdx.x & (kPanel - 1);
+            amp = fabs(c.T[k][j]) * c.nv[j];
+#pragma unroll
+            for (int o = kPanel / 2; o > 0; o >>= 1) amp += __shfl_xor_sync(0xffffffffu, amp, o);
+        }
         if (threadIdx.x == 0) {
             const double piv = c.A[k][k];
             int take = 1;
@@ -409,12 +420,9 @@ __device__ __forceinline__ void chol_factor(Chol& c, int n, bool first, const do
                 } else if (!(v2 > lim2 * (1.0 - 1e-6))) {
                     take = 0;  // what the basis so far leaves of the row is below the tolerance already
                     if (v2 != v2) c.slow = 1;
-                } else if (piv > 1e-6 * v2) {
-                    take = piv > lim2;
-                    if (fabs(piv - lim2) < 1e-6 * lim2) c.slow = 1;
                 } else {
-                    take = 0;  // dependent within the panel, if even 2e-13 ||v||^2 is below the tolerance
-                    if (!(piv < 1e-13 * v2 && 2e-13 * v2 < lim2)) c.slow = 1;
+                    take = piv > lim2;
+                    if (!(fabs(piv - lim2) >= fmax(gerr * amp * amp, 1e-6 * lim2))) c.slow = 1;
                 }
             }
             c.take = take;
@@ -491,7 +499,7 @@ __device__ __forceinline__ void chol_quick(Chol& c, int n, const double* cn, dou
             const float piv = __shfl_sync(0xffffffffu, a[k], k), dk = __shfl_sync(0xffffffffu, d, k),
                         lk = __shfl_sync(0xffffffffu, lim, k);
             if (k >= n || skip || na >= room) continue;  // (warp-uniform)
-            ok = ok && piv > 1e-3f * dk && piv > 1.001f * lk;
+            ok = ok && piv > 1e-3f * dk && piv > 1.01f * lk;
             const float rs = rsqrtf(piv), l = a[k] * rs;
 #pragma unroll
             for (int j = 0; j < kPanel; ++j) {
@@ -508,7 +516,8 @@ __device__ __forceinline__ void chol_quick(Chol& c, int n, const double* cn, dou
             taken |= 1u << k;
             ++na;
         }
-        // T's rounding reaches V' V'^T times (sum_j |t_j| ||v_j||)^2
+        // T's rounding reaches V' V'^T times (sum_j |t_j| ||v_j||)^2, and a pivot 18 x 2^-24 of that square: below
+        // 0.4 % of a taken one, which the 1 % from its tolerance covers
         float amp = 0.f;
 #pragma unroll
         for (int j = 0; j < kPanel; ++j) amp += fabsf(t[j]) * 2.f;
@@ -577,7 +586,7 @@ struct CholParams {
     const double* Gp;   // this round's Gram partials
     double* Gp2;        // the next round's (round 1)
     const double* cn;   // the panel rows' norms
-    double tau;
+    double tau, gerr;   // rank tolerance; bound of the first Gram matrix' relative error (see chol_factor)
     double* R64;        // the panel's first row
     int ldr, rmax;
     const int* r_start;
@@ -606,7 +615,7 @@ __global__ void __launch_bounds__(512) k_panel_chol(const CholParams p) {
             for (int e = tid; e < kPanel * kPanel; e += nt) p.st->G[e / kPanel][e % kPanel] = c.A[e / kPanel][e % kPanel];
         chol_quick(c, n, p.cn, p.tau, p.rmax - r0);
         if (!c.quick) {
-            chol_factor(c, n, true, p.cn, p.tau, p.rmax - r0);
+            chol_factor(c, n, true, p.cn, p.tau, p.rmax - r0, p.gerr);
             // V' = T V multiplies G's rounding by (sum_j |T_kj| ||v_j||)^2: beyond 1e8 the second round would
             // not bring it back to eps
             if (tid < p.bp && !c.slow) {
@@ -619,7 +628,7 @@ __global__ void __launch_bounds__(512) k_panel_chol(const CholParams p) {
             __syncthreads();
         }
     } else if (!chol_series(c, n)) {
-        chol_factor(c, n, false, p.cn, p.tau, p.rmax - r0);
+        chol_factor(c, n, false, p.cn, p.tau, p.rmax - r0, 0.0);
     }
     const bool slow = ROUND == 1 && c.slow != 0;
     if (ROUND == 1 && blockIdx.x == 0) {
@@ -997,6 +1006,9 @@ gs_status factor_rows(const float* C, int M, int D, int ldc, double tau, bool no
                                           std::max<size_t>(2 * (size_t)kPanel * jc, kPairs)) +
                         sizeof(float) * ((size_t)jc * vl + (size_t)kPanel * jc);
     const size_t smem_chol = sizeof(double) * (size_t)kPanel * vl;
+    // longest chains of sums behind an entry of a Gram matrix (w / 2 terms in a slice, the cluster's CTAs, the
+    // clusters) and behind a pivot (kPanel steps), a unit roundoff each, and twice that for the second order
+    const double gerr = 0x1p-52 * (w / 2 + kSliceCluster + ncl + kPanel + 4);
     for (auto fn : {k_panel_slice<kDots1>, k_panel_slice<kUpdDots>, k_panel_slice<kUpdGram>})
         GS_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
 
@@ -1063,7 +1075,7 @@ gs_status factor_rows(const float* C, int M, int D, int ldc, double tau, bool no
         cp.V = V, cp.Qw = Qw;
         cp.D = D, cp.w = w, cp.bp = bp, cp.ncl = ncl;
         cp.Gp = G1, cp.Gp2 = G2;
-        cp.cn = cn + p0, cp.tau = tau;
+        cp.cn = cn + p0, cp.tau = tau, cp.gerr = gerr;
         cp.R64 = R64 + (size_t)p0 * ldr, cp.ldr = ldr, cp.rmax = rmax;
         cp.r_start = r_at + pn, cp.r_next = r_at + pn + 1;
         cp.st = st;

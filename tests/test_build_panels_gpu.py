@@ -2,6 +2,7 @@
 the panels whose rank decisions the pivots cannot settle), against a row-by-row Gram-Schmidt in 64
 bits.  Q and R are held in fp32: 2^-23 of the entry's own size covers their rounding, and the factors
 themselves agree to 64-bit accuracy times the conditioning of the accepted rows (below 1e5 here)."""
+import numpy as np
 import pytest
 import torch
 
@@ -74,3 +75,29 @@ def test_scale(gs, scale):
     gs.stream_status()
     assert a.r == b.r
     assert float((a.Q - b.Q).abs().max()) <= 1e-7
+
+
+@pytest.mark.parametrize("rows", [3, 4])
+@pytest.mark.parametrize("tol", [1e-6, 1e-9])
+def test_rows_close_to_what_earlier_ones_left_over(gs, rows, tol):
+    """a, a + e b, b + d c, and a, a + e b, b + f c, c + d g, all exact in fp32: every row is off the span of
+    those before it by more than three times the tolerance, but the last pivot's noise in a Gram matrix,
+    2^-53 (2 / e)^2 of the row or 2^-53 (4 / (e f))^2, is above d^2."""
+    def exact(rng, bits):
+        return rng.integers(-2 ** bits, 2 ** bits + 1, 300) / 2.0 ** bits
+
+    for seed in range(100):
+        rng = np.random.default_rng([seed, rows])
+        e, f = 2.0 ** -rng.integers(7, 10), 2.0 ** -rng.integers(4, 8)
+        d = 2.0 ** -18 * rng.integers(1, 4)
+        a, b, c, g = exact(rng, 9), exact(rng, 9), exact(rng, 3 if rows == 3 else 9), exact(rng, 3)
+        if rows == 4:
+            e = 2.0 ** -rng.integers(4, 8)
+        C = np.stack([a, a + e * b, b + d * c] if rows == 3 else [a, a + e * b, b + f * c, c + d * g])
+        C = torch.from_numpy(C.astype(np.float32)).cuda()
+        b = gs.build_basis(C, rank_tol=tol)
+        assert b.r == rows, (seed, e, f, d)
+        Q, R = b.Q.double(), b.R.double()
+        # fp32 factors: 2^-24 of each of two factors per term
+        assert bool(((C.double() - R @ Q).abs() <= 2.0 ** -22 * (R.abs() @ Q.abs())).all()), seed
+    gs.stream_status()
