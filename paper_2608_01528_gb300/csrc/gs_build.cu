@@ -187,8 +187,17 @@ __device__ __forceinline__ double row_pow2(double n, int sign) {
     return __hiloint2double((1023 + sign * e) << 20, 0);
 }
 
+// shared memory of k_panel_slice for slices of w columns and chunks of jc basis rows
+constexpr size_t slice_smem(int w, int jc) {
+    return sizeof(double) * ((size_t)(kPanel + 2 * jc) * (w | 1) + (2 * kPanel * jc > kPairs ? 2 * kPanel * jc : kPairs)) +
+           sizeof(float) * ((size_t)jc * (w | 1) + (size_t)kPanel * jc);
+}
+constexpr int kSliceThreads = 512;  // at most
+constexpr size_t kSliceSmemMax = slice_smem(kMaxSlice, kSliceThreads / kPanel * 2);
+static_assert(kSliceSmemMax <= 227 * 1024, "a slice of the panel and its chunks of the basis fit a CTA's shared memory");
+
 template <int KIND>
-__global__ void __launch_bounds__(512) k_panel_slice(const SliceParams p) {
+__global__ void __launch_bounds__(kSliceThreads) k_panel_slice(const SliceParams p) {
     extern __shared__ double sm[];
     const int tid = threadIdx.x, nt = blockDim.x;
     const int r0 = *p.r_start;
@@ -997,20 +1006,20 @@ gs_status factor_rows(const float* C, int M, int D, int ldc, double tau, bool no
     const int nslices = ((D + w - 1) / w + kSliceCluster - 1) / kSliceCluster * kSliceCluster;
     const int ncl = nslices / kSliceCluster;
     // threads: the update's kPanel w outputs in as few full rounds as fit (at most three of 512)
-    const int rounds = (kPanel * w + 511) / 512;
+    const int rounds = (kPanel * w + kSliceThreads - 1) / kSliceThreads;
     int threads = ((kPanel * w + rounds - 1) / rounds + 31) / 32 * 32;
-    if (threads < 320) threads = 512;  // short rows: few outputs, so longer chunks of the basis instead
+    if (threads < 320) threads = kSliceThreads;  // short rows: few outputs, so longer chunks of the basis instead
     const int jc = threads / kPanel * 2;        // basis rows per chunk: two dot products a thread
     const int vl = w | 1;
-    const size_t smem = sizeof(double) * ((size_t)kPanel * vl + 2 * (size_t)jc * vl +
-                                          std::max<size_t>(2 * (size_t)kPanel * jc, kPairs)) +
-                        sizeof(float) * ((size_t)jc * vl + (size_t)kPanel * jc);
+    const size_t smem = slice_smem(w, jc);
     const size_t smem_chol = sizeof(double) * (size_t)kPanel * vl;
     // longest chains of sums behind an entry of a Gram matrix (w / 2 terms in a slice, the cluster's CTAs, the
     // clusters) and behind a pivot (kPanel steps), a unit roundoff each, and twice that for the second order
     const double gerr = 0x1p-52 * (w / 2 + kSliceCluster + ncl + kPanel + 4);
+    // the limit belongs to the function on the device: one that covers every D, since another thread may be
+    // building from rows of another length at the same time
     for (auto fn : {k_panel_slice<kDots1>, k_panel_slice<kUpdDots>, k_panel_slice<kUpdGram>})
-        GS_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        GS_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSliceSmemMax));
 
     // the factors, and one workspace for everything else
     GS_CK(cudaMalloc(&f.Qw, sizeof(double) * (size_t)rmax * D));

@@ -2,6 +2,8 @@
 the panels whose rank decisions the pivots cannot settle), against a row-by-row Gram-Schmidt in 64
 bits.  Q and R are held in fp32: 2^-23 of the entry's own size covers their rounding, and the factors
 themselves agree to 64-bit accuracy times the conditioning of the accepted rows (below 1e5 here)."""
+import concurrent.futures as cf
+
 import numpy as np
 import pytest
 import torch
@@ -100,4 +102,17 @@ def test_rows_close_to_what_earlier_ones_left_over(gs, rows, tol):
         Q, R = b.Q.double(), b.R.double()
         # fp32 factors: 2^-24 of each of two factors per term
         assert bool(((C.double() - R @ Q).abs() <= 2.0 ** -22 * (R.abs() @ Q.abs())).all()), seed
+    gs.stream_status()
+
+
+def test_builds_from_two_threads(gs):
+    """Codebooks of short and of long rows, whose kernels need different amounts of shared memory, at once."""
+    def build(D):
+        with torch.cuda.stream(torch.cuda.Stream()):
+            C = codebook(100, D)
+            return [gs.build_basis(C).r for _ in range(25)]
+
+    with cf.ThreadPoolExecutor(2) as ex:
+        for ranks in ex.map(build, [512, 14600]):
+            assert ranks == [100] * 25
     gs.stream_status()
