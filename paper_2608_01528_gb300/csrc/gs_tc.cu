@@ -678,6 +678,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                         mma_commit(&c.b_empty[sr]);
                     }
                 }
+                // K-blocks of Y that no codeword uses (R may end before r): the epilogue may still be reading
+                // them, and with a K split the peers' parts of them, where the scores go once S is there
+                for (; nsplit < (p.npad + kBK - 1) / kBK; ++nsplit)
+                    if (!wait_1t(&c.ysplit[nsplit], pt)) return false;
                 mma_commit(&c.s_full);
                 // the next tile's GEMM1 overwrites the columns GEMM2 reads: wait for it to finish
                 mma_commit(&c.gemm2_done);

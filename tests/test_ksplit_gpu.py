@@ -112,3 +112,23 @@ def test_zero_and_nan_rows(gs, N):
     tol = TOL * X[keep].double().norm(dim=1)[:, None] * C.double().norm(dim=1)[None, :]
     assert bool(((out["S"][keep].double() - S).abs() <= tol).all())
     assert torch.equal(out["S"][keep].argmax(1), out["argmax"][keep].long())
+
+
+@pytest.mark.parametrize("N", [500, 3000, 6000, 20000])
+@pytest.mark.parametrize("used", [40, 130])
+def test_codewords_that_use_part_of_the_basis(gs, N, used):
+    """A basis of 256 rows kept for a codebook of which only the first `used` entries are left: the scores are
+    there before the last columns of Y are, which are outputs all the same."""
+    C, X, _ = setup(256, 4160, N, [N, used])
+    full = gs.build_basis(C)
+    left = torch.arange(256, device="cuda") % used
+    b = gs.import_basis(full.Q, full.R[left].contiguous())
+    assert b.r == 256
+    Xd, Cd = X.double(), C[left].double()
+    S, Y = Xd @ Cd.T, Xd @ full.Q.double().T
+    tol_s = TOL * Xd.norm(dim=1)[:, None] * Cd.norm(dim=1)[None, :]
+    for _ in range(5):
+        out = gs.project_similarity(b, X, path="tensor", want_S=True, want_Y=True)
+        gs.stream_status()
+        assert bool(((out["S"].double() - S).abs() <= tol_s).all())
+        assert bool(((out["Y"].double() - Y).abs() <= TOL * Xd.norm(dim=1)[:, None]).all())
