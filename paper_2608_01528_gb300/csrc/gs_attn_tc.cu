@@ -584,7 +584,8 @@ __global__ void __launch_bounds__(kClThreads, 1)
                     ext = c2 >= 0.f ? row_extreme<false, false>(v, kClCols) : row_extreme<true, false>(v, kClCols);
                 else
                     ext = c2 >= 0.f ? row_extreme<false, true>(v, nvalid) : row_extreme<true, true>(v, nvalid);
-                const float mc = c2 * ext;
+                // (keys whose logits are all -inf, masked ones, add nothing: 2^(-inf - mc) with a finite mc)
+                const float mc = fmaxf(c2 * ext, -FLT_MAX);
                 float l8[8];
 #pragma unroll
                 for (int q = 0; q < 8; ++q) l8[q] = 0.f;

@@ -39,3 +39,25 @@ def test_unaligned_output(gs):
     gs.stream_status()
     ref = torch.softmax(0.1 * (q.double() @ k.double().transpose(1, 2)), dim=2)
     assert float((A.double() - ref).abs().max()) <= 1e-5
+
+
+# one unit a CTA (rows on and off 16-byte boundaries), two units, and the two-pass kernel past 4,096 keys
+@pytest.mark.parametrize("Lk", [640, 1023, 1537, 4096, 4100])
+@pytest.mark.parametrize("scale", [0.06, -0.06])
+def test_masked_keys(gs, Lk, scale):
+    """Keys masked by an infinity in a dimension of their own: weight 0, also where they fill whole chunks."""
+    g = torch.Generator(device="cuda").manual_seed(Lk)
+    q = torch.randn((4, 200, 72), generator=g, device="cuda").bfloat16()
+    k = torch.randn((4, Lk, 72), generator=g, device="cuda").bfloat16()
+    q[:, :, 0] = 1
+    k[:, :, 0] = 0
+    mask = torch.zeros((4, Lk), dtype=torch.bool, device="cuda")
+    mask[0, Lk // 3:] = True             # the tail, the head, every second chunk of 64, all but one key
+    mask[1, :Lk // 2] = True
+    mask[2] = torch.arange(Lk, device="cuda") // 64 % 2 == 1
+    mask[3, torch.arange(Lk, device="cuda") != 70] = True
+    k[:, :, 0][mask] = -float("inf") if scale > 0 else float("inf")
+    A = gs.attention_scores(q, k, scale, path="tensor")
+    gs.stream_status()
+    ref = torch.softmax(scale * (q.double() @ k.double().transpose(1, 2)), dim=2)
+    assert bool(((A.double() - ref).abs() <= 1e-4 * ref.amax(2, keepdim=True)).all())
