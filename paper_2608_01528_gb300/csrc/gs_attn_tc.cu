@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         const float m0 = __shfl_sync(0xffffffffu, m, r0), l0 = __shfl_sync(0xffffffffu, l, r0);
                         const float m1 = __shfl_sync(0xffffffffu, m, r0 + 8), l1 = __shfl_sync(0xffffffffu, l, r0 + 8);
                         const float mh[2] = {m0, m1};
-                        const float ih[2] = {l0 > 0.f ? 1.f / l0 : 0.f, l1 > 0.f ? 1.f / l1 : 0.f};
+                        const float ih[2] = {l0 != 0.f ? 1.f / l0 : 0.f, l1 != 0.f ? 1.f / l1 : 0.f};
                         int qrow[2];
                         float* arow[2];
 #pragma unroll
@@ -428,7 +428,7 @@ __device__ __forceinline__ float2 merge_stats(const float2* e, int n) {
     float L = 0.f;
 #pragma unroll
     for (int j = 0; j < MAXN; ++j)
-        if (j < n && e[j].y > 0.f) L += e[j].y * ex2_approx(e[j].x - M);
+        if (j < n && e[j].y != 0.f) L += e[j].y * ex2_approx(e[j].x - M);  // (a NaN stays one)
     return make_float2(M, L);
 }
 
@@ -594,7 +594,7 @@ __global__ void __launch_bounds__(kClThreads, 1)
                     if (nvalid == kClCols || j < nvalid) l8[j & 7] += ex2_approx(fmaf(v[j], c2, -mc));
                 const float lc = ((l8[0] + l8[1]) + (l8[2] + l8[3])) + ((l8[4] + l8[5]) + (l8[6] + l8[7]));
                 const float mn = fmaxf(m, mc);
-                l = (l > 0.f ? l * ex2_approx(m - mn) : 0.f) + lc * ex2_approx(mc - mn);
+                l = (l != 0.f ? l * ex2_approx(m - mn) : 0.f) + lc * ex2_approx(mc - mn);
                 m = mn;
             }
             // the row's two key halves meet in shared memory; the even-half warps merge them
@@ -628,7 +628,7 @@ __global__ void __launch_bounds__(kClThreads, 1)
                 for (int q = 0; q < kMax; ++q) e[q] = q < nunits ? xch[q * kBM + i] : make_float2(-INFINITY, 0.f);
                 const float2 rw = merge_stats<kMax>(e, nunits);
                 M = rw.x;
-                invL = rw.y > 0.f ? __fdividef(1.f, rw.y) : 0.f;
+                invL = rw.y != 0.f ? __fdividef(1.f, rw.y) : 0.f;  // no key has any weight: 0; a NaN: the row is NaN
             }
             // writing pass: 2^(c s_j - M) / L through 32 x 16 tiles (16-byte chunk q of row
             // `lane` at chunk q ^ ((lane / 2) % 4), the TMA's 64-byte swizzle) and tensor stores

@@ -61,3 +61,25 @@ def test_masked_keys(gs, Lk, scale):
     gs.stream_status()
     ref = torch.softmax(scale * (q.double() @ k.double().transpose(1, 2)), dim=2)
     assert bool(((A.double() - ref).abs() <= 1e-4 * ref.amax(2, keepdim=True)).all())
+
+
+@pytest.mark.parametrize("Lk", [640, 1023, 1537, 4096, 4100])
+@pytest.mark.parametrize("bad", ["nan key", "nan query", "inf"])
+def test_rows_without_a_softmax_are_nan(gs, Lk, bad):
+    """A NaN logit or one of +inf: no softmax of that row, and no finite weights that look like one."""
+    g = torch.Generator(device="cuda").manual_seed(Lk)
+    q = torch.randn((3, 200, 72), generator=g, device="cuda").bfloat16()
+    k = torch.randn((3, Lk, 72), generator=g, device="cuda").bfloat16()
+    rows = torch.zeros((3, 200), dtype=torch.bool, device="cuda")
+    if bad == "nan query":
+        q[1, 131, 5] = float("nan")
+        rows[1, 131] = True
+    else:
+        q[:, :, 0] = 1
+        k[1, Lk - 70, 0] = float("nan") if bad == "nan key" else float("inf")
+        rows[1] = True
+    A = gs.attention_scores(q, k, 0.06, path="tensor")
+    gs.stream_status()
+    ref = torch.softmax(0.06 * (q.double() @ k.double().transpose(1, 2)), dim=2)
+    assert bool(torch.isnan(ref[rows]).all()) and bool(torch.isnan(A[rows]).all())
+    assert bool(((A[~rows].double() - ref[~rows]).abs() <= 1e-4 * ref[~rows].amax(1, keepdim=True)).all())
