@@ -7,21 +7,25 @@
 //   A  m x K row-major, fp32 or bf16; B  fp32, n x K (b_trans) or K x n; C  fp32 or bf16; batched.
 //
 // Every fp32 operand is the sum of three bf16 numbers, x = h + m + l: h = bf16(x), m = bf16(x - h),
-// l = bf16(x - h - m), each difference exact in fp32, 3 x 8 significant bits and fp32's exponent
-// range.  Six of the nine products (hh, hm, mh, mm, hl, lh) are taken on the tensor core; the three
-// left out are below 2^-24 of each term.  The tensor core's fp32 accumulation loses a bounded
-// amount at every step, which grows with the number of steps rather than with its square root, so
-// (1) hh has an accumulator of its own, the five small products share another (their sum is ~2^-8 of
-// hh's, and so are its losses), and (2) hh's accumulator is emptied every kChunk K-blocks (128 terms)
+// l = bf16(x - h - m), each difference exact in fp32, 3 x 8 significant bits.  m and l are kept as 2^8 m and
+// 2^16 l, no larger than x: bf16 ends at 2^-133, and without the factors every operand below 2^-110 lost
+// bits of l, then of m (at 1e-37, 5e-4 of a row; now 6e-8 down to fp32's subnormals).  Six of the nine
+// products (hh, hm, mh, mm, hl, lh) are taken on the tensor core; the three left out are below 2^-24 of each
+// term.  The tensor core's fp32 accumulation loses a bounded amount at every step, which grows with the
+// number of steps rather than with its square root, so (1) hh has an accumulator of its own, as have the
+// products of each of the two scales, hm + mh and mm + hl + lh (their sums are ~2^-8 and 2^-16 of hh's, and so
+// are their losses), and (2) hh's accumulator is emptied every kChunk K-blocks (128 terms)
 // into fp32 registers (round to nearest).  Relative error against 64 bits, 16,384 x 922 -> 10,000:
 // 9e-8, the CUDA-core GEMM's 5.4e-7; at 300 terms 9e-8 and 3.1e-7.  (Chunks of 256 terms: 1.3e-7 at the
 // same speed, but 4.9e-7 against 4.1e-7 where all terms of a sum have one sign; of 512: 2.4e-7.)
-// Outputs of a thread that holds one that is not finite (an operand that is not, or beyond bf16's
-// range) are computed again as plain fp32 dot products, so infinities and NaN come out as the
+// Outputs of a thread that holds one that is not finite (an operand that is not, or beyond 2^120, where
+// the factors overflow) are computed again as plain fp32 dot products, so infinities and NaN come out as the
 // CUDA-core GEMM has them.
 //
 // Measured (GB300, reconstruction of 16,384 rows, r = 922, D = 10,000, rows of 922 floats): 8,240 us on
-// the CUDA cores (36.7 TFLOP/s), 1,700 us here (178 TFLOP/s).  What bounds it: the converters' loads
+// the CUDA cores (36.7 TFLOP/s), 1,800 us here (168 TFLOP/s; 1,734 without the factors and their third
+// accumulator; multiplying both differences on the way, rather than what the second is taken from, 1,900).
+// What bounds it: the converters' loads
 // (long scoreboard is the top stall, the tensor pipe 40 % active).  Shared memory would be next: per
 // K-block of 32 a 128 x 128 tile writes 48 KB of operand planes and its 12 MMAs read 96 KB of them,
 // 1125 clk at 128 B/clk against 768 clk of MMA.  Tried: one group of eleven converter warps (3,670 to
@@ -65,7 +69,9 @@ constexpr int kPairBytes = 6 * kPlane;              // A h, m, l then B h, m, l 
 constexpr int kStages = 4;                          // K-blocks: stage s is half s & 1 of pair s >> 1
 constexpr int kChunk = 4;                           // K-blocks of hh summed on the tensor core at a time
 constexpr int kSlots = 4;                           // tasks of one warp, per operand: 16 tasks over four warps
-constexpr int kTmemCols = 512;                      // hh: 2 x 128, small products: 2 x 128
+constexpr int kTmemCols = 512;                      // hh: 2 x 128, then hm + mh and mm + hl + lh: 128 each
+constexpr uint32_t kColMid = 256, kColLow = 384;
+constexpr float kPartScale = 256.f;                 // m and l are kept as 2^8 m and 2^16 l
 
 struct X3Params {
     const void* A;
@@ -84,7 +90,7 @@ struct X3Params {
 
 struct Ctl {
     uint64_t full[kStages], empty[kStages];
-    uint64_t a_full[2], a_empty[2], x_empty[2];
+    uint64_t a_full[2], a_empty[2], x_empty;
     uint64_t mma_done;
     uint32_t tmem_base;
     int abort_flag;
@@ -166,12 +172,38 @@ __device__ __forceinline__ float2 sub_bf16x2(float2 a, uint32_t w) {
     return r;
 }
 
-// two elements into their three bf16 parts, packed
+__device__ __forceinline__ float2 scale_part(float2 a) {
+    float2 r;
+    asm("{\n\t.reg .b64 x, y, z;\n\t"
+        "mov.b64 x, {%2, %3};\n\t"
+        "mov.b64 y, {%4, %4};\n\t"
+        "mul.rn.f32x2 z, x, y;\n\t"
+        "mov.b64 {%0, %1}, z;\n\t}"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(a.x), "f"(a.y), "f"(kPartScale));
+    return r;
+}
+
+// a minus kPartScale times the two bf16 values packed in w, exact here
+__device__ __forceinline__ float2 sub_scaled_bf16x2(float2 a, uint32_t w) {
+    float2 r;
+    asm("{\n\t.reg .b64 x, y, z, s;\n\t"
+        "mov.b64 x, {%2, %3};\n\t"
+        "mov.b64 y, {%4, %5};\n\t"
+        "mov.b64 s, {%6, %6};\n\t"
+        "fma.rn.f32x2 z, y, s, x;\n\t"
+        "mov.b64 {%0, %1}, z;\n\t}"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(a.x), "f"(a.y), "f"(__uint_as_float(w << 16)), "f"(__uint_as_float(w & 0xffff0000u)), "f"(-kPartScale));
+    return r;
+}
+
+// two elements into their three bf16 parts h, 2^8 m and 2^16 l, packed
 __device__ __forceinline__ void split3(float2 x, uint32_t& h, uint32_t& m, uint32_t& l) {
     h = pack_bf16(x.x, x.y);
-    x = sub_bf16x2(x, h);
+    x = scale_part(sub_bf16x2(x, h));
     m = pack_bf16(x.x, x.y);
-    x = sub_bf16x2(x, m);
+    x = sub_scaled_bf16x2(scale_part(x), m);
     l = pack_bf16(x.x, x.y);
 }
 
@@ -195,8 +227,8 @@ __global__ void __maxnreg__(96) k_gemm_x3(const __grid_constant__ X3Params p) {
         for (int b = 0; b < 2; ++b) {
             mbar_init(&c.a_full[b], 1);
             mbar_init(&c.a_empty[b], kEpiWarps);
-            mbar_init(&c.x_empty[b], kEpiWarps);
         }
+        mbar_init(&c.x_empty, kEpiWarps);
         mbar_init(&c.mma_done, 1);
         c.abort_flag = 0;
         fence_barrier_init();
@@ -226,9 +258,9 @@ __global__ void __maxnreg__(96) k_gemm_x3(const __grid_constant__ X3Params p) {
             int chunk = 0;  // chunks of hh issued so far: accumulator chunk & 1
             bool ok = true;
             for (int lt = 0; lt < ntiles && ok; ++lt) {
-                const int xb = lt & 1;
-                const uint32_t xt = tmem + 256u + (uint32_t)(xb * 128);
-                if (!mbar_wait_1t(&c.x_empty[xb], ((uint32_t)(lt >> 1) & 1u) ^ 1u, abort_flag, err)) break;
+                const uint32_t mid = tmem + kColMid, low = tmem + kColLow;
+                if (!mbar_wait_1t(&c.x_empty, ((uint32_t)lt & 1u) ^ 1u, abort_flag, err)) break;
+                tc_fence_after();
                 for (int kb = 0; kb < p.nkb; ++kb, rs.next(kStages)) {
                     const bool first = kb % kChunk == 0;
                     const int ab = chunk & 1;
@@ -249,11 +281,11 @@ __global__ void __maxnreg__(96) k_gemm_x3(const __grid_constant__ X3Params p) {
 #pragma unroll
                     for (int k = 0; k < kBK / 16; ++k) {
                         const uint64_t o = (uint64_t)(2 * k);
-                        mma_f16_ss(xt, ah + o, bl + o, idesc, (kb | k) != 0 ? 1u : 0u);
-                        mma_f16_ss(xt, al + o, bh + o, idesc, 1u);
-                        mma_f16_ss(xt, am + o, bm + o, idesc, 1u);
-                        mma_f16_ss(xt, ah + o, bm + o, idesc, 1u);
-                        mma_f16_ss(xt, am + o, bh + o, idesc, 1u);
+                        mma_f16_ss(low, ah + o, bl + o, idesc, (kb | k) != 0 ? 1u : 0u);
+                        mma_f16_ss(low, al + o, bh + o, idesc, 1u);
+                        mma_f16_ss(low, am + o, bm + o, idesc, 1u);
+                        mma_f16_ss(mid, ah + o, bm + o, idesc, (kb | k) != 0 ? 1u : 0u);
+                        mma_f16_ss(mid, am + o, bh + o, idesc, 1u);
                         mma_f16_ss(at, ah + o, bh + o, idesc, (!first || k != 0) ? 1u : 0u);
                     }
                     mma_commit(&c.empty[rs.idx]);
@@ -400,7 +432,6 @@ __global__ void __maxnreg__(96) k_gemm_x3(const __grid_constant__ X3Params p) {
         int chunk = 0;
         bool ok = true;
         for (int lt = 0; lt < ntiles && ok; ++lt) {
-            const int xb = lt & 1;
             float acc[4][16];  // [32 columns x 2][16-lane half x 2] in the 16x256b pattern
 #pragma unroll
             for (int q = 0; q < 4; ++q)
@@ -430,8 +461,23 @@ __global__ void __maxnreg__(96) k_gemm_x3(const __grid_constant__ X3Params p) {
                 if (lane == 0) mbar_arrive(&c.a_empty[ab]);
             }
             if (!ok) break;
-            add(256u + (uint32_t)(xb * 128));
-            if (lane == 0) mbar_arrive(&c.x_empty[xb]);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if (64 * half + 32 * (q >> 1) >= p.nt) continue;
+                const uint32_t tq = tb + ((uint32_t)(16 * (q & 1)) << 16) + (uint32_t)(32 * (q >> 1));
+                float t[16];
+                tmem_ld16x256b_x4(tq + kColLow, t);
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    float u[8];
+                    tmem_ld16x256b_x2(tq + kColMid + 16u * e, u);
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) acc[q][8 * e + j] = fmaf(fmaf(t[8 * e + j], 1.f / kPartScale, u[j]), 1.f / kPartScale, acc[q][8 * e + j]);
+                }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&c.x_empty);
 
             long long b, tm;
             int tn;

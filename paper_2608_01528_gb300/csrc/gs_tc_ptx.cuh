@@ -409,6 +409,19 @@ static __device__ __forceinline__ void tmem_ld16x256b_x4(uint32_t taddr, float* 
 #pragma unroll
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
+// The same pattern over 16 columns (the wait names the registers, so no use of them can be scheduled before it).
+static __device__ __forceinline__ void tmem_ld16x256b_x2(uint32_t taddr, float* v) {
+    uint32_t r[8];
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7])
+                 :
+                 : "memory");
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
 // 32 consecutive fp32 columns of this thread's TMEM lane, issued without waiting, so that
 // several loads are in flight; tmem_wait_ld32 then waits and names the registers as its
 // operands, so no use of them can be scheduled before the wait.

@@ -130,3 +130,37 @@ def test_split_k(gs, N, D, M):
     # six bf16 products of the three-way split leave 2^-24 of |x||q|, the fp32 sums of 128 terms a few more
     assert bool(((out["Y"][ok].double() - Y).abs() <= 1e-6 * Xd.norm(dim=1)[:, None]).all())
     assert torch.equal(out["argmax"][ok].long(), lab[ok])
+
+
+@pytest.mark.parametrize("e", [-108, -115, -122, -130])
+def test_small_operands(gs, e):
+    """Operands down to fp32's subnormals lose nothing: the bound holds with no absolute slack but fp32's own
+    rounding of subnormal sums, 2^-149 a term, twice."""
+    def close(X, ref, K, mag):
+        assert bool(((X.double() - ref).abs() <= (12 + -(-K // 128)) * 2.0 ** -23 * mag + K * 2.0 ** -148).all())
+
+    rng = np.random.default_rng(-e)
+    b = gs.build_basis(bipolar(rng, 161, 8200))
+    T = (torch.from_numpy(rng.standard_normal((2049, 161))).cuda() * 2.0 ** e).float()
+    close(gs.reconstruct(b, T), T.double() @ b.Q.double(), 161, T.double().abs() @ b.Q.double().abs())
+    q = (torch.from_numpy(rng.standard_normal((5, 391, 130))).cuda() * 2.0 ** e).float()
+    k = (torch.from_numpy(rng.standard_normal((5, 1517, 130))).cuda() * 2.0 ** 40).float()
+    for x, y in ((q, k), (k, q)):
+        A = gs.attention_scores(x, y, 1.0, apply_softmax=False)
+        xt, yt = x.double(), y.double().transpose(1, 2)
+        close(A, xt @ yt, 130, xt.abs() @ yt.abs())
+    gs.stream_status()
+
+
+def test_large_operands(gs):
+    """Beyond 2^120 the parts' factors overflow: the plain fp32 dot product instead."""
+    rng = np.random.default_rng(6)
+    b = gs.build_basis(bipolar(rng, 161, 8200))
+    T = torch.from_numpy(rng.standard_normal((2049, 161)).astype(np.float32)).cuda()
+    T[5] *= 1e36
+    T[700:900] *= 3e35
+    X = gs.reconstruct(b, T)
+    gs.stream_status()
+    ref = T.double() @ b.Q.double()
+    # (161 terms in order: 161 x 2^-24)
+    assert bool(((X.double() - ref).abs() <= bound(161, T.double().abs() @ b.Q.double().abs()) * (161 / 14)).all())
