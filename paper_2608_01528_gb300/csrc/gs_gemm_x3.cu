@@ -86,6 +86,7 @@ struct X3Params {
     float alpha;
     const float* rownorm;
     const float* colnorm;
+    const int* b_rowlen;  // as in GemmArgs: B's row j is zero from there on
 };
 
 struct Ctl {
@@ -542,8 +543,16 @@ __global__ void __maxnreg__(96) k_gemm_x3(const __grid_constant__ X3Params p) {
                     const long long row = tm * kBM + quad * 32 + 16 * ((e >> 2) & 1) + (lane >> 2) + 8 * ((e >> 1) & 1);
                     if (cl >= p.nt || col >= p.n || row >= p.m) continue;
                     float g = 0.f;
+                    // where B's rows end: the CUDA-core GEMM multiplies no zeros past the longest of 64 (an
+                    // infinity or a NaN of A's row that lies there does not reach these columns)
+                    int end = kend;
+                    if (p.b_rowlen) {
+                        end = 0;
+                        for (int j = col & ~63; j < min(p.n, (col & ~63) + 64); ++j) end = max(end, p.b_rowlen[j]);
+                        end = min(end, kend);
+                    }
 #pragma unroll 4
-                    for (int k = 0; k < kend; ++k)
+                    for (int k = 0; k < end; ++k)
                         g = fmaf(lda1<TA>(Ab, row * p.lda + k),
                                  __ldg(Bb + (BT ? (long long)col * p.ldb + k : (long long)k * p.ldb + col)), g);
                     g = finish(g, row, col);
@@ -602,6 +611,7 @@ static cudaError_t launch_gemm_x3(const GemmArgs& g, int k_last, int sms, int de
     p.alpha = g.alpha;
     p.rownorm = g.rownorm;
     p.colnorm = g.colnorm;
+    p.b_rowlen = g.b_rowlen;
     const size_t smem = 1024 + (size_t)(kStages / 2) * kPairBytes + sizeof(Ctl);
     const int grid = (int)std::min<long long>(sms, p.tiles);
 #define GS_X3_CASE(TA, BT, VEC)                                                                     \

@@ -164,3 +164,24 @@ def test_large_operands(gs):
     ref = T.double() @ b.Q.double()
     # (161 terms in order: 161 x 2^-24)
     assert bool(((X.double() - ref).abs() <= bound(161, T.double().abs() @ b.Q.double().abs()) * (161 / 14)).all())
+
+
+@pytest.mark.parametrize("bad", [float("inf"), float("nan")])
+def test_not_finite_past_the_end_of_a_codeword(gs, bad):
+    """Entry i's coordinates end at i + 1: a bad coordinate past it is not multiplied by the zeros there, tile
+    by tile of 64 entries as on the CUDA cores."""
+    rng = np.random.default_rng(7)
+    b = gs.build_basis(bipolar(rng, 333, 2000))
+    Y = torch.from_numpy(rng.standard_normal((4000, b.r)).astype(np.float32)).cuda()
+    Y[17, 140] = bad
+    Y[3999, 332] = bad
+    for mode in ("raw", "cosine"):
+        out = gs.similarity_coeffs(b, Y, mode=mode, want_S=True)
+        ref = gs.similarity_coeffs(b, Y, mode=mode, want_S=True, path="simt")
+        gs.stream_status()
+        assert bool(torch.isfinite(ref["S"][17, :128]).all())
+        for f in (torch.isnan, torch.isposinf, torch.isneginf):
+            assert torch.equal(f(out["S"]), f(ref["S"]))
+        fin = torch.isfinite(ref["S"])
+        top = (Y[:17].norm(dim=1).max() * b.cnorm.max()) if mode == "raw" else 1.0
+        assert bool(((out["S"] - ref["S"])[fin].abs() <= 1e-4 * top).all())
