@@ -355,10 +355,15 @@ gs_status gs_project_similarity(const gs_basis* h, const float* X, long long N, 
         a.c_type = gs::MAT_F32;
         a.m = nc; a.n = r; a.k = D; a.batch = 1; a.alpha = 1.f;
         const bool wanted = S || argmax || maxval;
+        // k_scores scores a row with one warp: it has the scores where one staged chunk of shared memory holds the
+        // codebook and rows x codewords are few, a product and a row pass beyond (r = 40, argmax, k_scores against
+        // the others: 1,024 rows of D = 4096 and 128 codewords 33 / 39 us, 256: 37 / 39, 384: 46 / 40, 1,024: 70 /
+        // 42; of D = 1023, 4,096 rows and 128: 35 / 37, 256: 42 / 39; 30,000 rows and 64: 112 / 104)
+        const bool narrow = r <= gs::kMaxScoresR && M <= gs::scores_chunk(r) && nc * M <= 1 << 19;
         // narrow bases: the projection's K chunks (with the rows' squared norms for the cosine) go
         // straight to the scoring kernel, which sums them, scores and picks in the same launch (1,024
         // queries, D = 8192, r = M = 40, cosine: 83 us as norms, product, sum, product and row pass, 45 here)
-        if (r <= gs::kMaxScoresR && !gs::gemm_fp32_on_tensor(a, simt, h->device)) {
+        if (narrow && !gs::gemm_fp32_on_tensor(a, simt, h->device)) {
             const long long room = h->scratch_floats / (nc * (r + 1));
             a.ksplit = (int)std::min<long long>(gemm_ksplit(nc, r, D, h->device), room);
             a.kpart = scr;
@@ -401,7 +406,7 @@ gs_status gs_project_similarity(const gs_basis* h, const float* X, long long N, 
         cudaError_t e = gs::launch_gemm_fp32(a, simt, h->device, s);
         if (e != cudaSuccess) return from_cuda(e);
         if (!wanted) continue;
-        if (r <= gs::kMaxScoresR) {
+        if (narrow) {
             gs::ScoreArgs q{};
             q.Y = Ybuf; q.ldy = (int)ldyb; q.xnorm = xn;
             q.N = nc; q.r = r; q.R = h->R; q.ldr = h->ldr; q.M = M; q.cnorm = h->cnorm;

@@ -111,6 +111,7 @@ cudaError_t launch_ps_small(const float* X, long long N, int ldx, int D, const f
 // when given; xx: ||x||^2 in ks parts, for the cosine).  With Y, xnorm (optional) holds ||x_n||;
 // otherwise ||y_n|| stands for it (Eq. 3).
 constexpr int kMaxScoresR = 64;
+int scores_chunk(int r);  // codewords of r coordinates that a block keeps in shared memory
 struct ScoreArgs {
     const float* Y; int ldy;
     const float* part; const float* xx; int ks;

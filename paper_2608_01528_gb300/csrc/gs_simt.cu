@@ -923,6 +923,9 @@ cudaError_t launch_ps_small(const float* X, long long N, int ldx, int D, const f
     return cudaGetLastError();
 }
 
+static int scores_pitch(int r) { return 4 * (((r + 3) / 4) | 1); }
+int scores_chunk(int r) { return (kRSmemFloats - kCoefWarps * kCoefR) / scores_pitch(r); }
+
 cudaError_t launch_scores(const ScoreArgs& a, cudaStream_t s) {
     if (a.N <= 0) return cudaSuccess;
     if (a.r < 1 || a.r > kCoefR) return cudaErrorInvalidValue;
@@ -935,9 +938,8 @@ cudaError_t launch_scores(const ScoreArgs& a, cudaStream_t s) {
     p.R = a.R, p.ldr = a.ldr, p.M = a.M, p.cnorm = a.cnorm;
     p.mode = a.mode, p.scale = a.scale;
     p.S = a.S, p.lds = a.lds, p.argmax = a.argmax, p.maxval = a.maxval;
-    const int r4 = (a.r + 3) / 4;
-    p.pitch = 4 * (r4 | 1);
-    p.chunk = std::min(a.M, (kRSmemFloats - kCoefWarps * kCoefR) / p.pitch);
+    p.pitch = scores_pitch(a.r);
+    p.chunk = std::min(a.M, scores_chunk(a.r));
     const size_t smem = sizeof(float) * ((size_t)p.chunk * p.pitch + kCoefWarps * kCoefR);
     // a block stages R once, so at most about two blocks' worth of rounds per SM of a large batch
     const long long blocks = std::min<long long>((a.N + kCoefWarps - 1) / kCoefWarps, 152LL * 8);

@@ -54,6 +54,21 @@ def test_project_similarity(gs, N, D, M, r, mode):
     assert bool(((out["Y"].double() - Y).abs() <= tol * X.double().norm(dim=1)[:, None] + 1e-30).all())
 
 
+# 64 coordinates: 173 codewords fit a staged chunk, one more takes the product and the row pass; rows x codewords
+# at and past 2^19
+@pytest.mark.parametrize("N,M,r", [(300, 173, 64), (300, 174, 64), (8192, 64, 64), (8193, 64, 64)])
+@pytest.mark.parametrize("mode", ["raw", "cosine", "softmax"])
+def test_route_edges(gs, N, M, r, mode):
+    C, X = setup(N, 515, M, r, [N, M])
+    b = gs.build_basis(C)
+    scale = 4.0 / 515 if mode == "softmax" else 1.0
+    out = gs.project_similarity(b, X, mode=mode, scale=scale, path="simt", want_S=True)
+    few = gs.project_similarity(b, X, mode=mode, scale=scale, path="simt")
+    gs.stream_status()
+    check(out, X, C, mode, scale, (515 + b.r) * 2.0 ** -24 + 1e-6)
+    assert torch.equal(few["argmax"], out["argmax"]) and torch.equal(few["maxval"], out["maxval"])
+
+
 @pytest.mark.parametrize("N,M,r", [(1, 1, 1), (8, 5, 4), (9, 33, 7), (1300, 40, 40), (10000, 1024, 61), (300, 2500, 64)])
 @pytest.mark.parametrize("mode", ["raw", "cosine", "softmax"])
 def test_similarity_coeffs(gs, N, M, r, mode):
