@@ -30,11 +30,13 @@
  *    valid no-op.
  *  - All functions are callable from any host thread; a gs_basis must not be
  *    destroyed while work that uses it is in flight.  Some paths keep
- *    intermediate results in a scratch area owned by the gs_basis (the two-GEMM
- *    similarity for bases the fused kernel cannot hold, the tensor-core
- *    reconstruct, gs_similarity_coeffs), so calls on one gs_basis that may run
- *    at the same time on the GPU (different streams) must be ordered by the
- *    caller.
+ *    intermediate results in a scratch area owned by the gs_basis:
+ *    gs_project_similarity off the fused kernel (the two-GEMM path, and the fp32 path
+ *    with r > 32, whose partial products lie there whatever the outputs are),
+ *    gs_project_similarity_host, gs_similarity_coeffs with r > 64 or on the
+ *    tensor-core path, the tensor-core gs_reconstruct, and gs_reconstruct_bind.  Such
+ *    calls on one gs_basis that may run at the same time on the GPU (different
+ *    streams) must be ordered by the caller.
  */
 #ifndef GRAMSPACE_H
 #define GRAMSPACE_H
@@ -95,8 +97,11 @@ typedef struct gs_basis gs_basis;
  * Gram-Schmidt, Sec. 3.3; rank k = algebraic rank, Sec. 3.2).
  *
  * Orthonormalises the rows of C (M x D, fp32, ld = ldc) in row order by
- * Gram-Schmidt with two projection passes per row (reorthogonalisation),
- * computed in fp64 on the device in panels of rows.  Row i is accepted as a
+ * Gram-Schmidt with two projection passes per row (reorthogonalisation) on
+ * the device, in panels of rows: rank decisions, coefficients and rows in fp64;
+ * in fp32 only the second pass' products, whose coefficients are the first
+ * one's rounding (~1e-16 of the row), and a first guess at the transform inside a
+ * panel, which is then applied and corrected in fp64.  Row i is accepted as a
  * new basis direction when the norm left after both passes exceeds
  * rank_tol * ||c_i||; otherwise it is dependent and keeps only its
  * coefficients.  Produces Q (r x D) with Q Q^T = I_r, R (M x r, lower echelon,
@@ -268,8 +273,9 @@ GS_API gs_status gs_project_similarity_host(const gs_basis* h, const float* X, l
  * r = 0 (every score is then 0).
  * Tensor-core path (GS_PATH_AUTO for large N·M·r): Y and R split into bf16 hi /
  * lo, three products, fp32 accumulation (~2^-16 relative); needs Y 16-byte
- * aligned and ldy % 4 == 0.  Otherwise at fp32 accuracy, as gs_prob_vectorize.  Uses the basis'
- * scratch for cosine norms and, when S is NULL, for the scores.
+ * aligned and ldy % 4 == 0.  Otherwise at fp32 accuracy, as gs_prob_vectorize.  With
+ * r > 64, or on the tensor-core path, uses the basis' scratch for cosine norms and,
+ * when S is NULL, for the scores.
  */
 GS_API gs_status gs_similarity_coeffs(const gs_basis* h, const float* Y, long long N, int ldy, int mode,
                                       float scale, unsigned flags, float* S, int lds, int* argmax,
@@ -384,7 +390,8 @@ GS_API gs_status gs_reconstruct_bind(const gs_basis* h, const void* T, int t_dty
  * in_dtype (GS_F32 or GS_BF16) with row stride ldy elements; A is
  * B x Lq x Lk fp32, dense.  scale = 1/sqrt(D) reproduces full-dimension
  * attention.  Tensor-core path: bf16 inputs, fp32 accumulation.  fp32 inputs: at fp32
- * accuracy, as gs_prob_vectorize.
+ * accuracy, as gs_prob_vectorize.  With the softmax, a key whose logit is -inf weighs 0
+ * beside others, and a row with a logit that is NaN or +inf is NaN.
  */
 GS_API gs_status gs_attention_scores(const void* Yq, const void* Yk, int in_dtype, int B, int Lq,
                               int Lk, int r, int ldy, float scale, int apply_softmax, float* A,
