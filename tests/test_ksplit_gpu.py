@@ -77,13 +77,26 @@ def test_repeated_calls_agree(gs):
     gs.stream_status()
 
 
-def test_unaligned_score_rows(gs):
-    C, X, lab = setup(60, 4096, 5000, 4)
+@pytest.mark.parametrize("N", [5000, 12000])  # a shared K range, and none
+@pytest.mark.parametrize("mode", ["raw", "cosine", "softmax"])
+def test_unaligned_score_rows(gs, N, mode):
+    C, X, lab = setup(60, 4096, N, [N, 4])
     b = gs.build_basis(C)
-    S = torch.empty((5000, 61), device="cuda")[:, :60]
-    out = gs.project_similarity(b, X, mode="softmax", scale=8 / 4096, want_S=True, out={"S": S})
+    scale = 8 / 4096 if mode == "softmax" else 1.0
+    buf = torch.full((N, 61), -7.0, device="cuda")
+    out = gs.project_similarity(b, X, mode=mode, scale=scale, path="tensor", want_S=True, out={"S": buf[:, :60]})
     gs.stream_status()
-    assert float((out["S"].sum(1) - 1).abs().max()) <= 1e-5
+    S = X.double() @ C.double().T
+    mag = X.double().norm(dim=1)[:, None] * C.double().norm(dim=1)[None, :]
+    if mode == "raw":
+        tol = TOL * mag
+    elif mode == "cosine":
+        S, tol = S / mag, TOL
+    else:
+        S, tol = torch.softmax(scale * S, 1), 2 * TOL * scale * mag.max() + 1e-5
+    assert bool(((out["S"].double() - S).abs() <= tol).all())
+    assert torch.equal(out["argmax"].long(), lab)
+    assert bool((buf[:, 60] == -7.0).all())  # nothing between the rows
 
 
 # clusters of 8, 4 and 2, no split: more codewords than the basis has rows, so that the scores of a row

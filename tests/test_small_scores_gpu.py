@@ -83,13 +83,37 @@ def test_similarity_coeffs(gs, N, M, r, mode):
     assert torch.equal(few["argmax"], out["argmax"]) and torch.equal(few["maxval"], out["maxval"])
 
 
+# k_ps_small, k_scores on the projection's parts, the product and the row pass; k_scores on given rows
+@pytest.mark.parametrize("M,r", [(25, 20), (60, 50), (400, 50)])
+@pytest.mark.parametrize("given", [False, True])
 @pytest.mark.parametrize("mode", ["raw", "cosine", "softmax"])
-def test_not_finite(gs, mode):
-    """NaN rows give index 0; an infinite row gives what plain fp32 arithmetic gives."""
-    C, X = setup(40, 300, 20, 20, 3)
+def test_not_finite(gs, M, r, given, mode):
+    """Rows with a NaN or an infinity have NaN and infinities where the products, in the same form but in 64
+    bits, have them; a NaN never wins (entry 0 when nothing else does), and no other row notices."""
+    C, X = setup(40, 300, M, r, 3)
     b = gs.build_basis(C)
-    X[7] = float("nan")
-    out = gs.project_similarity(b, X, mode=mode, scale=0.01, path="simt", want_S=True)
+    Q, R = b.Q.double(), b.R.double()
+    if given:
+        X = (X.double() @ Q.T).float()
+    bad = [7, 9, 11]
+    X[bad, 13] = torch.tensor([float("nan"), float("inf"), -float("inf")], device="cuda")
+    if given:
+        out = gs.similarity_coeffs(b, X, mode=mode, scale=0.01, path="simt", want_S=True)
+    else:
+        out = gs.project_similarity(b, X, mode=mode, scale=0.01, path="simt", want_S=True)
     gs.stream_status()
-    assert int(out["argmax"][7]) == 0
-    assert bool(torch.isfinite(out["S"][:7]).all()) and bool(torch.isfinite(out["S"][8:]).all())
+    Y = X.double() if given else X.double() @ Q.T
+    S = 0.01 * (Y @ R.T)
+    if mode == "cosine":
+        den = X.double().norm(dim=1)[:, None] * C.double().norm(dim=1)[None, :]
+        S = torch.where(den > 0, S / den, torch.zeros_like(S))
+    best = torch.where(torch.isnan(S), torch.full_like(S, -float("inf")), S).max(1)
+    index = torch.where(best.values > -float("inf"), best.indices, torch.zeros_like(best.indices))
+    if mode == "softmax":
+        S = torch.softmax(S, 1)
+    for f in (torch.isnan, torch.isposinf, torch.isneginf):
+        assert torch.equal(f(out["S"]), f(S))
+    assert torch.equal(out["argmax"][bad].long(), index[bad])
+    good = [i for i in range(40) if i not in bad]
+    err = (320 * 2.0 ** -24 + 1e-6) * (0.01 * Y[good].norm(dim=1).max() * R.norm(dim=1).max() if mode == "raw" else 1.0)
+    assert bool(((out["S"][good].double() - S[good]).abs() <= 8 * err).all())
