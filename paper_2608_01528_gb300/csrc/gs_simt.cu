@@ -463,11 +463,25 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs& g, long long m0, int n
     }
     const bool b_in = n0 + lr < g.n;
     const long long brow = BT ? (long long)(b_in ? n0 + lr : g.n - 1) * g.ldb : 0;
+    // bf16 operands, which no 16-byte load takes here: consecutive threads on consecutive elements, k sk of rows sr +
+    // 16 t (four of a row each: 64 x 64 x 1,100 x 128 53 us, 46 so)
+    const int sr = tid / 16, sk = tid % 16;
+    const int rows = (int)(g.m - m0 < 16 * MT ? g.m - m0 : 16 * MT), cols = min(kTN, g.n - n0);
     float av[AR][4], bv[4], xx[AR] = {};
     auto load = [&](int k0) {
+        if (TA == MAT_F32) {
 #pragma unroll
-        for (int h = 0; h < AR; ++h) ld4<TA>(Ab, arow[h] + k0 + lk, a_in[h] ? kend - (k0 + lk) : 0, g.a_vec, av[h]);
-        if (BT)
+            for (int h = 0; h < AR; ++h) ld4<TA>(Ab, arow[h] + k0 + lk, a_in[h] ? kend - (k0 + lk) : 0, g.a_vec, av[h]);
+        } else {
+#pragma unroll
+            for (int t = 0; t < 4 * AR; ++t)
+                av[t / 4][t % 4] = sr + 16 * t < rows && k0 + sk < kend ? ld_elem<TA>(Ab, (m0 + sr + 16 * t) * g.lda + k0 + sk) : 0.f;
+        }
+        if (TB == MAT_BF16) {  // (n x k)
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+                bv[t] = sr + 16 * t < cols && k0 + sk < kend ? ld_elem<TB>(Bb, (long long)(n0 + sr + 16 * t) * g.ldb + k0 + sk) : 0.f;
+        } else if (BT)
             ld4<TB>(Bb, brow + k0 + lk, b_in ? kend - (k0 + lk) : 0, g.b_vec, bv);
         else
             ld4<TB>(Bb, (long long)(k0 + br) * g.ldb + n0 + bc, k0 + br < kend ? g.n - (n0 + bc) : 0, g.b_vec, bv);
@@ -477,10 +491,15 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs& g, long long m0, int n
         for (int u = 0; u < 4; ++u) {
 #pragma unroll
             for (int h = 0; h < AR; ++h) {
-                As[buf][lk + u][lr + 64 * h] = av[h][u];
-                xx[h] = fmaf(av[h][u], av[h][u], xx[h]);
+                if (TA == MAT_F32) {
+                    As[buf][lk + u][lr + 64 * h] = av[h][u];
+                    xx[h] = fmaf(av[h][u], av[h][u], xx[h]);
+                } else {
+                    As[buf][sk][sr + 16 * (4 * h + u)] = av[h][u];
+                }
             }
-            if (BT) Bs[buf][lk + u][lr] = bv[u];
+            if (TB == MAT_BF16) Bs[buf][sk][sr + 16 * u] = bv[u];
+            else if (BT) Bs[buf][lk + u][lr] = bv[u];
         }
         if (!BT) *reinterpret_cast<float4*>(&Bs[buf][br][bc]) = make_float4(bv[0], bv[1], bv[2], bv[3]);
     };

@@ -185,3 +185,30 @@ def test_not_finite_past_the_end_of_a_codeword(gs, bad):
         fin = torch.isfinite(ref["S"])
         top = (Y[:17].norm(dim=1).max() * b.cnorm.max()) if mode == "raw" else 1.0
         assert bool(((out["S"] - ref["S"])[fin].abs() <= 1e-4 * top).all())
+
+
+# the CUDA-core GEMM's tiles of 64 and of 128 rows, its last ones ragged; rows that 16-byte loads may take and not
+@pytest.mark.parametrize("B,Lq,Lk,r", [(64, 37, 70, 33), (200, 64, 129, 64), (40, 113, 500, 17), (40, 128, 500, 20),
+                                       (30, 129, 501, 48), (1, 2500, 1100, 15), (1, 1, 1, 1)])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_cuda_core_tiles(gs, B, Lq, Lk, r, dtype):
+    g = torch.Generator(device="cuda").manual_seed(B + Lq)
+    q = torch.randn((B, Lq, r), generator=g, device="cuda").to(dtype)
+    k = torch.randn((B, Lk, r), generator=g, device="cuda").to(dtype)
+    A = gs.attention_scores(q, k, 0.5, apply_softmax=False, path="simt")
+    gs.stream_status()
+    qd, kd = q.double(), k.double().transpose(1, 2)
+    assert bool(((A.double() - 0.5 * (qd @ kd)).abs() <= r * 2.0 ** -24 * (qd.abs() @ kd.abs()) + 1e-30).all())
+
+
+@pytest.mark.parametrize("M,N", [(33, 700), (64, 700), (130, 65), (260, 20000)])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_cuda_core_columns(gs, M, N, dtype):
+    """The same for a second operand that is read by columns."""
+    rng = np.random.default_rng([M, N])
+    b = gs.build_basis(bipolar(rng, M, 333))
+    T = torch.from_numpy(rng.standard_normal((N, b.r)).astype(np.float32)).cuda().to(dtype)
+    X = gs.reconstruct(b, T, path="simt")
+    gs.stream_status()
+    Td, Q = T.double(), b.Q.double()
+    assert bool(((X.double() - Td @ Q).abs() <= b.r * 2.0 ** -24 * (Td.abs() @ Q.abs())).all())
