@@ -363,9 +363,8 @@ gs_status gs_project_similarity(const gs_basis* h, const float* X, long long N, 
         // narrow bases: the projection's K chunks (with the rows' squared norms for the cosine) go
         // straight to the scoring kernel, which sums them, scores and picks in the same launch (1,024
         // queries, D = 8192, r = M = 40, cosine: 83 us as norms, product, sum, product and row pass, 45 here)
+        a.ksplit = (int)std::min<long long>(gemm_ksplit(nc, r, D, h->device), h->scratch_floats / (nc * (r + 1)));
         if (narrow && !gs::gemm_fp32_on_tensor(a, simt, h->device)) {
-            const long long room = h->scratch_floats / (nc * (r + 1));
-            a.ksplit = (int)std::min<long long>(gemm_ksplit(nc, r, D, h->device), room);
             a.kpart = scr;
             a.xx_part = mode == GS_SCORE_COSINE ? scr + (long long)a.ksplit * nc * r : nullptr;
             cudaError_t e = gs::launch_gemm_simt_parts(a, s, false);

@@ -646,10 +646,16 @@ static int x3_ksplit(const GemmArgs& g, bool simt, int device) {
     // times of both kernels, fitted to measured ones: a wave of tiles takes ~0.9 us per K-block and ~6 us
     // around it (512 x 3001 x 257: 21 us against 36 on the CUDA cores; 3000 x 1000 x 300: 32 / 56; 20,000 x
     // 777 x 131: 95 / 128; 1,300 x 13,823 x 130: 84 / 154); the CUDA-core GEMM runs at 28 to 45 TFLOP/s
-    const double simt_us = 2e-6 * g.m * g.n * g.k * g.batch / 30.0;
-    if (!takes || simt_us <= 15.0 || !tc_available(device)) return 0;
+    // where it is full, and unsplit takes at least 0.42 us a step of 16 and 0.4 more for each of an SM's 64 x 64
+    // tiles (700 x 922 x 922, two on some SMs: 84 us; 100 x 922 x 922, one: 50)
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+    double simt_us = 2e-6 * g.m * g.n * g.k * g.batch / 30.0;
+    if (g.ksplit <= 1) {
+        const double t64 = (double)((g.m + 63) / 64) * ((g.n + 63) / 64) * g.batch;
+        simt_us = std::max(simt_us, g.k / 16 * (0.42 + 0.4 * std::ceil(t64 / std::max(sms, 1))));
+    }
+    if (!takes || simt_us <= 15.0 || !tc_available(device)) return 0;
     const double tiles = (double)((g.m + kBM - 1) / kBM) * ((g.n + kBN - 1) / kBN) * g.batch;
     const int nkb = (g.k + kBK - 1) / kBK;
     // few tiles over a deep K: chunks of at least eight K-blocks to partial products in the caller's
