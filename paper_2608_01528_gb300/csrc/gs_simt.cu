@@ -997,10 +997,11 @@ cudaError_t launch_gemm_simt_parts(const GemmArgs& args, cudaStream_t s, bool su
         return cudaGetLastError();
     }
     const long long z = g.ksplit > 1 ? g.ksplit : g.batch, tn = (g.n + kTN - 1) / kTN;
-    // 128-row tiles: about two of them for every SM, and at most an eighth more rows of padding than 64-row ones (64
-    // products of 64 x 1,100 x 128 took 62 us in half-empty ones, 44 so)
+    // 128-row tiles: about two of them for every SM, and at most a quarter more rows of padding than 64-row ones (64
+    // products of 64 x 1,100 x 128 took 62 us in half-empty ones, 44 so; 40 of 129 x 1,100 x 64 43.6 / 39.4; but 300 x
+    // 9,001 x 63, a fifth more, 16.8 in 128-row tiles, 20.6 in 64-row ones)
     const long long t128 = (g.m + 127) / 128, t64 = (g.m + 63) / 64;
-    const bool tall = t128 * tn * z >= 300 && 16 * t128 <= 9 * t64;
+    const bool tall = t128 * tn * z >= 300 && 8 * t128 <= 5 * t64;
     const int tm = tall ? 128 : kTM;
     dim3 grid((unsigned)tn, (unsigned)((g.m + tm - 1) / tm), (unsigned)z);
     if (grid.y > 65535u) return cudaErrorInvalidConfiguration;
