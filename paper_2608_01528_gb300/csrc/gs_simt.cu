@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(kCoefWarps * 32) k_scores(const ScoreParams p)
 // 1024, r = 30: 45 us, now 14.5; of D = 2560: 103, now 29); four queries' products in one warp's registers left
 // few for loads in flight (19 and 57 us; at 512 queries, r = 10, it was the faster one, 5 us against 8).
 constexpr int kSmallR = 32;
-constexpr int kSmallM = 64;   // codewords kept in shared memory
+constexpr int kSmallM = 64;   // codewords kept in shared memory of their own
 constexpr int kSmallKC = 128, kSmallPitch = kSmallKC + 4;
 // ring depth: the few-query blocks have an SM each and are bound by latency alone
 constexpr int small_stages(int qb) { return qb == 4 ? 8 : 4; }
@@ -240,7 +240,8 @@ __device__ __forceinline__ float dot4(const float4& a, const float4& b) {
     return fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, a.w * b.w)));
 }
 
-template <int QB, int RB, bool VEC>
+// BIG: more than kSmallM codewords (a template parameter: the usual small codebooks' kernel keeps its registers)
+template <int QB, int RB, bool VEC, bool BIG>
 __global__ void __launch_bounds__(256) k_ps_small(const float* __restrict__ X, long long N, int ldx, int D,
                                                   const float* __restrict__ Q, int r, const float* __restrict__ R,
                                                   int ldr, int M, const float* __restrict__ cnorm, int mode,
@@ -250,7 +251,7 @@ __global__ void __launch_bounds__(256) k_ps_small(const float* __restrict__ X, l
     extern __shared__ float4 small_sm[];
     float* ring = reinterpret_cast<float*>(small_sm);  // kSmallStages x kRows rows: the queries, then Q
     __shared__ float ysm[QB][kSmallR], xsm[QB];
-    __shared__ float Rs[kSmallM][kSmallR + 1];  // codewords (up to kSmallM), odd pitch: a row per lane
+    __shared__ float Rs[BIG ? 1 : kSmallM][kSmallR + 1];  // the codewords, odd pitch: a row per lane
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long n0 = (long long)blockIdx.x * QB;
     const int nch = (D + kSmallKC - 1) / kSmallKC;
@@ -275,8 +276,7 @@ __global__ void __launch_bounds__(256) k_ps_small(const float* __restrict__ X, l
         if (c < nch) fetch(c);
         else asm volatile("cp.async.commit_group;" ::: "memory");
     }
-    const bool staged = M <= kSmallM;
-    if (staged)  // in flight under the projection
+    if (!BIG)  // in flight under the projection
         for (int e = threadIdx.x; e < M * RB; e += 256) {
             const int i = e / RB, j = e % RB;
             Rs[i][j] = j < r ? __ldg(R + (size_t)i * ldr + j) : 0.f;
@@ -336,6 +336,76 @@ __global__ void __launch_bounds__(256) k_ps_small(const float* __restrict__ X, l
         }
     }
     __syncthreads();
+    if (BIG) {
+        // the codebook goes through the ring's memory, as much of it at a time as fits (read in place, a row per lane
+        // and r loads of 32 lines a codeword: 20,000 queries of D = 256, r = 20 against 700 codewords 269 us, 772
+        // with the softmax and scores; 97 and 202 so)
+        constexpr int NW = (QB + 7) / 8;  // queries of a warp
+        constexpr int kCap = kSmallStages * kRows * kSmallPitch / (RB + 1) / 32 * 32;
+        const int passes = mode != GS_SCORE_SOFTMAX ? 1 : S ? 3 : 2;
+        float bv[NW], z[NW];
+        int bi[NW];
+#pragma unroll
+        for (int v = 0; v < NW; ++v) bv[v] = -FLT_MAX, z[v] = 0.f, bi[v] = 0x7fffffff;
+        for (int pass = 0; pass < passes; ++pass) {
+            for (int i0 = 0; i0 < M; i0 += kCap) {
+                const int nc = min(kCap, M - i0);
+                if (pass == 0 || M > kCap) {
+                    __syncthreads();  // every warp is through with the last chunk
+                    for (int e = threadIdx.x; e < nc * RB; e += 256) {
+                        const int i = e / RB, j = e % RB;
+                        ring[i * (RB + 1) + j] = j < r ? __ldg(R + (size_t)(i0 + i) * ldr + j) : 0.f;
+                    }
+                    __syncthreads();
+                }
+#pragma unroll
+                for (int v = 0; v < NW; ++v) {
+                    const int qi = warp + 8 * v;
+                    if (qi >= QB || n0 + qi >= N) continue;
+                    const long long n = n0 + qi;
+                    const float xnorm = sqrtf(xsm[qi]);
+                    float y[RB];
+#pragma unroll
+                    for (int j = 0; j < RB; ++j) y[j] = j < r ? ysm[qi][j] : 0.f;
+                    for (int c = lane; c < nc; c += 32) {
+                        const int i = i0 + c;
+                        float g = 0.f;
+#pragma unroll
+                        for (int j = 0; j < RB; ++j) g = fmaf(y[j], ring[c * (RB + 1) + j], g);
+                        g *= scale;
+                        if (mode == GS_SCORE_COSINE) {
+                            const float den = xnorm * cnorm[i];
+                            g = den > 0.f ? g / den : 0.f;
+                        }
+                        if (pass == 0) {
+                            if (g > bv[v]) {
+                                bv[v] = g;
+                                bi[v] = i;
+                            }
+                            if (S && mode != GS_SCORE_SOFTMAX) S[(size_t)n * lds + i] = g;
+                        } else if (pass == 1) {
+                            z[v] += __expf(g - bv[v]);
+                        } else {
+                            S[(size_t)n * lds + i] = __expf(g - bv[v]) * z[v];
+                        }
+                    }
+                }
+            }
+#pragma unroll
+            for (int v = 0; v < NW; ++v) {
+                if (pass == 0) warp_argmax(bv[v], bi[v]);
+                if (pass == 1) z[v] = 1.f / warp_sum(z[v]);
+            }
+        }
+#pragma unroll
+        for (int v = 0; v < NW; ++v) {
+            const int qi = warp + 8 * v;
+            if (lane != 0 || qi >= QB || n0 + qi >= N) continue;
+            if (argmax) argmax[n0 + qi] = bi[v] == 0x7fffffff ? 0 : bi[v];
+            if (maxval) maxval[n0 + qi] = mode == GS_SCORE_SOFTMAX ? z[v] : bv[v];
+        }
+        return;
+    }
     for (int qi = warp; qi < QB; qi += 8) {
         const long long n = n0 + qi;
         if (n >= N) break;
@@ -347,15 +417,8 @@ __global__ void __launch_bounds__(256) k_ps_small(const float* __restrict__ X, l
         // scores: lane handles codewords i = lane, lane + 32, ...
         auto score = [&](int i) {
             float g = 0.f;
-            if (staged) {
 #pragma unroll
-                for (int j = 0; j < RB; ++j) g = fmaf(y[j], Rs[i][j], g);
-            } else {
-                const float* Ri = R + (size_t)i * ldr;
-#pragma unroll
-                for (int j = 0; j < RB; ++j)
-                    if (j < r) g = fmaf(y[j], __ldg(Ri + j), g);
-            }
+            for (int j = 0; j < RB; ++j) g = fmaf(y[j], Rs[i][j], g);
             g *= scale;
             if (mode == GS_SCORE_COSINE) {
                 const float den = xnorm * cnorm[i];
@@ -921,12 +984,15 @@ cudaError_t launch_ps_small(const float* X, long long N, int ldx, int D, const f
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
 #define GS_SMALL_CASE(QB, RB)                                                                          \
     if (!opted[dev])                                                                                   \
-        for (auto fn : {k_ps_small<QB, RB, true>, k_ps_small<QB, RB, false>}) {                        \
+        for (auto fn : {k_ps_small<QB, RB, true, false>, k_ps_small<QB, RB, false, false>,             \
+                        k_ps_small<QB, RB, true, true>, k_ps_small<QB, RB, false, true>}) {            \
             e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);     \
             if (e != cudaSuccess) return e;                                                            \
         }                                                                                              \
-    if (qb == QB && rb == RB) kern = vec ? k_ps_small<QB, RB, true> : k_ps_small<QB, RB, false>;
-    auto kern = k_ps_small<4, 8, true>;
+    if (qb == QB && rb == RB)                                                                          \
+        kern = M <= kSmallM ? (vec ? k_ps_small<QB, RB, true, false> : k_ps_small<QB, RB, false, false>) \
+                            : (vec ? k_ps_small<QB, RB, true, true> : k_ps_small<QB, RB, false, true>);
+    auto kern = k_ps_small<4, 8, true, false>;
     GS_SMALL_CASE(4, 8)
     GS_SMALL_CASE(4, 16)
     GS_SMALL_CASE(4, 32)

@@ -69,6 +69,21 @@ def test_route_edges(gs, N, M, r, mode):
     assert torch.equal(few["argmax"], out["argmax"]) and torch.equal(few["maxval"], out["maxval"])
 
 
+# up to 32 coordinates: 65 codewords go through the ring, 768 (16 queries, 32 coordinates) to 1,408 (4, 8) fill it
+@pytest.mark.parametrize("N,M,r", [(5, 65, 8), (100, 1409, 8), (601, 65, 16), (1000, 3000, 12), (2433, 768, 32), (2450, 769, 30),
+                                   (1, 5000, 32)])
+@pytest.mark.parametrize("mode", ["raw", "cosine", "softmax"])
+def test_more_codewords_than_kept(gs, N, M, r, mode):
+    C, X = setup(N, 261, M, r, [N, M])
+    b = gs.build_basis(C)
+    scale = 4.0 / 261 if mode == "softmax" else 1.0
+    out = gs.project_similarity(b, X, mode=mode, scale=scale, path="simt", want_S=True)
+    few = gs.project_similarity(b, X, mode=mode, scale=scale, path="simt")
+    gs.stream_status()
+    check(out, X, C, mode, scale, (261 + b.r) * 2.0 ** -24 + 1e-6)
+    assert torch.equal(few["argmax"], out["argmax"]) and torch.equal(few["maxval"], out["maxval"])
+
+
 @pytest.mark.parametrize("N,M,r", [(1, 1, 1), (8, 5, 4), (9, 33, 7), (1300, 40, 40), (10000, 1024, 61), (300, 2500, 64)])
 @pytest.mark.parametrize("mode", ["raw", "cosine", "softmax"])
 def test_similarity_coeffs(gs, N, M, r, mode):
